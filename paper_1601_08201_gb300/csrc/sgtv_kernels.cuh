@@ -2106,30 +2106,155 @@ __device__ __forceinline__ double block_reduce(double v, double *sh)
     return v;
 }
 
-// Deviance partials: ybar accumulated in FP64 from the stored A values and f.
+// One measurement's deviance term, yb - y + y log(y / yb) with 0 log 0 = 0.
+__device__ __forceinline__ double dev_term(double yb, double yi)
+{
+    double t = yb - yi;
+    if (yi > 0.0) t += yi * log(yi / yb);
+    return t;
+}
+
+// A value of A as an FP64 factor scaled by 2^-kF64Shift, and that factor's
+// partner, a dense operand scaled by 2^+kF64Shift: their product is the
+// unscaled one, rounded alike. The bits of a nonnegative FP32 (or BF16) value
+// shifted into an FP64 pattern read as that value times 2^(127 - 1023)
+// (subnormals included), so the conversion is two integer instructions. The
+// device's FP64 unit, which a real conversion also occupies, does about 2
+// lanes per clock and SM (0.5 T/s measured for the conversion as for the
+// multiply-add), so the deviance below is bound by it.
+constexpr double kF64Up = 0x1p896;
+__device__ __forceinline__ double f64_scaled(float v)
+{
+    const uint32_t u = __float_as_uint(v);
+    return __hiloint2double(int(u >> 3), int(u << 29));
+}
+// BF16 rounding can reach infinity: it stays one.
+__device__ __forceinline__ double f64_scaled_bf16(float v)
+{
+    const uint32_t u = __float_as_uint(v);
+    return __hiloint2double((u >> 23) == 0xFFu ? int(0x7FF00000u | (u & 0x7FFFFFu) >> 3) : int(u >> 3), 0);
+}
+template <typename V> __device__ __forceinline__ double val_scaled(float v) { return f64_scaled(v); }
+template <> __device__ __forceinline__ double val_scaled<__nv_bfloat16>(float v) { return f64_scaled_bf16(v); }
+template <typename V> __device__ __forceinline__ double val_scaled(double v) { return v; }
+template <typename T> __device__ __forceinline__ double dense_scaled(T x) { return double(x) * kF64Up; }
+template <> __device__ __forceinline__ double dense_scaled<double>(double x) { return x; }
+
+// Deviance partials over the measurements [i0, i1), from the plain CSR form
+// (matrices without tiles, and tiles whose staging would fill an SM): ybar
+// accumulated in FP64 from the stored A values and f. A warp takes 8 rows in
+// turn, lane k keeps row k's ybar, and the 8 terms (a division and a
+// logarithm in FP64, which cost a warp the same for one lane as for 32) are
+// formed side by side.
 template <typename T, typename V>
 __global__ void __launch_bounds__(256)
-k_dev_partials(int64_t I, const int64_t *__restrict__ rowptr, const int32_t *__restrict__ col,
+k_dev_partials(int64_t i0, int64_t i1, const int64_t *__restrict__ rowptr, const int32_t *__restrict__ col,
                const V *__restrict__ val, const T *__restrict__ f, const T *__restrict__ r,
                int r_scalar, const T *__restrict__ y, double *__restrict__ part)
 {
     __shared__ double sh[32];
+    constexpr int R = 8;
     const int lane = threadIdx.x & 31;
     const int64_t nwarps = (int64_t(gridDim.x) * blockDim.x) >> 5;
     double mine = 0.0;
-    for (int64_t i = (int64_t(blockIdx.x) * blockDim.x + threadIdx.x) >> 5; i < I; i += nwarps) {
-        double acc = 0.0;
-        const int64_t start = rowptr[i], end = rowptr[i + 1];
-        for (int64_t p = start + lane; p < end; p += 32)
-            acc = fma(to_f64(val[p]), double(f[col[p]]), acc);
-        acc = warp_sum_d(acc);
-        if (lane == 0) {
-            const double yb = acc + double(r_scalar ? r[0] : r[i]);
-            const double yi = double(y[i]);
-            double t = yb - yi;
-            if (yi > 0.0) t += yi * log(yi / yb);
-            mine += t;
+    for (int64_t k0 = i0 + R * ((int64_t(blockIdx.x) * blockDim.x + threadIdx.x) >> 5); k0 < i1; k0 += R * nwarps) {
+        const int n = int(i1 - k0 < R ? i1 - k0 : R);
+        double yb = 0.0;
+        for (int k = 0; k < n; k++) {
+            double acc = 0.0;
+            const int64_t start = rowptr[k0 + k], end = rowptr[k0 + k + 1];
+            for (int64_t p = start + lane; p < end; p += 32)
+                acc = fma(to_f64(val[p]), double(f[col[p]]), acc);
+            acc = warp_sum_d(acc);
+            if (lane == k) yb = acc;
         }
+        if (lane < n) mine += dev_term(yb + double(r_scalar ? r[0] : r[k0 + lane]), double(y[k0 + lane]));
+    }
+    double tot = block_reduce<false>(mine, sh);
+    if (threadIdx.x == 0) part[blockIdx.x] = tot;
+}
+
+// The same from the tiled form (16-bit local indices): a block takes tiles
+// blockIdx.x, + gridDim.x, ... that meet [i0, i1), stages the tile's f in
+// shared memory as scaled FP64, and each warp forms 8 rows' products with one
+// FP64 multiply-add per nonzero and no other FP64 work in the loop. The lanes'
+// sums are folded by all 256 threads (a warp-wide tree would take 5 FP64
+// additions per row and lane, as much again as 5/8 of the products), and the
+// 64 terms are formed by 64 threads side by side. The lanes take consecutive
+// elements because an FP64 instruction costs a warp the same for any number
+// of active lanes (4-wide chunks, whose last chunk is mostly empty, took a
+// third more). Bound: the FP64 unit (2^28 nonzeros at 0.5 T/s: 0.53 ms).
+// Measured on that problem: 0.85 ms, against 5.11 ms for the plain form with
+// one row and one lane's term at a time.
+template <typename T, typename V>
+__global__ void __launch_bounds__(256, 4)
+k_dev_partials_tli(int64_t i0, int64_t i1, int64_t ntiles, const int64_t *__restrict__ rowptr, TliTiles tl,
+                   const V *__restrict__ val, const T *__restrict__ f, const T *__restrict__ r, int r_scalar,
+                   const T *__restrict__ y, double *__restrict__ part)
+{
+    extern __shared__ __align__(128) unsigned char smem_raw[];
+    __shared__ double rows[kTliTile][33];
+    __shared__ double sh[32];
+    double *xs = reinterpret_cast<double *>(smem_raw);
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    constexpr int R = kTliTile / 8;
+    double mine = 0.0;
+    for (int64_t t = i0 / kTliTile + blockIdx.x; t < ntiles && t * kTliTile < i1; t += gridDim.x) {
+        const int64_t t0 = t * kTliTile, t1 = t0 + kTliTile < i1 ? t0 + kTliTile : i1;
+        if (threadIdx.x == 0) prefetch_segments_l2(rowptr, t0, t1, tl.lidx, val);
+        const int wl = tl.wlen[t];
+        const int64_t u0 = tl.uoff[t];
+        const int nstage = wl > 0 ? wl : int(tl.uoff[t + 1] - u0);
+        const int64_t wb = tl.wbase[t];
+        for (int k = threadIdx.x; k < nstage; k += blockDim.x)
+            xs[k] = dense_scaled<T>(f[wl > 0 ? wb + k : int64_t(tl.uidx[u0 + k])]);
+        __syncthreads();
+        const int64_t w0 = t0 + warp * R;
+        const int n = w0 < t1 ? int(t1 - w0 < R ? t1 - w0 : R) : 0;
+        const int64_t bound = lane <= n && n > 0 ? rowptr[w0 + lane] : 0;
+#pragma unroll 1
+        for (int k = 0; k < n; k++) {
+            const int64_t s = __shfl_sync(0xffffffffu, bound, k), e = __shfl_sync(0xffffffffu, bound, k + 1);
+            double a0 = 0.0, a1 = 0.0;
+            const int n_el = int(e - s);  // a row holds at most J < 2^31 nonzeros
+            const uint16_t *__restrict__ li = tl.lidx + s;
+            const V *__restrict__ va = val + s;
+            for (int p = 0; p < n_el; p += 256) {
+                int32_t c[8];
+                T v[8];
+#pragma unroll
+                for (int u = 0; u < 8; u++) {
+                    c[u] = 0;
+                    v[u] = T(0);
+                    if (p + 32 * u + lane < n_el) {
+                        c[u] = ld_idx(li + p + 32 * u + lane);
+                        v[u] = T(ld_val(va + p + 32 * u + lane));
+                    }
+                }
+#pragma unroll
+                for (int u = 0; u < 8; u++)
+                    if (p + 32 * u < n_el) {  // warp-uniform: no FP64 instruction past the row's end
+                        double &a = (u & 1) ? a1 : a0;
+                        if (p + 32 * u + lane < n_el) a = fma(val_scaled<V>(v[u]), xs[c[u]], a);
+                    }
+            }
+            rows[warp * R + k][lane] = a0 + a1;
+        }
+        __syncthreads();
+        // 4 threads per row: 8 lanes' sums each, then the quad's total in every thread of it
+        const int rr = threadIdx.x >> 2, qd = threadIdx.x & 3;
+        double yb = 0.0;
+#pragma unroll
+        for (int m = 0; m < 8; m++) yb += rows[rr][qd + 4 * m];
+        yb += __shfl_xor_sync(0xffffffffu, yb, 1);
+        yb += __shfl_xor_sync(0xffffffffu, yb, 2);
+        __syncthreads();
+        if (qd == 0) rows[rr][0] = yb;
+        __syncthreads();
+        const int64_t i = t0 + threadIdx.x;
+        if (threadIdx.x < kTliTile && i >= i0 && i < t1)
+            mine += dev_term(rows[threadIdx.x][0] + double(r_scalar ? r[0] : r[i]), double(y[i]));
+        __syncthreads();  // rows and xs are rewritten by the next tile
     }
     double tot = block_reduce<false>(mine, sh);
     if (threadIdx.x == 0) part[blockIdx.x] = tot;

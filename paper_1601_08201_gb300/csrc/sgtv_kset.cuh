@@ -402,13 +402,25 @@ struct Impl {
         k_sum_partials<T><<<d.red_blocks, kThreads, 0, st>>>(n, static_cast<const T *>(a), d.part);
         finalize(d.part, d.red_blocks, 1, 0u, d.red + slot, st);
     }
+    // Tiled wherever the largest tile's f fits in 24 KB as FP64 (two blocks' worth of staging next
+    // to the row sums keeps at least 4 blocks on an SM): list tiles and short windows. Wide windows
+    // (small problems whose tiles span most of the image) read f from L2 in the plain form.
     static void deviance(const Dev &d, const void *f, int64_t i0, int64_t i1, int slot, cudaStream_t st)
     {
-        k_dev_partials<T, V><<<d.red_blocks, kThreads, 0, st>>>(
-            i1 - i0, d.rowptr + i0, d.col, static_cast<const V *>(d.rval), static_cast<const T *>(f),
-            static_cast<const T *>(d.r) + (d.r_scalar ? 0 : i0), d.r_scalar, static_cast<const T *>(d.y) + i0,
-            d.part);
-        finalize(d.part, d.red_blocks, 1, 0u, d.red + slot, st);
+        const T *ff = static_cast<const T *>(f), *r = static_cast<const T *>(d.r), *y = static_cast<const T *>(d.y);
+        const V *val = static_cast<const V *>(d.rval);
+        int blocks = d.red_blocks;
+        if (d.tr.fmt != 0 && d.tr.max_stage * int(sizeof(double)) <= 24 * 1024) {
+            // one partial field is free for up to 4 red_blocks blocks (Dev::part)
+            const int64_t tiles = (i1 + kTliTile - 1) / kTliTile - i0 / kTliTile;
+            blocks = int(tiles < 4 * int64_t(d.red_blocks) ? (tiles > 0 ? tiles : 1) : 4 * int64_t(d.red_blocks));
+            k_dev_partials_tli<T, V><<<blocks, kThreads, d.tr.max_stage * int(sizeof(double)), st>>>(
+                i0, i1, d.tr.ntiles, d.rowptr, tiles_of(d.tr), val, ff, r, d.r_scalar, y, d.part);
+        } else {
+            k_dev_partials<T, V><<<blocks, kThreads, 0, st>>>(i0, i1, d.rowptr, d.col, val, ff, r, d.r_scalar, y,
+                                                              d.part);
+        }
+        finalize(d.part, blocks, 1, 0u, d.red + slot, st);
     }
     static void tv(const Dev &d, const Geom &g, const void *f, const void *dsplit, int64_t s0, int64_t s1, int slot,
                    cudaStream_t st)

@@ -1,0 +1,62 @@
+"""The deviance reduction's tiled and plain forms against the FP64 oracle at
+the GPU's own iterate, at the edges of its tiles (64 rows), its row chunks (256
+nonzeros) and its ranges (scans of a batch that end inside a tile).
+
+Tolerance: each side forms every ybar and term in FP64 with relative errors of
+a few 1e-16 times the row length's square root, and sums at most some thousand
+nonnegative terms: 1e-12 relative is two orders above both."""
+import numpy as np
+import pytest
+
+import oracle as O
+from paper_1601_08201_gb300 import sgtv, synth
+
+pytestmark = pytest.mark.gpu
+
+torch = pytest.importorskip("torch")
+if not torch.cuda.is_available():  # pragma: no cover
+    pytest.skip("needs a CUDA GPU", allow_module_level=True)
+
+
+def scan(I, nnz_col, shape=(8, 6, 16), seed=0):
+    P = synth.make_problem(*shape, I, nnz_col, n_regions=2, mean_counts=3.0, seed=seed)
+    P.y[::7] = 0.0  # terms without a logarithm
+    return P
+
+
+def oracle_of(P, precision):
+    if precision == "bf16":
+        return O.from_problem(P, csr_val=synth.round_to_bf16(P.csr_val), csc_val=synth.round_to_bf16(P.csc_val))
+    return O.from_problem(P)
+
+
+# rows of about nnz_col * 768 / I nonzeros: 256 and more, short ones, none at all in part of the rows;
+# tiles of 64 rows and one row more or less; (20, 1, 200): windows too wide for the FP64 staging
+@pytest.mark.parametrize("precision", ["fp32", "bf16", "fp64"])
+@pytest.mark.parametrize("I,nnz_col,shape", [(63, 24, (8, 6, 16)), (64, 22, (8, 6, 16)), (65, 20, (8, 6, 16)),
+                                             (129, 43, (8, 6, 16)), (700, 3, (8, 6, 16)), (2000, 1, (8, 6, 16)),
+                                             (200, 70, (20, 1, 200))])
+def test_objective_at_tile_and_row_edges(precision, I, nnz_col, shape):
+    P = scan(I, nnz_col, shape)
+    op = oracle_of(P, precision)
+    with sgtv.Handle(P, precision=precision, flags=sgtv.FLAG_NO_AUTOTUNE) as h:
+        h.iterate(2)
+        f = h.get_state_f64()[0]
+        phi, dev, tv = h.objective()
+    ophi, odev, otv = O.objective(op, f)
+    assert dev == pytest.approx(odev, rel=1e-12)
+    assert phi == pytest.approx(ophi, rel=1e-12)
+
+
+def test_objective_of_scans_that_end_inside_a_tile():
+    scans = [scan(I, nc, seed=k) for k, (I, nc) in enumerate([(30, 9), (100, 20), (64, 16), (7, 2), (190, 40)])]
+    with sgtv.Handle(scans, flags=sgtv.FLAG_NO_AUTOTUNE) as h:
+        h.iterate(2)
+        f = h.get_state_f64()[0]
+        off = h.batch_info()["vox_off"]
+        each = [h.objective_scan(k) for k in range(len(scans))]
+        total = h.objective()
+    for k, P in enumerate(scans):
+        ref = O.objective(O.from_problem(P), np.ascontiguousarray(f[off[k]:off[k + 1]]))
+        assert each[k] == pytest.approx(ref, rel=1e-12), k
+    assert total[1] == pytest.approx(sum(e[1] for e in each), rel=1e-12)
