@@ -325,7 +325,8 @@ def algorithmic_bytes(P, precision, variants=None, tli=None, n_dirs=4, survey_ba
     window copies are L2 re-reads of f / ratio and are not counted. The
     single-pass row-stream variants ("sp_") stream the same 2-byte indices and
     values with each row padded to a multiple of 4 elements, plus their own
-    row pointers. Survey basis (survey_basis=True): every SpMV streams a plain
+    row pointers. The stacked forms ("stack") stream the values and one record
+    per lane and pair of rows. Survey basis (survey_basis=True): every SpMV streams a plain
     int32 index and a value per nonzero (4 + V bytes), the accounting of the
     planning survey's roofline table."""
     T = 8 if precision == "fp64" else 4
@@ -346,6 +347,8 @@ def algorithmic_bytes(P, precision, variants=None, tli=None, n_dirs=4, survey_ba
             rl = np.diff(P.csr_rowptr)
             nsp = int(((rl + 3) // 4 * 4).sum())
             return nsp * (2 + V) + meta + 8 * (I + 1)
+        if name.startswith("stack"):  # values, and at least a 32-bit record per lane and pair of rows
+            return nnz * V + 64 * I
         return nnz * (4 + V)
 
     # A by rows, row pointers, f gathered once, y, r, ratio written
@@ -353,6 +356,10 @@ def algorithmic_bytes(P, precision, variants=None, tli=None, n_dirs=4, survey_ba
     # A by columns, column pointers, ratio gathered once, f (read), s, f_new (write), d and c
     out["k_back_update"] = (stream("k_back_update", "csc", J) + (J + 1) * 8 + I * T + 3 * J * T
                             + 2 * n_dirs * J * T)
+    if variants.get("k_back_update", "").startswith("stack") and not survey_basis:
+        # the stacked pair reads A in its forward pass: at least one partial sum per hyper-voxel and its
+        # place, s, f (read), f_new (write), u = d - c
+        out["k_back_update"] = J * T + (J + 1) * 4 + 3 * J * T + n_dirs * J * T
     single = "k_scatter" in variants
     # f_new, c read; d, c written (and, in the single-pass form, u = d - c
     # for the f-update)
@@ -411,7 +418,7 @@ def recorded_traffic(kernel, workload, precision, variant=None):
 
 # ------------------------------------------------------------------------------------------
 
-def batch_bytes(scans, precision, form, tli):
+def batch_bytes(scans, precision, form, tli, tuning=None):
     """Algorithmic bytes of one iteration over all scans of a batch (format
     basis, as algorithmic_bytes for one problem; the tiled forms' unique lists
     counted from the handle)."""
@@ -423,11 +430,12 @@ def batch_bytes(scans, precision, form, tli):
     nt_r, nt_c = (I + 63) // 64, (J + 63) // 64
     meta_r = 16 * nt_r + 8 + 4 * tli["csr"]["list_entries"]
     meta_c = 16 * nt_c + 8 + 4 * tli["csc"]["list_entries"]
-    return sum(batch_bytes_by_kernel(scans, precision, form, tli).values())
+    return sum(batch_bytes_by_kernel(scans, precision, form, tli, tuning).values())
 
 
-def batch_bytes_by_kernel(scans, precision, form, tli):
-    """batch_bytes split by kernel."""
+def batch_bytes_by_kernel(scans, precision, form, tli, tuning=None):
+    """batch_bytes split by kernel; `tuning`: the chosen variants by kernel (the stacked forms stream other bytes)."""
+    stacked = any(v.startswith("stack") for v in (tuning or {}).values())
     T = 8 if precision == "fp64" else 4
     V = {"fp32": 4, "bf16": 2, "fp64": 8}[precision]
     I = sum(P.I for P in scans)
@@ -439,8 +447,12 @@ def batch_bytes_by_kernel(scans, precision, form, tli):
     if form == "single_pass":
         nsp = sum(int(((np.diff(P.csr_rowptr) + 3) // 4 * 4).sum()) for P in scans)
         # f-update: e, s, f, u (4 directions), f_new, e cleared; shrink: f, c read, d, c, u written
-        return {"k_scatter": nsp * (2 + V) + meta_r + 16 * (I + 1) + T * (J + 2 * I + J),
+        rows = nnz * V + 64 * I if stacked else nsp * (2 + V) + meta_r + 16 * (I + 1)
+        return {"k_scatter": rows + T * (J + 2 * I + J),
                 "k_fupdate": T * J * 9, "k_shrink": T * J * 17}
+    if stacked:
+        return {"k_forward": nnz * V + 64 * I + T * (J + 3 * I), "k_back_update": 4 * (J + 1) + 8 * T * J,
+                "k_shrink": 17 * T * J}
     return {"k_forward": nnz * (2 + V) + meta_r + 8 * (I + 1) + T * (J + 3 * I),
             "k_back_update": nnz * (2 + V) + meta_c + 8 * (J + 1) + T * I + 3 * T * J + 8 * T * J,
             "k_shrink": 13 * T * J}
@@ -468,8 +480,11 @@ def batched_form(sgtv, synth, args, stream, torch, form, K, W, sample_clocks=Fal
             h.profile(False)
             h.sync()
             tli = h.tli_info()
+            names = h.variant_names()
+            tuning = ({"k_scatter": names["k_scatter"][h.get_variant(sgtv.K_SCATTER)]} if form == "single_pass" else
+                      {"k_forward": names["k_forward"][h.get_variants()[0]]})
             h.close()
-            return {"prof": prof, "tli": tli}
+            return {"prof": prof, "tli": tli, "tuning": tuning}
         sampler = ClockSampler(gpu_uuid(torch)) if clocks else None
         if sampler:
             sampler.start()
@@ -502,9 +517,9 @@ def batched_form(sgtv, synth, args, stream, torch, form, K, W, sample_clocks=Fal
         ref = b["f"][off[k]:off[k + 1]]
         max_rel = max(max_rel, float(np.linalg.norm(o["f"] - ref) / max(np.linalg.norm(o["f"]), 1e-300)))
     peak, peak_kind = measured_peaks()
-    by = batch_bytes(scans, args.precision, form, b["tli"])
+    by = batch_bytes(scans, args.precision, form, b["tli"], b["tuning"])
     att = run(scans, form_flags(sgtv, form) | sgtv.FLAG_SERIAL, attribute=True)
-    kb = batch_bytes_by_kernel(scans, args.precision, form, att["tli"])
+    kb = batch_bytes_by_kernel(scans, args.precision, form, att["tli"], att["tuning"])
     per_kernel = {k: {"avg_us": 1e3 * v[0] / v[1], "launches": v[1], "algorithmic_bytes": kb.get(k),
                       "frac_of_measured_hbm": (kb[k] / (v[0] / v[1] / 1e3) / 1e9 / peak) if k in kb else None}
                   for k, v in att["prof"].items()}

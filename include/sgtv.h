@@ -237,17 +237,19 @@ int sgtv_set_state_f64(sgtv_t h, const double *f, const double *d, const double 
  * 4-wide forms ("v4" in the name) split a segment among lanes differently and
  * round differently (equally deterministic), so with the autotuner on, the
  * chosen pair decides the last bits; pin the variants (SGTV_FLAG_NO_AUTOTUNE +
- * sgtv_set_variants) for bit-reproducible runs. sgtv_autotune times every variant
- * `reps` times on the handle's own problem (writing only scratch buffers, the
- * ADMM state is untouched) and keeps the fastest; sgtv_setup runs it with
+ * sgtv_set_variants) for bit-reproducible runs. The stacked pair ("stack_v4"
+ * in both products: A read once, by rows, e from partial sums added in a fixed
+ * order) is chosen for both or for neither. sgtv_autotune times every variant
+ * up to `reps` times on the handle's own problem (writing only scratch buffers,
+ * the ADMM state is untouched) and keeps the fastest; sgtv_setup runs it with
  * reps = 10 unless SGTV_FLAG_NO_AUTOTUNE is set. In persistent mode it also
  * times the fused kernel's forms (the four tile-form pairs, with and without a
  * register cap) and selects the tiled variants ("tli_u8" / "tli_v4x2") of the
  * fastest; sgtv_set_variants then picks the pair and keeps the register cap.
  * With SGTV_FLAG_SINGLE_PASS it also times the single-pass scatter's forms
  * (one accumulator per block with shared-memory atomic adds, or one per warp
- * summed in a fixed order; prefetch depth; register cap) that fit in shared
- * memory. kernel is SGTV_K_FORWARD, SGTV_K_BACK_UPDATE or SGTV_K_SCATTER (the
+ * summed in a fixed order; prefetch depth; register cap; "stack": sums in
+ * registers) that fit in shared memory. kernel is SGTV_K_FORWARD, SGTV_K_BACK_UPDATE or SGTV_K_SCATTER (the
  * latter in sgtv_variant_count / _name and sgtv_get_variant / sgtv_set_variant
  * only). The set functions return SGTV_ERR_ARG (not sticky) for an index out
  * of range or a form that does not fit; sgtv_variant_name returns "" for one. */

@@ -65,6 +65,7 @@ struct sgtv_ctx {
     bool use_graph = false;     // iterations replayed from captured CUDA graphs
     bool single_pass = false;   // A streamed once per surrogate step (scatter + f-update)
     void *e_acc = nullptr;      // its accumulator of e (all zero between iterations)
+    void *u_buf = nullptr;      // u = d - c of a two-pass handle's stacked form (in Dev::u while that form is chosen)
     int v_scatter = 0;          // its scatter variant (KernelSet::scatter)
     int64_t max_warp_span = 0;  // most nonzeros in kTliTile / 8 consecutive rows
     int64_t max_sp_span = 0;    // the same in the single-pass row stream (padded rows)
@@ -190,9 +191,10 @@ int check_live(sgtv_t h)
 
 // Whether an SpMV variant can run on this handle (its tiled form was built
 // and, for the TMA pipelines, NS stages fit in shared memory).
-bool variant_ok(const TliMat &m, int need)
+bool variant_ok(const Dev &d, const TliMat &m, int need)
 {
     if (need == 0) return true;
+    if (need == 2) return d.st.built && d.st.part;
     if (m.fmt == 0) return false;
     if (need == 1) return true;
     return m.tma_stage_bytes > 0 && int64_t(need) * m.tma_stage_bytes <= m.smem_optin - 1024;
@@ -270,8 +272,9 @@ int validate_ptr(sgtv_t h, const int64_t *ptr, int64_t n, int64_t nnz, const cha
 bool scatter_fits(sgtv_t h, int v)
 {
     const TliMat &m = h->d.tr;
+    if (h->ks->scatter_sp[v] == 2) return h->d.st.built;
     if (m.fmt == 0 || h->max_warp_span >= (int64_t(1) << 31)) return false;
-    const bool sp = h->ks->scatter_sp[v] != 0;
+    const bool sp = h->ks->scatter_sp[v] == 1;
     if (sp && (!h->d.sp.built || h->max_sp_span >= (int64_t(1) << 31))) return false;
     // the row-stream forms keep one more slot (the padding's dummy entry)
     const int64_t cap = sp ? ((int64_t(m.max_stage) + 2) & ~int64_t(1)) : ((int64_t(m.max_stage) + 1) & ~int64_t(1));
@@ -523,6 +526,204 @@ int build_tli(sgtv_t h, const int64_t *ptr, const int64_t *host_ptr, const int32
         m.tma_stage_bytes = int(stage);
     }
     return SGTV_OK;
+}
+
+// Build the stacked row form (sgtv_stack.cu) where it applies: FP32 vectors,
+// tiles of at most 32 * kStkMaxWords columns, a schedule that fits the ring,
+// and a size no larger than the tiled form's by more than a quarter (thin
+// tiles, whose columns most rows miss, pay a bit per column and row) unless it
+// stays in the L2 cache anyway (64 MB). Where
+// it does not apply, or its memory is refused, the handle runs without it:
+// d.st.built stays 0. `parts`: with the two-pass form's partial sums.
+int build_stack(sgtv_t h, bool parts)
+{
+    Dev &d = h->d;
+    StackMat &m = d.st;
+    m = StackMat{};
+    if (h->ks->elem_size != int(sizeof(float))) return SGTV_OK;
+    cudaStream_t st = h->stream;
+    const int64_t I = d.I, J = d.J, nnz = d.nnz;
+    const int vb = h->ks->val_size;
+    std::vector<void *> mine, tmp;
+    cudaError_t ae;
+    auto get = [&](size_t bytes, std::vector<void *> &list) {
+        void *p = dev_alloc(h, bytes, &ae);
+        if (p) list.push_back(p);
+        else cudaGetLastError();  // an optional form: out of memory is no error of the handle
+        return p;
+    };
+    auto drop = [&](std::vector<void *> &list) {
+        for (void *p : list) dev_free(h, p);
+        list.clear();
+    };
+    auto without = [&]() {
+        drop(tmp);
+        drop(mine);
+        m = StackMat{};
+        return SGTV_OK;
+    };
+    auto broken = [&](cudaError_t e) {
+        drop(tmp);
+        drop(mine);
+        m = StackMat{};
+        return cuda_fail(h, e, "stacked row form");
+    };
+    int *cnt = reinterpret_cast<int *>(d.red);  // scratch until the first reduction
+    int most = 0;
+    auto count = [&](int rows) {
+        cudaError_t e = cudaMemsetAsync(cnt, 0, sizeof(int) * 4, st);
+        if (e == cudaSuccess) e = stk_count(I, J, rows, d.rowptr, d.col, cnt, st);
+        if (e == cudaSuccess) e = cudaMemcpyAsync(&most, cnt, sizeof(int), cudaMemcpyDeviceToHost, st);
+        if (e == cudaSuccess) e = cudaStreamSynchronize(st);
+        return e;
+    };
+    static const int sizes[] = {4, 6, 8, 10, 12, 14, 16, 18, 20, 22, 24};
+    auto words_of = [&](int cols) {
+        for (int w : sizes)
+            if (32 * w >= cols) return w;
+        return kStkMaxWords;
+    };
+    // Rows per tile. A tile costs its rows and about 9 rows' worth of reading
+    // its columns' f and adding its sums; the last wave of warps is half
+    // empty. Measured, microseconds for 64 / 32 / 16 rows: 2^28 nonzeros 252 /
+    // 273 / 369, 2^26 84 / 79 / 105, 2^25 47 / 49 / 57; a 41 x 9 x 54 scan,
+    // whose tiles fill no wave, takes 8 (whole iterations: 16.4 for 32, 12.0
+    // for 16, 10.4 for 8, 10.8 for 4).
+    cudaError_t ce = count(kStkMaxRows);
+    if (ce != cudaSuccess) return broken(ce);
+    const double slots = double(stk_min_blocks(words_of(most))) * d.sm_count;
+    int tr = kStkMaxRows;
+    double least = 0.0;
+    for (int rows = kStkMaxRows; rows >= 8; rows >>= 1) {
+        const double waves = double((I + rows - 1) / rows) / slots;
+        const double cost = (waves <= 1.0 ? 1.0 : waves + 0.5) * (rows + 9);
+        if (rows == kStkMaxRows || cost < least) {
+            least = cost;
+            tr = rows;
+        }
+    }
+    for (; tr < kStkMaxRows || most > 32 * kStkMaxWords; tr >>= 1) {
+        if (tr < 8) return without();
+        if ((ce = count(tr)) != cudaSuccess) return broken(ce);
+        if (most <= 32 * kStkMaxWords) break;
+    }
+    m.words = words_of(most);
+    m.tr = tr;
+    m.ntiles = (I + tr - 1) / tr;
+    const int64_t places = m.ntiles * 32 * m.words;
+    const int64_t pairs = (I + 1) / 2, rec_bytes = pairs * 32 * stk_rec_bytes(m.words);
+    const int64_t tiled = (nnz * (vb + 2) + 16 * (I / kTliTile + 1)) * 5 / 4, small = int64_t(64) << 20;
+    const int64_t most_bytes = tiled > small ? tiled : small;
+    if (places >= (int64_t(1) << 31) || rec_bytes + nnz * vb + places * 4 > most_bytes) return without();
+    // two allocations: what stays, and what the set-up alone needs
+    auto r256 = [](int64_t v) { return (v + 255) & ~int64_t(255); };
+    const int64_t nd = h->g.n_dirs;
+    const int64_t keep[] = {r256(4 * places), r256(rec_bytes), r256(4 * pairs), r256(8 * (m.ntiles + 1)),
+                            parts ? r256(4 * (J + 1)) : 0, parts ? r256(4 * places) : 0, parts ? r256(4 * J * nd) : 0};
+    const int64_t work[] = {r256(places), r256(2 * nnz), r256(64 * pairs), r256(4 * m.ntiles), parts ? r256(4 * J) : 0};
+    int64_t n_keep = 0, n_work = 0;
+    for (int64_t v : keep) n_keep += v;
+    for (int64_t v : work) n_work += v;
+    char *pk = static_cast<char *>(get(size_t(n_keep), mine)), *pw = static_cast<char *>(get(size_t(n_work), tmp));
+    if (!pk || !pw) return without();
+    auto next = [](char *&p, int64_t bytes) {
+        char *q = p;
+        p += bytes;
+        return static_cast<void *>(q);
+    };
+    m.uidx = static_cast<int32_t *>(next(pk, keep[0]));
+    m.rec = next(pk, keep[1]);
+    m.ctl = static_cast<uint32_t *>(next(pk, keep[2]));
+    m.lvl = static_cast<int64_t *>(next(pk, keep[3]));
+    uint8_t *lanes = static_cast<uint8_t *>(next(pw, work[0]));
+    uint16_t *rank = static_cast<uint16_t *>(next(pw, work[1]));
+    uint16_t *start = static_cast<uint16_t *>(next(pw, work[2]));
+    int32_t *height = static_cast<int32_t *>(next(pw, work[3]));
+    int stats[1] = {0};
+    std::vector<int32_t> hh(m.ntiles);
+    cudaError_t e = cudaMemsetAsync(cnt, 0, sizeof(int) * 4, st);
+    if (e == cudaSuccess) e = stk_build(I, J, m, d.rowptr, d.col, lanes, rank, start, height, cnt, st);
+    if (e == cudaSuccess) e = cudaMemcpyAsync(stats, cnt, sizeof(stats), cudaMemcpyDeviceToHost, st);
+    if (e == cudaSuccess)
+        e = cudaMemcpyAsync(hh.data(), height, sizeof(int32_t) * m.ntiles, cudaMemcpyDeviceToHost, st);
+    if (e == cudaSuccess) e = cudaStreamSynchronize(st);
+    if (e != cudaSuccess) return broken(e);
+    // one level more than needed, so that every place in the ring stands for one level
+    m.ring = stats[0] + 1 > 2 * m.words + kStkMirror ? stats[0] + 1 : 2 * m.words + kStkMirror;
+    std::vector<int64_t> lvl(m.ntiles + 1, 0);
+    for (int64_t t = 0; t < m.ntiles; t++) lvl[t + 1] = lvl[t] + hh[t];
+    if (m.ring > kStkMaxRing || lvl[m.ntiles] * 32 * vb + rec_bytes + places * 4 > most_bytes) return without();
+    m.val = get(size_t(lvl[m.ntiles]) * 32 * vb + 16, mine);
+    if (!m.val) return without();
+    int hflag = 0;
+    e = cudaMemcpyAsync(m.lvl, lvl.data(), sizeof(int64_t) * (m.ntiles + 1), cudaMemcpyHostToDevice, st);
+    if (e == cudaSuccess) e = cudaMemsetAsync(m.val, 0, size_t(lvl[m.ntiles]) * 32 * vb + 16, st);
+    if (e == cudaSuccess) e = cudaMemsetAsync(d.flag, 0, sizeof(int), st);
+    if (e == cudaSuccess)
+        e = stk_fill(I, J, m, d.rowptr, d.col, d.rval, vb, lanes, rank, start, d.flag, d.sm_count, st);
+    if (e == cudaSuccess) e = cudaMemcpyAsync(&hflag, d.flag, sizeof(int), cudaMemcpyDeviceToHost, st);
+    if (e == cudaSuccess) e = cudaMemsetAsync(d.flag, 0, sizeof(int), st);
+    if (e == cudaSuccess) e = cudaStreamSynchronize(st);
+    if (e != cudaSuccess) return broken(e);
+    if (hflag) {
+        drop(tmp);
+        drop(mine);
+        m = StackMat{};
+        return fail(h, SGTV_ERR_CUDA, "internal: the stacked row form failed its set-up check");
+    }
+    if (parts) {
+        m.poff = static_cast<int32_t *>(next(pk, keep[4]));
+        m.ppos = static_cast<int32_t *>(next(pk, keep[5]));
+        void *const u = next(pk, keep[6]);
+        int32_t *col_cnt = static_cast<int32_t *>(next(pw, work[4]));
+        std::vector<int32_t> hc(J), off(J + 1, 0);
+        e = cudaMemsetAsync(col_cnt, 0, sizeof(int32_t) * J, st);
+        if (e == cudaSuccess) {
+            stk_colcount(m, col_cnt, st);
+            e = cudaGetLastError();
+        }
+        if (e == cudaSuccess) e = cudaMemcpyAsync(hc.data(), col_cnt, sizeof(int32_t) * J, cudaMemcpyDeviceToHost, st);
+        if (e == cudaSuccess) e = cudaStreamSynchronize(st);
+        if (e != cudaSuccess) return broken(e);
+        int32_t widest = 0;
+        for (int64_t j = 0; j < J; j++) {  // at most `places` < 2^31 in all
+            off[j + 1] = off[j] + hc[j];
+            if (hc[j] > widest) widest = hc[j];
+        }
+        // a column in very many tiles would make its one thread sort and add for long
+        if (widest > 1024) return without();
+        int32_t *ent = static_cast<int32_t *>(get(sizeof(int32_t) * off[J], tmp));
+        m.part = get(sizeof(float) * off[J], mine);
+        if (!ent || !m.part) return without();
+        e = cudaMemcpyAsync(m.poff, off.data(), sizeof(int32_t) * (J + 1), cudaMemcpyHostToDevice, st);
+        if (e == cudaSuccess) e = cudaMemsetAsync(m.ppos, 0xFF, sizeof(int32_t) * places, st);
+        if (e == cudaSuccess) e = cudaMemsetAsync(m.part, 0, sizeof(float) * off[J], st);
+        if (e == cudaSuccess) {
+            stk_place(J, m, col_cnt, ent, st);
+            e = cudaGetLastError();
+        }
+        if (e == cudaSuccess) e = cudaStreamSynchronize(st);
+        if (e != cudaSuccess) return broken(e);
+        h->u_buf = u;
+    }
+    drop(tmp);
+    m.built = 1;
+    return SGTV_OK;
+}
+
+// Two-pass handles: the stacked pair reads u = d - c, which the shrink writes
+// while Dev::u is set; called whenever the chosen variants change.
+cudaError_t follow_variants(sgtv_t h)
+{
+    if (h->single_pass) return cudaSuccess;
+    const bool stacked = h->ks->back_need[h->v_back] == 2;
+    const bool was = h->d.u != nullptr;
+    h->d.u = stacked ? h->u_buf : nullptr;
+    if (!stacked || was) return cudaSuccess;
+    cudaError_t e = join_shrink(h);
+    if (e != cudaSuccess) return e;
+    h->ks->sub(h->d.J * h->g.n_dirs, h->d.d, h->d.c, h->d.u, h->stream);
+    return cudaGetLastError();
 }
 
 }  // namespace
@@ -901,6 +1102,10 @@ static int setup_impl(sgtv_t *out, int32_t nscans, const sgtv_scan *sc, const sg
         SK(cudaStreamSynchronize(st));
         if (hflag & 32) return bail(fail(h, SGTV_ERR_CUDA, "the single-pass row stream failed its set-up check"));
         d.sp.built = 1;
+    }
+    if (nnz > 0 && !h->persistent) {
+        const int trc = build_stack(h, !h->single_pass);
+        if (trc != SGTV_OK) return bail(trc);
     }
     // y and r (expanded to one value per measurement unless a single scalar)
     {
@@ -1326,47 +1531,81 @@ int sgtv_autotune(sgtv_t h, int32_t reps)
     cudaEvent_t a, b;
     CK(h, cudaEventCreate(&a));
     CK(h, cudaEventCreate(&b));
-    auto time_it = [&](auto &&launch, float *ms) -> cudaError_t {
+    // Mean time of `reps` launches. Where a launch is long (50 us, so that one
+    // more wait for the stream counts for little), a form whose first launch
+    // after the warm-up takes over 1.5 times the best so far is out of the
+    // running at once.
+    auto time_it = [&](auto &&launch, float *ms, float so_far) -> cudaError_t {
         launch();  // warm-up (also the first-launch occupancy query)
-        cudaError_t e = cudaEventRecord(a, st);
-        for (int k = 0; k < reps; k++) launch();
-        if (e == cudaSuccess) e = cudaEventRecord(b, st);
-        if (e == cudaSuccess) e = cudaEventSynchronize(b);
-        if (e == cudaSuccess) e = cudaEventElapsedTime(ms, a, b);
-        if (e == cudaSuccess) e = cudaGetLastError();
+        cudaError_t e = cudaSuccess;
+        for (int pass = so_far > 0.05f ? 0 : 1; pass < 2 && e == cudaSuccess; pass++) {
+            const int n = pass == 0 ? 1 : reps;
+            e = cudaEventRecord(a, st);
+            for (int k = 0; k < n; k++) launch();
+            if (e == cudaSuccess) e = cudaEventRecord(b, st);
+            if (e == cudaSuccess) e = cudaEventSynchronize(b);
+            if (e == cudaSuccess) e = cudaEventElapsedTime(ms, a, b);
+            if (e == cudaSuccess) e = cudaGetLastError();
+            *ms /= float(n);
+            if (*ms > 1.5f * so_far) break;
+        }
         return e;
     };
     // Only scratch is written (ratio, f_next): the ADMM state is untouched.
     // The single-pass form times only its scatter forms (the two-pass
     // products serve it only for the KKT measure).
-    float best = 3.4e38f;
-    int best_v = 0;
+    // The stacked pair is one choice: timed together, against the sum of the
+    // best of the others.
+    float best = 3.4e38f, other = 0.f;
+    int best_v = 0, stk_f = -1, stk_b = -1;
+    for (int v = 0; v < h->ks->n_fwd; v++)
+        if (h->ks->fwd_need[v] == 2 && variant_ok(d, d.tr, 2)) stk_f = v;
+    for (int v = 0; v < h->ks->n_back; v++)
+        if (h->ks->back_need[v] == 2 && variant_ok(d, d.tc, 2)) stk_b = v;
     for (int v = 0; v < h->ks->n_fwd && !h->single_pass; v++) {
-        if (!variant_ok(d.tr, h->ks->fwd_need[v])) continue;
+        if (h->ks->fwd_untimed[v] || h->ks->fwd_need[v] == 2 || !variant_ok(d, d.tr, h->ks->fwd_need[v])) continue;
         float ms = 0;
-        cudaError_t e = time_it([&] { h->ks->fwd[v](d, d.f, d.ratio, st); }, &ms);
+        cudaError_t e = time_it([&] { h->ks->fwd[v](d, d.f, d.ratio, st); }, &ms, best);
         if (e != cudaSuccess) { cudaEventDestroy(a); cudaEventDestroy(b); return cuda_fail(h, e, "autotune forward"); }
         if (ms < best) { best = ms; best_v = v; }
     }
     h->v_fwd = best_v;
     h->ks->fwd[h->v_fwd](d, d.f, d.ratio, st);
+    other = best;
     best = 3.4e38f;
     best_v = 0;
     for (int v = 0; v < h->ks->n_back && !h->single_pass; v++) {
-        if (!variant_ok(d.tc, h->ks->back_need[v])) continue;
+        if (h->ks->back_untimed[v] || h->ks->back_need[v] == 2 || !variant_ok(d, d.tc, h->ks->back_need[v])) continue;
         float ms = 0;
-        cudaError_t e = time_it([&] { h->ks->back[v](d, h->g, d.f, d.f_next, st); }, &ms);
+        cudaError_t e = time_it([&] { h->ks->back[v](d, h->g, d.f, d.f_next, st); }, &ms, best);
         if (e != cudaSuccess) { cudaEventDestroy(a); cudaEventDestroy(b); return cuda_fail(h, e, "autotune backprojection"); }
         if (ms < best) { best = ms; best_v = v; }
     }
     h->v_back = best_v;
+    if (!h->single_pass && !h->persistent && stk_f >= 0 && stk_b >= 0) {
+        void *const u = d.u;
+        d.u = h->u_buf;
+        float ms = 0;
+        cudaError_t e = time_it(
+            [&] {
+                h->ks->fwd[stk_f](d, d.f, d.ratio, st);
+                h->ks->back[stk_b](d, h->g, d.f, d.f_next, st);
+            },
+            &ms, other + best);
+        d.u = u;
+        if (e != cudaSuccess) { cudaEventDestroy(a); cudaEventDestroy(b); return cuda_fail(h, e, "autotune stacked form"); }
+        if (ms < other + best) {
+            h->v_fwd = stk_f;
+            h->v_back = stk_b;
+        }
+    }
     if (h->single_pass) {
         // the scatter accumulates into e_acc: cleared again after the timing
         float bests = 3.4e38f;
-        for (int v = 0; v < h->ks->n_scatter; v++) {
-            if (!scatter_fits(h, v)) continue;
+        for (int v = h->ks->n_scatter - 1; v >= 0; v--) {  // the likeliest first
+            if (h->ks->scatter_untimed[v] || !scatter_fits(h, v)) continue;
             float ms = 0;
-            cudaError_t e = time_it([&] { h->ks->scatter[v](d, d.f, h->e_acc, st); }, &ms);
+            cudaError_t e = time_it([&] { h->ks->scatter[v](d, d.f, h->e_acc, st); }, &ms, bests);
             if (e != cudaSuccess) { cudaEventDestroy(a); cudaEventDestroy(b); return cuda_fail(h, e, "autotune scatter"); }
             if (ms < bests) { bests = ms; h->v_scatter = v; }
         }
@@ -1390,7 +1629,7 @@ int sgtv_autotune(sgtv_t h, int32_t reps)
         for (int pv = 0; pv < h->ks->n_pers; pv++) {
             float ms = 0;
             cudaError_t lerr = cudaSuccess;
-            cudaError_t e = time_it([&] { lerr = h->ks->pers[pv](d, h->g, d.f, d.f_next, 0, h->bar, st); }, &ms);
+            cudaError_t e = time_it([&] { lerr = h->ks->pers[pv](d, h->g, d.f, d.f_next, 0, h->bar, st); }, &ms, bestp);
             if (e == cudaSuccess) e = lerr;
             if (e != cudaSuccess) { cudaEventDestroy(a); cudaEventDestroy(b); return cuda_fail(h, e, "autotune persistent"); }
             if (ms < bestp) {
@@ -1404,6 +1643,7 @@ int sgtv_autotune(sgtv_t h, int32_t reps)
     drop_graphs(h);
     cudaEventDestroy(a);
     cudaEventDestroy(b);
+    CK(h, follow_variants(h));
     int fl = 0;
     CK(h, cudaMemcpy(&fl, h->d.flag, sizeof(int), cudaMemcpyDeviceToHost));
     if (fl & 2) return fail(h, SGTV_ERR_TIMEOUT, "a bounded device-side wait gave up");
@@ -1424,14 +1664,17 @@ int sgtv_set_variants(sgtv_t h, int32_t fwd, int32_t back)
     if (rc) return rc;
     if (fwd < 0 || fwd >= h->ks->n_fwd || back < 0 || back >= h->ks->n_back)
         return SGTV_ERR_ARG;  // not sticky: the handle keeps its variants
-    if (!variant_ok(h->d.tr, h->ks->fwd_need[fwd]) || !variant_ok(h->d.tc, h->ks->back_need[back]))
+    if (!variant_ok(h->d, h->d.tr, h->ks->fwd_need[fwd]) || !variant_ok(h->d, h->d.tc, h->ks->back_need[back]))
         return SGTV_ERR_ARG;  // that tiled form was not built for this matrix
+    if ((h->ks->fwd_need[fwd] == 2) != (h->ks->back_need[back] == 2))
+        return SGTV_ERR_ARG;  // the stacked backprojection reads what the stacked forward pass left
     if (h->persistent && pers_index(h, fwd, back) < 0)
         return SGTV_ERR_ARG;  // the persistent kernel fuses only the tli_u8 / tli_v4x2 forms
     if (h->persistent) h->v_pers = (h->v_pers & 4) | pers_index(h, fwd, back);
     h->v_fwd = fwd;
     h->v_back = back;
     drop_graphs(h);
+    CK(h, follow_variants(h));
     return SGTV_OK;
 }
 

@@ -66,6 +66,38 @@ struct SpStream {
     int built;
 };
 
+// Stacked row form (FP32 vectors; see sgtv_stack.cu): per tile of `tr` rows
+// the columns dealt to the lanes of one warp, per row a bit per (lane, word),
+// the values in 32 stacks.
+constexpr int kStkMaxWords = 24;  // columns of a tile <= 32 * 24
+constexpr int kStkMaxRows = 64;   // even: rows are taken in pairs
+constexpr int kStkAhead = 2;      // pairs of rows whose levels are in flight ahead of the one at work
+constexpr int kStkMirror = 8;     // the ring's first levels are repeated behind its end
+constexpr int kStkMaxRing = 128;  // levels: a place in the ring takes 12 bits
+constexpr int kStkShortWords = 10;  // 32-bit records up to here
+constexpr int stk_rec_bytes(int words) { return words <= kStkShortWords ? 4 : 8; }
+// Resident one-warp blocks per multiprocessor asked of the register allocator:
+// f, the sums and two rows' values are 4 registers per word, about 30 more (at
+// 20 words 16 blocks without spills and 18 with a few take the same time, 22
+// half as much again).
+constexpr int stk_min_blocks(int words) { return words <= 8 ? 28 : (words <= 12 ? 24 : (words <= 20 ? 18 : 16)); }
+struct StackMat {
+    int built;
+    int tr;               // rows per tile
+    int words;            // columns per lane (one of the instantiated sizes)
+    int ring;             // levels of the ring
+    int64_t ntiles;
+    int32_t *uidx;        // [ntiles][words][32] column of (word, lane); -1: none
+    void *rec;            // [(I + 1) / 2][32] records of stk_rec_bytes(words) bytes
+    uint32_t *ctl;        // [(I + 1) / 2] the copy that brings the pair's levels (copy_code)
+    int64_t *lvl;         // [ntiles + 1] first level of each tile
+    void *val;            // [lvl[ntiles]][32] values of type V
+    // partial sums of e by column (two-pass form; NULL otherwise)
+    int32_t *ppos;        // [ntiles][words][32] place in part; -1: none
+    int32_t *poff;        // [J + 1] first partial of each column
+    void *part;           // [poff[J]]
+};
+
 // Device pointers of one problem; vector element type depends on the precision
 // (float, or double in the FP64 mode), A's value type on the precision too.
 struct Dev {
@@ -83,12 +115,13 @@ struct Dev {
     void *d_prev;             // d before the last shrink, [n_dirs][J]; the next shrink
                               // writes there and the two buffers swap
     void *u;                  // u = d - c, [n_dirs][J], kept by the shrink for the
-                              // single-pass f-update (NULL in the other forms)
+                              // f-update of the single-pass and stacked forms (else NULL)
     double *part;             // reduction partials, >= 4 * red_blocks doubles
     double *red;              // reduced results (device), >= 8 doubles
     int *flag;                // bit 0: non-finite iterate, bit 1: a bounded wait gave up
     TliMat tr, tc;            // tiled local-index forms of the CSR and CSC copies
     SpStream sp;              // single-pass row stream (sp.built = 0 unless requested)
+    StackMat st;              // stacked row form (st.built = 0 where it does not apply)
     int sm_count;
     int smem_optin;           // opt-in shared memory per block (bytes)
     int red_blocks;           // grid of the reduction kernels
@@ -116,7 +149,11 @@ struct KernelSet {
     int n_fwd;
     ForwardFn fwd[kMaxVariants];
     const char *fwd_name[kMaxVariants];
-    int fwd_need[kMaxVariants];     // 0 plain; 1 tiled (Dev::tr); NS >= 3: TMA pipeline of NS stages
+    // *_untimed = 1: kept for callers that pin it, but not a candidate of the autotuner (another form of
+    // the list was faster on every problem measured)
+    int fwd_untimed[kMaxVariants], back_untimed[kMaxVariants], scatter_untimed[kMaxVariants];
+    int fwd_need[kMaxVariants];     // 0 plain; 1 tiled (Dev::tr); 2 stacked (Dev::st with partial sums;
+                                    // both products or neither); NS >= 3: TMA pipeline of NS stages
     int n_back;
     BackUpdateFn back[kMaxVariants];
     const char *back_name[kMaxVariants];
@@ -131,7 +168,7 @@ struct KernelSet {
     void (*scatter[kMaxVariants])(const Dev &, const void *f, void *e, cudaStream_t);
     const char *scatter_name[kMaxVariants];
     int scatter_bufs[kMaxVariants];  // staging-sized shared-memory buffers the variant needs (with the f stage)
-    int scatter_sp[kMaxVariants];    // 1: reads the single-pass row stream (Dev::sp)
+    int scatter_sp[kMaxVariants];    // 1: reads the single-pass row stream (Dev::sp); 2: the stacked form (Dev::st)
     void (*fupdate)(const Dev &, const Geom &, void *e, const void *f, void *f_new, cudaStream_t);
     int n_pers;                      // persistent one-launch iterations (need Dev::tr and Dev::tc)
     PersistentFn pers[8];
@@ -204,6 +241,22 @@ cudaError_t tli_list_build(const int64_t *ptr, const int32_t *idx, int64_t nseg,
 cudaError_t sp_build(int64_t I, const int64_t *rowptr, const uint16_t *lidx, const void *val, int val_bytes,
                      const int64_t *sp_rp, const int32_t *wlen, const int64_t *uoff, uint16_t *sp_lidx, void *sp_val,
                      int *flag, int sm_count, cudaStream_t st);
+
+// Stacked row form (sgtv_stack.cu). stk_count: *out = largest number of
+// distinct columns of a tile. stk_build: uidx, rec, ctl, the lane of each
+// column of the ascending list, each nonzero's place in that list, each
+// record's first level and stack, the tile heights, stats[0] = levels the ring
+// needs. stk_fill: the values (m.val zeroed beforehand), then a check (flag
+// bit 64). stk_colcount / stk_place: where the partial sums of e go.
+cudaError_t stk_count(int64_t I, int64_t J, int tr, const int64_t *ptr, const int32_t *idx, int *out,
+                      cudaStream_t st);
+cudaError_t stk_build(int64_t I, int64_t J, const StackMat &m, const int64_t *ptr, const int32_t *idx, uint8_t *lanes,
+                      uint16_t *rank, uint16_t *start, int32_t *height, int *stats, cudaStream_t st);
+cudaError_t stk_fill(int64_t I, int64_t J, const StackMat &m, const int64_t *ptr, const int32_t *idx, const void *val,
+                     int val_bytes, const uint8_t *lanes, const uint16_t *rank, const uint16_t *start, int *flag,
+                     int sm_count, cudaStream_t st);
+void stk_colcount(const StackMat &m, int32_t *cnt, cudaStream_t st);
+void stk_place(int64_t J, const StackMat &m, int32_t *cnt, int32_t *ent, cudaStream_t st);
 
 // a[k] += off for k < n (offsetting one scan's indices inside a batch).
 void add_offset_i32(int32_t *a, int64_t n, int32_t off, cudaStream_t st);

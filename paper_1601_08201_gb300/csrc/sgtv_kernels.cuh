@@ -18,6 +18,8 @@
 #include <cuda_runtime.h>
 #include <stdint.h>
 
+#include <type_traits>
+
 #include "sgtv_internal.h"
 
 namespace sgtv {
@@ -1609,10 +1611,22 @@ k_scatter_sp(int64_t I, int64_t J, const int64_t *__restrict__ rp, const uint16_
 // offsets) is found once per warp, and QB q-steps of every lane issue all
 // their loads before any arithmetic, which is that of voxel_update_at in the
 // same order.
-template <typename T, int QB>
+//
+// poff = NULL: e is the accumulated vector, cleared here. Else e holds
+// partial sums (k_rows_stack), those of hyper-voxel j at poff[j] .. poff[j+1],
+// added up in that order.
+template <typename T>
+__device__ __forceinline__ T sum_parts(const T *__restrict__ part, const int32_t *__restrict__ poff, int64_t j)
+{
+    T a = T(0);
+    for (int k = poff[j], k1 = poff[j + 1]; k < k1; k++) a += part[k];
+    return a;
+}
+
+template <typename T, int QB, bool PART = false>
 __global__ void __launch_bounds__(256, QB == 1 ? 4 : 3)
 k_fupdate_site(Geom g, T *__restrict__ e, const T *__restrict__ s, const T *__restrict__ f,
-               const T *__restrict__ u, T *__restrict__ f_new)
+               const T *__restrict__ u, T *__restrict__ f_new, const int32_t *__restrict__ poff = nullptr)
 {
     const int lane = threadIdx.x & 31;
     const int64_t nwarps = (int64_t(gridDim.x) * blockDim.x) >> 5;
@@ -1640,7 +1654,7 @@ k_fupdate_site(Geom g, T *__restrict__ e, const T *__restrict__ s, const T *__re
                 const int q = q0 + 32 * b + lane;
                 const bool act = q < L.Nq;
                 const int64_t j = v0 + (act ? q : 0);
-                ej[b] = e[j];
+                ej[b] = PART ? sum_parts<T>(e, poff, j) : e[j];
                 fj[b] = f[j];
                 sj[b] = s[j];
 #pragma unroll
@@ -1657,7 +1671,7 @@ k_fupdate_site(Geom g, T *__restrict__ e, const T *__restrict__ s, const T *__re
                 const int q = q0 + 32 * b + lane;
                 if (q >= L.Nq) continue;
                 const int64_t j = v0 + q;
-                e[j] = T(0);
+                if (!PART) e[j] = T(0);
                 T alpha = T(0), gamma = T(0);
 #pragma unroll
                 for (int p = 0; p < 4; p++) {
@@ -1685,14 +1699,14 @@ k_fupdate_site(Geom g, T *__restrict__ e, const T *__restrict__ s, const T *__re
 }
 
 // Same update, one thread per hyper-voxel.
-template <typename T>
+template <typename T, bool PART = false>
 __global__ void __launch_bounds__(256)
 k_fupdate(Geom g, T *__restrict__ e, const T *__restrict__ s, const T *__restrict__ f, const T *__restrict__ d,
-          const T *__restrict__ c, T *__restrict__ f_new)
+          const T *__restrict__ c, T *__restrict__ f_new, const int32_t *__restrict__ poff = nullptr)
 {
     for (int64_t j = int64_t(blockIdx.x) * blockDim.x + threadIdx.x; j < g.J; j += int64_t(gridDim.x) * blockDim.x) {
-        const T ej = e[j];
-        e[j] = T(0);
+        const T ej = PART ? sum_parts<T>(e, poff, j) : e[j];
+        if (!PART) e[j] = T(0);
         f_new[j] = voxel_update<T, true>(g, j, ej, s, f, d, c);
     }
 }
@@ -1967,6 +1981,275 @@ k_back_update_tma(TmaMat m, TmaLayout L, Geom g, const V *__restrict__ val, cons
     TmaPipe<T, V, kTliTile, NS, NW>::run(m, L, val, ratio, flag, [&](int64_t j, T e) {
         f_new[j] = voxel_update<T>(g, j, e, s, f, d, c);
     });
+}
+
+// ---------------------------------------------------------------------------------------
+// The row pass over the stacked form (sgtv_stack.cu): a1 and a2 in one read
+// of A, by one warp per tile.
+//
+// Each lane keeps its columns' f and sums of a_ij ratio_i in registers, so a
+// nonzero costs neither a gather nor a scatter: per row and word a lane tests
+// its bit, reads the next value of its stack from the ring if it is set, and
+// two packed FP32 multiply-adds (one per word pair in the product, one in the
+// sums) take two words at once; words without a nonzero add 0.
+//
+// The row stream it replaces as the first choice (k_scatter_sp) is bound by
+// instruction issue: 12.4 warp instructions per 32 nonzeros for the gather,
+// the accumulator's read and write and the index, and 134 per row. Here a row
+// takes about 4.5 per word (32 columns) and about 45, and A is 4.1 + 0.5
+// bytes per nonzero on the 2^28-nonzero problem (256 a row, 19 words) instead
+// of 6. The measured times stand at the launcher (RowsStack).
+//
+// Ring: level l of the tile sits at place l mod ring; the first levels are
+// repeated behind the end, so a lane's pointer is wrapped once per 8 words. One
+// copy and one mbarrier phase per pair of rows, kStkAhead pairs ahead.
+//
+// PART = false: the sums go to e by global adds (single-pass form, order set
+// by the adds). PART = true: ratio is written and each sum goes to its place
+// among its column's partial sums, ordered by tile, which the f-update adds
+// up in that order (two-pass form: deterministic).
+
+// d = a * b + c on two packed FP32 lanes, each rounded as fmaf rounds.
+__device__ __forceinline__ uint64_t fma2(uint64_t a, uint64_t b, uint64_t c)
+{
+    uint64_t d;
+    asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(d) : "l"(a), "l"(b), "l"(c));
+    return d;
+}
+__device__ __forceinline__ uint64_t pack2(float x, float y)
+{
+    uint64_t d;
+    asm("mov.b64 %0, {%1, %2};" : "=l"(d) : "f"(x), "f"(y));
+    return d;
+}
+__device__ __forceinline__ void unpack2(uint64_t v, float &x, float &y)
+{
+    asm("mov.b64 {%0, %1}, %2;" : "=f"(x), "=f"(y) : "l"(v));
+}
+
+// If bit `bit` of mk is set: v = the value at the shared-memory address ptr, and
+// ptr moves up one level; else v = 0 (what the load found there is dropped).
+template <typename V>
+__device__ __forceinline__ void stk_pop(float &v, uint32_t &ptr, uint32_t mk, uint32_t bit)
+{
+    if constexpr (sizeof(V) == 4) {
+        asm volatile("{\n\t.reg .pred p;\n\t.reg .b32 t;\n\t.reg .f32 x;\n\t"
+                     "ld.shared.f32 x, [%1];\n\t"
+                     "and.b32 t, %2, %3;\n\tsetp.ne.u32 p, t, 0;\n\t"
+                     "@p add.u32 %1, %1, 128;\n\tselp.f32 %0, x, 0f00000000, p;\n\t}"
+                     : "=f"(v), "+r"(ptr) : "r"(mk), "r"(bit));
+    } else {
+        asm volatile("{\n\t.reg .pred p;\n\t.reg .b32 t, x;\n\t.reg .b16 h;\n\t"
+                     "ld.shared.b16 h, [%1];\n\t"
+                     "and.b32 t, %2, %3;\n\tsetp.ne.u32 p, t, 0;\n\t"
+                     "@p add.u32 %1, %1, 64;\n\tcvt.u32.u16 x, h;\n\tshl.b32 x, x, 16;\n\t"
+                     "selp.b32 %0, x, 0, p;\n\t}"
+                     : "=f"(v), "+r"(ptr) : "r"(mk), "r"(bit));
+    }
+}
+
+// A lane's record of a pair of rows: both rows' bits and the first value's
+// place in the ring (sgtv_stack.cu).
+__device__ __forceinline__ void stk_split(uint32_t v, uint32_t &a, uint32_t &b, uint32_t &at)
+{
+    a = v;  // bits past the words are not looked at
+    b = v >> 10;
+    at = v >> 20;
+}
+__device__ __forceinline__ void stk_split(uint64_t v, uint32_t &a, uint32_t &b, uint32_t &at)
+{
+    a = uint32_t(v);
+    b = uint32_t(v >> 24);
+    at = uint32_t(v >> 48);
+}
+
+// One lane issues: the predicate keeps the warp converged.
+__device__ __forceinline__ void mbar_expect_if(bool p, uint32_t bar, uint32_t bytes)
+{
+    asm volatile("{\n\t.reg .pred q;\n\tsetp.ne.b32 q, %2, 0;\n\t"
+                 "@q mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;\n\t}"
+                 ::"r"(bar), "r"(bytes), "r"(int(p)) : "memory");
+}
+__device__ __forceinline__ void bulk_g2s_if(bool p, uint32_t dst, const void *src, uint32_t bytes, uint32_t bar)
+{
+    asm volatile("{\n\t.reg .pred q;\n\tsetp.ne.b32 q, %4, 0;\n\t"
+                 "@q cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];\n\t}"
+                 ::"r"(dst), "l"(src), "r"(bytes), "r"(bar), "r"(int(p)) : "memory");
+}
+__device__ __forceinline__ bool mbar_try(uint32_t bar, uint32_t parity)
+{
+    uint32_t done;
+    asm volatile("{\n\t.reg .pred p;\n\t"
+                 "mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n\t"
+                 "selp.u32 %0, 1, 0, p;\n\t}"
+                 : "=r"(done) : "r"(bar), "r"(parity) : "memory");
+    return done != 0;
+}
+
+template <typename V, int W, bool PART>
+__global__ void __launch_bounds__(32, stk_min_blocks(W))
+k_rows_stack(int64_t I, StackMat m, const float *__restrict__ f, const float *__restrict__ r, int r_scalar,
+             const float *__restrict__ y, float *__restrict__ out, float *__restrict__ ratio, int *__restrict__ flag)
+{
+    using M = typename std::conditional<(W <= kStkShortWords), uint32_t, uint64_t>::type;
+    constexpr uint32_t kLevel = 32 * uint32_t(sizeof(V));  // bytes of one level
+    extern __shared__ __align__(128) unsigned char smem_raw[];
+    __shared__ uint64_t bar[kStkAhead];
+    const int lane = threadIdx.x;
+    const int64_t t = blockIdx.x, r0 = t * m.tr;
+    const int n = int(I - r0 < m.tr ? I - r0 : m.tr);
+    const int np = (n + 1) >> 1;
+    const uint32_t ring0 = smem_u32(smem_raw), ring_bytes = uint32_t(m.ring) * kLevel;
+    const uint32_t ring_end = ring0 + ring_bytes, bar0 = smem_u32(bar);
+    const uint32_t *__restrict__ cp = m.ctl + (r0 >> 1);
+    const unsigned char *src = static_cast<const unsigned char *>(m.val) + m.lvl[t] * int64_t(kLevel);
+    // the copy of one pair's levels (copy_code in sgtv_stack.cu), completing on `b`
+    auto issue = [&](uint32_t c, uint32_t b) {
+        const uint32_t a = (c & 127u) * kLevel, n1 = ((c >> 13) & 127u) * kLevel, n2 = ((c >> 20) & 63u) * kLevel;
+        const bool over = (c >> 26) != 0u;
+        mbar_expect_if(lane == 0, b, n1 + n2);
+        bulk_g2s_if(lane == 0 && n1 != 0u, ring0 + a, src, n1, b);
+        if (n2 != 0u)  // warp-uniform; every third pair or so
+            bulk_g2s_if(lane == 0, over ? ring0 : ring_end + a, src + (over ? ring_bytes - a : 0u), n2, b);
+        src += ((c >> 7) & 63u) * kLevel;
+    };
+    if (lane == 0) {
+        for (int k = 0; k < kStkAhead; k++) mbar_init(&bar[k], 1);
+        asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+        asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+    }
+    __syncwarp();
+    for (int k = 0; k < kStkAhead && k < np; k++) issue(__ldg(cp + k), bar0 + 8 * k);
+
+    const int32_t *__restrict__ cols = m.uidx + (t * W) * 32 + lane;
+    uint64_t fv[W / 2], acc[W / 2];
+#pragma unroll
+    for (int w = 0; w < W / 2; w++) {
+        const int32_t a = __ldg(cols + 64 * w), b = __ldg(cols + 64 * w + 32);
+        fv[w] = pack2(a >= 0 ? __ldg(f + a) : 0.f, b >= 0 ? __ldg(f + b) : 0.f);
+        acc[w] = 0;
+    }
+    const M *__restrict__ rp = static_cast<const M *>(m.rec) + (r0 >> 1) * 32 + lane;
+    const float rs = r_scalar ? r[0] : 0.f;
+    M rec = __ldcs(rp);
+    uint32_t slot = 0, phase = 0;
+    bool bad = false;
+    auto landed = [&](uint32_t b, uint32_t ph) {  // false: not within 1 s, far beyond any healthy copy
+        bool ok = mbar_try(b, ph);
+        if (!ok) {
+            const uint64_t t0 = global_ns();
+            while (!(ok = mbar_try(b, ph)) && global_ns() - t0 < 1000000000ull) {}
+        }
+        return ok;
+    };
+#pragma unroll 1
+    for (int g0 = 0; g0 < n && !bad; g0 += 32) {
+        const int gn = n - g0 < 32 ? n - g0 : 32;
+        const int64_t row = r0 + g0 + lane;
+        const float yl = lane < gn ? y[row] : 0.f;
+        const float rl = (!r_scalar && lane < gn) ? r[row] : 0.f;
+        const int pc = (g0 >> 1) + kStkAhead + lane;  // the copies to issue in this group of rows
+        const uint32_t cl = pc < np ? __ldcs(cp + pc) : 0u;
+        float rat = 0.f;
+#pragma unroll 1
+        for (int k = 0; k < gn; k += 2) {  // two rows at a time (the second may be past the tile: no bits)
+            uint32_t mka, mkb, ptr;
+            stk_split(rec, mka, mkb, ptr);
+            ptr = ring0 + ptr * uint32_t(sizeof(V));
+            rp += 32;
+            if (g0 + k + 2 < n) rec = __ldcs(rp);  // the next pair's, in flight
+            if (!__all_sync(0xffffffffu, landed(bar0 + 8 * slot, phase))) {
+                bad = true;
+                break;
+            }
+            uint64_t va[W / 2], vb[W / 2], da0 = 0, da1 = 0, db0 = 0, db1 = 0;
+#pragma unroll
+            for (int w = 0; w < W; w += 2) {
+                if ((w & 7) == 0) ptr = ptr >= ring_end ? ptr - ring_bytes : ptr;
+                float x, z;
+                stk_pop<V>(x, ptr, mka, 1u << w);
+                stk_pop<V>(z, ptr, mka, 2u << w);
+                va[w / 2] = pack2(x, z);
+                if (w & 2) da1 = fma2(va[w / 2], fv[w / 2], da1);
+                else da0 = fma2(va[w / 2], fv[w / 2], da0);
+            }
+#pragma unroll
+            for (int w = 0; w < W; w += 2) {
+                if ((w & 7) == 0) ptr = ptr >= ring_end ? ptr - ring_bytes : ptr;
+                float x, z;
+                stk_pop<V>(x, ptr, mkb, 1u << w);
+                stk_pop<V>(z, ptr, mkb, 2u << w);
+                vb[w / 2] = pack2(x, z);
+                if (w & 2) db1 = fma2(vb[w / 2], fv[w / 2], db1);
+                else db0 = fma2(vb[w / 2], fv[w / 2], db0);
+            }
+            // both products in one tree: the lower half-warp ends with row k's, the upper with row k + 1's
+            float s0, s1, s2, s3;
+            unpack2(da0, s0, s1);
+            unpack2(da1, s2, s3);
+            const float pa = (s0 + s1) + (s2 + s3);
+            unpack2(db0, s0, s1);
+            unpack2(db1, s2, s3);
+            const float pb = (s0 + s1) + (s2 + s3);
+            const bool up = lane >= 16;
+            float dot = (up ? pb : pa) + __shfl_xor_sync(0xffffffffu, up ? pa : pb, 16);
+#pragma unroll
+            for (int o = 8; o > 0; o >>= 1) dot += __shfl_xor_sync(0xffffffffu, dot, o);
+            const int kk = k + (up ? 1 : 0);
+            const float yi = __shfl_sync(0xffffffffu, yl, kk);
+            const float ri = r_scalar ? rs : __shfl_sync(0xffffffffu, rl, kk);
+            const float q = yi != 0.f ? yi / (dot + ri) : 0.f;
+            const float qa = __shfl_sync(0xffffffffu, q, 0), qb = __shfl_sync(0xffffffffu, q, 16);
+            if (qa != 0.f) {  // warp-uniform; a zero count adds nothing
+                const uint64_t q2 = pack2(qa, qa);
+#pragma unroll
+                for (int w = 0; w < W / 2; w++) acc[w] = fma2(va[w], q2, acc[w]);
+            }
+            if (qb != 0.f) {
+                const uint64_t q2 = pack2(qb, qb);
+#pragma unroll
+                for (int w = 0; w < W / 2; w++) acc[w] = fma2(vb[w], q2, acc[w]);
+            }
+            if (PART) {
+                if (lane == k) rat = qa;
+                if (lane == k + 1) rat = qb;
+            }
+            // every lane has read its values (the sums needed them): the pair's barrier and the room
+            // below are free for the copy kStkAhead pairs on
+            const uint32_t c = __shfl_sync(0xffffffffu, cl, k >> 1);
+            if ((g0 + k) / 2 + kStkAhead < np) issue(c, bar0 + 8 * slot);
+            if (++slot == kStkAhead) {
+                slot = 0;
+                phase ^= 1;
+            }
+        }
+        if (PART && lane < gn) ratio[row] = rat;
+    }
+    if (bad) {  // a copy never landed: record it, wait (bounded) for the ones in flight, leave
+        if (lane == 0) atomicOr(flag, 2);
+        for (int k = 0; k < kStkAhead; k++) {
+            landed(bar0 + 8 * slot, phase);
+            if (++slot == kStkAhead) {
+                slot = 0;
+                phase ^= 1;
+            }
+        }
+        return;
+    }
+    const int32_t *__restrict__ dst = PART ? m.ppos + (t * W) * 32 + lane : cols;
+#pragma unroll
+    for (int w = 0; w < W / 2; w++) {
+        float a, b;
+        unpack2(acc[w], a, b);
+        const int32_t ia = __ldg(dst + 64 * w), ib = __ldg(dst + 64 * w + 32);
+        if (PART) {
+            if (ia >= 0) out[ia] = a;
+            if (ib >= 0) out[ib] = b;
+        } else {
+            if (ia >= 0 && a != 0.f) atomicAdd(out + ia, a);
+            if (ib >= 0 && b != 0.f) atomicAdd(out + ib, b);
+        }
+    }
 }
 
 // ---------------------------------------------------------------------------------------

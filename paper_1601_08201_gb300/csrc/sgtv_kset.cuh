@@ -178,6 +178,54 @@ struct ScatterSp {
     }
 };
 
+// Row pass over the stacked form, by the number of words. One warp per tile,
+// with the ring's levels in shared memory. Measured against the forms it was
+// chosen over (microseconds, FP32 / BF16 values): 2^28 nonzeros, 256 a row:
+// 254 / 252 against 391 / 366 for the row-stream scatter; both products of a
+// two-pass iteration 284 with the f-update, against 607; 41 x 9 x 54 scan,
+// whose row-stream tiles stage 80 KB windows: 7.4 against 19.0.
+
+template <typename V, bool PART, int W>
+inline void rows_stack_w(const Dev &d, const void *f, void *out, void *ratio, cudaStream_t st)
+{
+    static int granted = 48 * 1024;
+    auto kern = k_rows_stack<V, W, PART>;
+    static const bool carved =
+        cudaFuncSetAttribute(kern, cudaFuncAttributePreferredSharedMemoryCarveout, 100) == cudaSuccess;
+    (void)carved;
+    const int smem = (d.st.ring + kStkMirror + 1) * 32 * int(sizeof(V));  // a lane may look one level past its last
+    ensure_smem(kern, smem, granted);
+    kern<<<unsigned(d.st.ntiles), 32, smem, st>>>(d.I, d.st, static_cast<const float *>(f),
+                                                  static_cast<const float *>(d.r), d.r_scalar,
+                                                  static_cast<const float *>(d.y), static_cast<float *>(out),
+                                                  static_cast<float *>(ratio), d.flag);
+}
+
+template <typename V, bool PART>
+struct RowsStack {
+    static void launch(const Dev &d, const void *f, void *out, void *ratio, cudaStream_t st)
+    {
+        switch (d.st.words) {
+        case 4: return rows_stack_w<V, PART, 4>(d, f, out, ratio, st);
+        case 6: return rows_stack_w<V, PART, 6>(d, f, out, ratio, st);
+        case 8: return rows_stack_w<V, PART, 8>(d, f, out, ratio, st);
+        case 10: return rows_stack_w<V, PART, 10>(d, f, out, ratio, st);
+        case 12: return rows_stack_w<V, PART, 12>(d, f, out, ratio, st);
+        case 14: return rows_stack_w<V, PART, 14>(d, f, out, ratio, st);
+        case 16: return rows_stack_w<V, PART, 16>(d, f, out, ratio, st);
+        case 18: return rows_stack_w<V, PART, 18>(d, f, out, ratio, st);
+        case 20: return rows_stack_w<V, PART, 20>(d, f, out, ratio, st);
+        case 22: return rows_stack_w<V, PART, 22>(d, f, out, ratio, st);
+        default: return rows_stack_w<V, PART, 24>(d, f, out, ratio, st);
+        }
+    }
+    static void scatter(const Dev &d, const void *f, void *e, cudaStream_t st) { launch(d, f, e, nullptr, st); }
+    static void forward(const Dev &d, const void *f, void *ratio, cudaStream_t st)
+    {
+        launch(d, f, d.st.part, ratio, st);
+    }
+};
+
 inline TmaMat tma_mat(const TliMat &m, const int64_t *ptr, int64_t nseg)
 {
     return TmaMat{ptr, m.lidx, m.wbase, m.wlen, m.uoff, m.uidx, nseg, m.ntiles};
@@ -357,6 +405,27 @@ struct Impl {
                                                   static_cast<const T *>(f), static_cast<const T *>(d.d),
                                                   static_cast<const T *>(d.c), static_cast<T *>(f_new));
     }
+    // The f-update from the partial sums that the stacked forward pass left.
+    template <int QB>
+    static void back_stack_site(const Dev &d, const Geom &g, const void *f, void *f_new, cudaStream_t st)
+    {
+        static const int nb = resident_blocks(k_fupdate_site<T, QB, true>);
+        k_fupdate_site<T, QB, true><<<grid_for(g.S, d.sm_count * nb), kThreads, 0, st>>>(
+            g, static_cast<T *>(d.st.part), static_cast<const T *>(d.s), static_cast<const T *>(f),
+            static_cast<const T *>(d.u), static_cast<T *>(f_new), d.st.poff);
+    }
+    static void back_stack(const Dev &d, const Geom &g, const void *f, void *f_new, cudaStream_t st)
+    {
+        if (g.max_nq >= 16) {
+            if (g.max_nq <= 32) back_stack_site<1>(d, g, f, f_new, st);
+            else back_stack_site<2>(d, g, f, f_new, st);
+            return;
+        }
+        int64_t blocks = (d.J + kThreads - 1) / kThreads;
+        k_fupdate<T, true><<<unsigned(blocks), kThreads, 0, st>>>(
+            g, static_cast<T *>(d.st.part), static_cast<const T *>(d.s), static_cast<const T *>(f),
+            static_cast<const T *>(d.d), static_cast<const T *>(d.c), static_cast<T *>(f_new), d.st.poff);
+    }
     static void backproject(const Dev &d, const void *v, void *out, cudaStream_t st)
     {
         k_backproject<T, V><<<grid_for(d.J, d.sm_count * 8), kThreads, 0, st>>>(
@@ -451,19 +520,22 @@ struct Impl {
         k.fwd[n] = FwdTli<T, V, kTliTile / 8, 8, false, 2>::launch; k.fwd_name[n] = "tli_v4x2"; k.fwd_need[n++] = 1;
         k.fwd[n] = FwdTli<T, V, kTliTile / 8, 8, false, 3>::launch; k.fwd_name[n] = "tli_v4x3"; k.fwd_need[n++] = 1;
         k.fwd[n] = FwdTli<T, V, kTliTile / 8, 8, false, 2, 8>::launch; k.fwd_name[n] = "tli_v4x2_min8";
-        k.fwd_need[n++] = 1;
+        k.fwd_untimed[n] = 1; k.fwd_need[n++] = 1;
         k.fwd[n] = FwdTli<T, V, kTliTile / 8, 8, false, 3, 6>::launch; k.fwd_name[n] = "tli_v4x3_min6";
-        k.fwd_need[n++] = 1;
+        k.fwd_untimed[n] = 1; k.fwd_need[n++] = 1;
         // the same forms with the block's tile stream bulk-prefetched into L2 at its start
         k.fwd[n] = FwdTli<T, V, kTliTile / 8, 8, false, 3, 1, true>::launch; k.fwd_name[n] = "tli_v4x3_l2pf";
         k.fwd_need[n++] = 1;
         k.fwd[n] = FwdTli<T, V, kTliTile / 8, 8, false, 2, 8, true>::launch; k.fwd_name[n] = "tli_v4x2_min8_l2pf";
-        k.fwd_need[n++] = 1;
+        k.fwd_untimed[n] = 1; k.fwd_need[n++] = 1;
         k.fwd[n] = FwdTli<T, V, kTliTile / 8, 8, false, 3, 6, true>::launch; k.fwd_name[n] = "tli_v4x3_min6_l2pf";
         k.fwd_need[n++] = 1;
         k.fwd[n] = FwdTma<T, V, 3, 16>::launch;  k.fwd_name[n] = "tma_ns3_w16"; k.fwd_need[n++] = 3;
         k.fwd[n] = FwdTma<T, V, 3, 8>::launch;   k.fwd_name[n] = "tma_ns3_w8"; k.fwd_need[n++] = 3;
         k.fwd[n] = FwdTma<T, V, 4, 16>::launch;  k.fwd_name[n] = "tma_ns4_w16"; k.fwd_need[n++] = 4;
+        if constexpr (sizeof(T) == 4) {
+            k.fwd[n] = RowsStack<V, true>::forward; k.fwd_name[n] = "stack_v4"; k.fwd_need[n++] = 2;
+        }
         k.n_fwd = n;
         n = 0;
         k.back[n] = Back<T, V, 8, 8, false, 8>::launch;  k.back_name[n++] = "cols8_u8_min8";
@@ -471,9 +543,9 @@ struct Impl {
         k.back[n] = BackTli<T, V, kTliTile / 8, 8, false, 2>::launch; k.back_name[n] = "tli_v4x2"; k.back_need[n++] = 1;
         k.back[n] = BackTli<T, V, kTliTile / 8, 8, false, 3>::launch; k.back_name[n] = "tli_v4x3"; k.back_need[n++] = 1;
         k.back[n] = BackTli<T, V, kTliTile / 8, 8, false, 0, 6>::launch; k.back_name[n] = "tli_u8_min6";
-        k.back_need[n++] = 1;
+        k.back_untimed[n] = 1; k.back_need[n++] = 1;
         k.back[n] = BackTli<T, V, kTliTile / 8, 8, false, 2, 6>::launch; k.back_name[n] = "tli_v4x2_min6";
-        k.back_need[n++] = 1;
+        k.back_untimed[n] = 1; k.back_need[n++] = 1;
         k.back[n] = BackTli<T, V, kTliTile / 8, 8, false, 2, 6, true>::launch; k.back_name[n] = "tli_v4x2_min6_l2pf";
         k.back_need[n++] = 1;
         k.back[n] = BackTli<T, V, kTliTile / 8, 8, false, 2, 1, true>::launch; k.back_name[n] = "tli_v4x2_l2pf";
@@ -483,6 +555,9 @@ struct Impl {
         k.back[n] = BackTma<T, V, 3, 16>::launch;  k.back_name[n] = "tma_ns3_w16"; k.back_need[n++] = 3;
         k.back[n] = BackTma<T, V, 3, 8>::launch;   k.back_name[n] = "tma_ns3_w8"; k.back_need[n++] = 3;
         k.back[n] = BackTma<T, V, 4, 16>::launch;  k.back_name[n] = "tma_ns4_w16"; k.back_need[n++] = 4;
+        if constexpr (sizeof(T) == 4) {
+            k.back[n] = back_stack; k.back_name[n] = "stack_v4"; k.back_need[n++] = 2;
+        }
         k.n_back = n;
         // index = 4 * (register cap) + 2 * (forward 4-wide) + (back 4-wide)
         k.n_pers = 8;
@@ -499,24 +574,24 @@ struct Impl {
         k.scatter[n] = Scatter<T, V, kTliTile / 8, 8, false, true, 4>::launch;
         k.scatter_name[n] = "tli_u8_atomic_keep"; k.scatter_bufs[n++] = 2;
         k.scatter[n] = Scatter<T, V, kTliTile / 8, 8, true, true, 4>::launch;
-        k.scatter_name[n] = "tli_u8_private_keep"; k.scatter_bufs[n++] = 9;
+        k.scatter_name[n] = "tli_u8_private_keep"; k.scatter_untimed[n] = 1; k.scatter_bufs[n++] = 9;
         k.scatter[n] = ScatterV4<T, V, kTliTile / 8, 3, true, 4>::launch;
-        k.scatter_name[n] = "tli_v4x3_private_min4"; k.scatter_bufs[n++] = 9;
+        k.scatter_name[n] = "tli_v4x3_private_min4"; k.scatter_untimed[n] = 1; k.scatter_bufs[n++] = 9;
         k.scatter[n] = ScatterV4<T, V, kTliTile / 8, 2, true, 5>::launch;
-        k.scatter_name[n] = "tli_v4x2_private_min5"; k.scatter_bufs[n++] = 9;
+        k.scatter_name[n] = "tli_v4x2_private_min5"; k.scatter_untimed[n] = 1; k.scatter_bufs[n++] = 9;
         k.scatter[n] = ScatterV4<T, V, kTliTile / 8, 2, true, 5, true>::launch;
-        k.scatter_name[n] = "tli_v4x2_private_min5_l2pf"; k.scatter_bufs[n++] = 9;
+        k.scatter_name[n] = "tli_v4x2_private_min5_l2pf"; k.scatter_untimed[n] = 1; k.scatter_bufs[n++] = 9;
         k.scatter[n] = ScatterSp<T, V, 3, 3, true>::launch;
-        k.scatter_name[n] = "sp_v4x3_min3_l2pf"; k.scatter_sp[n] = 1; k.scatter_bufs[n++] = 9;
+        k.scatter_name[n] = "sp_v4x3_min3_l2pf"; k.scatter_sp[n] = 1; k.scatter_untimed[n] = 1; k.scatter_bufs[n++] = 9;
         // one block-shared accumulator (2 staging-sized buffers): the form that still fits when the
         // per-warp accumulators do not (large staging, FP64)
         k.scatter[n] = ScatterSp<T, V, 2, 4, false, false>::launch;
         k.scatter_name[n] = "sp_v4x2_atomic_min4"; k.scatter_sp[n] = 1; k.scatter_bufs[n++] = 2;
         // no register prefetch (the L2 prefetch hides the stream's latency): fewer registers, more warps
         k.scatter[n] = ScatterSp<T, V, 2, 5, true, true, false>::launch;
-        k.scatter_name[n] = "sp_v4x2_nopf_min5_l2pf"; k.scatter_sp[n] = 1; k.scatter_bufs[n++] = 9;
+        k.scatter_name[n] = "sp_v4x2_nopf_min5_l2pf"; k.scatter_sp[n] = 1; k.scatter_untimed[n] = 1; k.scatter_bufs[n++] = 9;
         k.scatter[n] = ScatterSp<T, V, 3, 4, true, true, false>::launch;
-        k.scatter_name[n] = "sp_v4x3_nopf_min4_l2pf"; k.scatter_sp[n] = 1; k.scatter_bufs[n++] = 9;
+        k.scatter_name[n] = "sp_v4x3_nopf_min4_l2pf"; k.scatter_sp[n] = 1; k.scatter_untimed[n] = 1; k.scatter_bufs[n++] = 9;
         // each chunk's accumulator reads ahead of its writes; no zero-fill past a row's end
         k.scatter[n] = ScatterSp<T, V, 2, 5, true, true, false, kSpBatch4 | kSpLean>::launch;
         k.scatter_name[n] = "sp_v4x2_batch_min5_l2pf"; k.scatter_sp[n] = 1; k.scatter_bufs[n++] = 9;
@@ -524,6 +599,10 @@ struct Impl {
         k.scatter_name[n] = "sp_v4x2_batch_min4_l2pf"; k.scatter_sp[n] = 1; k.scatter_bufs[n++] = 9;
         k.scatter[n] = ScatterSp<T, V, 3, 4, true, true, false, kSpBatch4 | kSpLean>::launch;
         k.scatter_name[n] = "sp_v4x3_batch_min4_l2pf"; k.scatter_sp[n] = 1; k.scatter_bufs[n++] = 9;
+        if constexpr (sizeof(T) == 4) {
+            k.scatter[n] = RowsStack<V, false>::scatter;
+            k.scatter_name[n] = "stack"; k.scatter_sp[n] = 2; k.scatter_bufs[n++] = 0;
+        }
         k.n_scatter = n;
         k.fupdate = fupdate;
         k.backproject = backproject;
