@@ -2,13 +2,23 @@
 // trained and run with hand-written kernels. BF16 weights, FP32 activations,
 // FP32 accumulation; FP32 master weights updated by Adam.
 //
-// Convolutions are 3x3, stride 1, zero padding, computed as implicit GEMMs on
-// the CUDA cores: a block owns 32 output channels x an 8 x 16 pixel tile of
-// one sample, stages 16 input channels (with halo) and their weights in shared
-// memory per step, and each thread accumulates 4 channels x 4 pixels. The
-// data gradient is the same kernel on the flipped, channel-transposed weights;
-// the weight gradient accumulates 16 x 16 (output, input) channel pairs over
-// pixel tiles and adds its partial into the gradient buffer atomically.
+// Convolutions are 3x3, stride 1, zero padding, as implicit GEMMs. Three forms:
+//   k_conv       inference, on the tensor cores with the precision of FP32
+//                arithmetic: the weights are BF16 already, an FP32 activation is
+//                the exact sum of three BF16 terms, every product is exact, and
+//                only one 16-wide step of one kernel offset is summed inside the
+//                matrix unit, from zero; the steps are added up in FP32
+//                registers, rounded to nearest (chained in the unit, whose adds
+//                truncate, 144 steps are off by 2e-6 to 6e-6; this way by 2e-7,
+//                a serial FP32 multiply-add chain by 3e-7 to 6e-7)
+//   k_conv_fma   the training step's forward pass and data gradients, FP32
+//                multiply-adds in one fixed order per output: a training step
+//                has ReLU masks and sign-like Adam updates behind it, so a
+//                rounding that differs anywhere in the forward pass is a
+//                different step (tried on the tensor cores: errors as above,
+//                0.6 ms instead of 1.2 for the protocol's step of 8 samples, but
+//                one seed in three steps to another side of some ReLU)
+//   k_conv_wgrad the training step's weight gradients, the same way
 #include <cuda_bf16.h>
 #include <cuda_runtime.h>
 #include <math.h>
@@ -23,8 +33,6 @@
 namespace {
 
 constexpr int kT = 256;
-constexpr int TC = 32, TH = 8, TW = 16, CK = 16;  // forward tile: channels, rows, columns, input chunk
-constexpr int WC = 16, WI = 16;                    // weight-gradient tile: output x input channels
 
 int blocks_for(int64_t n)
 {
@@ -33,226 +41,572 @@ int blocks_for(int64_t n)
     return int(b < 1 ? 1 : b);
 }
 
-template <bool RELU>
-__global__ void __launch_bounds__(256)
-k_conv_fwd(const float *__restrict__ x, const __nv_bfloat16 *__restrict__ w, const float *__restrict__ b,
-           float *__restrict__ y, int Ci, int Co, int H, int W)
+// d = a * b + c on the tensor cores: a 16 x 16 (rows: output channels, columns:
+// input channels), b 16 x 8 (columns: pixels), BF16 operands, FP32 sums.
+__device__ __forceinline__ void mma16816(float (&d)[4], const uint4 &a, const uint2 &b, const float (&c)[4])
 {
-    __shared__ float xs[CK][TH + 2][TW + 3];
-    __shared__ float ws[TC][CK * 9 + 1];
-    const int tiles_w = (W + TW - 1) / TW;
-    const int th0 = (blockIdx.x / tiles_w) * TH, tw0 = (blockIdx.x % tiles_w) * TW;
-    const int co0 = blockIdx.y * TC;
-    const int n = blockIdx.z;
-    const int t = threadIdx.x;
-    const int cg = t >> 5;  // warp: 4 output channels
-    const int pg = t & 31;  // lane: 4 consecutive pixels of one row
-    const int py = (pg * 4) / TW, px = (pg * 4) % TW;
-    float acc[4][4];
-#pragma unroll
-    for (int o = 0; o < 4; o++)
-#pragma unroll
-        for (int p = 0; p < 4; p++) acc[o][p] = 0.f;
-    const float *xn = x + size_t(n) * Ci * H * W;
-    for (int ci0 = 0; ci0 < Ci; ci0 += CK) {
-        for (int k = t; k < CK * (TH + 2) * (TW + 2); k += blockDim.x) {
-            const int c = k / ((TH + 2) * (TW + 2)), r = k % ((TH + 2) * (TW + 2));
-            const int yy = r / (TW + 2), xx = r % (TW + 2);
-            const int gy = th0 + yy - 1, gx = tw0 + xx - 1, gc = ci0 + c;
-            float v = 0.f;
-            if (gc < Ci && gy >= 0 && gy < H && gx >= 0 && gx < W) v = xn[(size_t(gc) * H + gy) * W + gx];
-            xs[c][yy][xx] = v;
-        }
-        for (int k = t; k < TC * CK * 9; k += blockDim.x) {
-            const int co = k / (CK * 9), r = k % (CK * 9);
-            const int c = r / 9, kk = r % 9;
-            const int gco = co0 + co, gc = ci0 + c;
-            float v = 0.f;
-            if (gco < Co && gc < Ci) v = __bfloat162float(w[(size_t(gco) * Ci + gc) * 9 + kk]);
-            ws[co][r] = v;
-        }
-        __syncthreads();
-        const int cmax = Ci - ci0 < CK ? Ci - ci0 : CK;
-        for (int c = 0; c < cmax; c++) {
-#pragma unroll
-            for (int kh = 0; kh < 3; kh++) {
-                float xv[6];
-#pragma unroll
-                for (int q = 0; q < 6; q++) xv[q] = xs[c][py + kh][px + q];
-#pragma unroll
-                for (int kw = 0; kw < 3; kw++)
-#pragma unroll
-                    for (int o = 0; o < 4; o++) {
-                        const float wv = ws[cg * 4 + o][c * 9 + kh * 3 + kw];
-#pragma unroll
-                        for (int p = 0; p < 4; p++) acc[o][p] = fmaf(wv, xv[p + kw], acc[o][p]);
-                    }
-            }
-        }
-        __syncthreads();
+    asm("mma.sync.aligned.m16n8k16.row.col.f32.bf16.bf16.f32 {%0, %1, %2, %3}, {%4, %5, %6, %7}, {%8, %9}, "
+        "{%10, %11, %12, %13};"
+        : "=f"(d[0]), "=f"(d[1]), "=f"(d[2]), "=f"(d[3])
+        : "r"(a.x), "r"(a.y), "r"(a.z), "r"(a.w), "r"(b.x), "r"(b.y), "f"(c[0]), "f"(c[1]), "f"(c[2]), "f"(c[3]));
+}
+
+// (x, y) = t[0] + t[1] + t[2] exactly, each word a pair of BF16 numbers (x below):
+// the leading 8 bits rounded to nearest, those of the rest, and the rest of
+// that. What would round to infinity is cut instead; an infinity or NaN is all
+// in t[0].
+__device__ __forceinline__ void split_pair(float x, float y, uint32_t (&t)[3])
+{
+    const __nv_bfloat162 h = __floats2bfloat162_rn(x, y);
+    t[0] = *reinterpret_cast<const uint32_t *>(&h);
+    float rx = x - __uint_as_float(t[0] << 16), ry = y - __uint_as_float(t[0] & 0xFFFF0000u);
+    if ((t[0] & 0x7F80u) == 0x7F80u || (t[0] & 0x7F800000u) == 0x7F800000u) {
+        const bool fx = isfinite(x), fy = isfinite(y);
+        const uint32_t cx = fx ? __float_as_uint(x) >> 16 : t[0] & 0xFFFFu;
+        const uint32_t cy = fy ? __float_as_uint(y) & 0xFFFF0000u : t[0] & 0xFFFF0000u;
+        t[0] = cx | cy;
+        rx = fx ? x - __uint_as_float(cx << 16) : 0.f;
+        ry = fy ? y - __uint_as_float(cy) : 0.f;
     }
+    const __nv_bfloat162 m = __floats2bfloat162_rn(rx, ry);
+    t[1] = *reinterpret_cast<const uint32_t *>(&m);
+    const __nv_bfloat162 l =
+        __floats2bfloat162_rn(rx - __uint_as_float(t[1] << 16), ry - __uint_as_float(t[1] & 0xFFFF0000u));
+    t[2] = *reinterpret_cast<const uint32_t *>(&l);
+}
+
+// Forward convolution. A block makes 16 MT output channels of a tile of RG NT / 2 rows x
+// 16 columns of one sample: warp (m, g) 16 channels of NT / 2 rows (MT x RG
+// warps, NT runs of 8 pixels each). Per step of 16 input channels the block
+// stages the tile with its halo as three BF16 terms, [pixel][channel], while
+// the next step's values are on their way, and each warp goes through the nine
+// offsets. Weights come from global memory (L2) in fragment order, one 16-byte
+// load a lane and offset, one row of offsets ahead. The activations of a
+// pixel's 16 channels are 32 bytes in the order that a lane's two words (pairs
+// k and k + 8) lie side by side; stores and fragment loads are both contiguous
+// over the lanes.
+template <int MT, int RG, int NT, bool RELU>
+__global__ void __launch_bounds__(32 * MT * RG, 16 / (MT * RG))  // 128 registers
+k_conv(const float *__restrict__ x, const uint4 *__restrict__ wf, const float *__restrict__ b,
+       float *__restrict__ y, int Ci, int Co, int H, int W)
+{
+    constexpr int kThreads = 32 * MT * RG, kRows = RG * NT / 2, kPW = 18, kPix = (kRows + 2) * kPW;
+    constexpr int kItems = (4 * kPix + kThreads - 1) / kThreads;  // 4 channels of a pixel each
+    __shared__ uint2 xs[3][kItems * kThreads];
+    const int tiles_w = (W + 15) / 16;
+    const int h0 = int(blockIdx.x) / tiles_w * kRows, w0 = int(blockIdx.x) % tiles_w * 16;
+    const int n = blockIdx.z, lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const int mt = warp % MT, rg = warp / MT;
+    const int nci = (Ci + 15) / 16, co16 = int(blockIdx.y) * MT + mt;
+    const bool live = co16 * 16 < Co;
+    const int HW = H * W;
+    const float *xn = x + size_t(n) * Ci * HW;
+    // this thread's staging items: channels 2 cp, + 1, + 8, + 9 of the pixels (k kThreads + thread) / 4
+    const int cp = threadIdx.x & 3;
+    int off[kItems];  // the pixel's offset, -1 outside the image (or past the tile)
 #pragma unroll
-    for (int o = 0; o < 4; o++) {
-        const int co = co0 + cg * 4 + o;
-        const int hh = th0 + py;
-        if (co >= Co || hh >= H) continue;
+    for (int k = 0; k < kItems; k++) {
+        const int p = (k * kThreads + int(threadIdx.x)) >> 2;
+        const int gy = h0 + p / kPW - 1, gx = w0 + p % kPW - 1;
+        off[k] = (p < kPix && gy >= 0 && gy < H && gx >= 0 && gx < W) ? gy * W + gx : -1;
+    }
+    float v[kItems][4];
+    auto fetch = [&](int c0) {
+#pragma unroll
+        for (int q = 0; q < 4; q++) {
+            const int c = c0 + 2 * cp + (q & 1) + 8 * (q >> 1);
+            const float *xc = xn + size_t(c) * HW;
+#pragma unroll
+            for (int k = 0; k < kItems; k++) v[k][q] = (off[k] >= 0 && c < Ci) ? __ldg(xc + off[k]) : 0.f;
+        }
+    };
+    fetch(0);
+    float acc[NT][4];
+#pragma unroll
+    for (int t = 0; t < NT; t++)
+#pragma unroll
+        for (int q = 0; q < 4; q++) acc[t][q] = 0.f;
+    const uint4 *wp = wf + (size_t(live ? co16 : 0) * nci * 9) * 32 + lane;
+    uint4 a[3], an[3];
+#pragma unroll
+    for (int k = 0; k < 3; k++) an[k] = __ldg(wp + k * 32);
+    const int il = (rg * (NT / 2) * kPW + (lane >> 2)) * 4 + (lane & 3);  // this lane's words of its first pixel
+#pragma unroll 1
+    for (int c = 0; c < nci; c++) {
+        if (c > 0) __syncthreads();
+#pragma unroll
+        for (int k = 0; k < kItems; k++) {
+            uint32_t t0[3], t1[3];
+            split_pair(v[k][0], v[k][1], t0);
+            split_pair(v[k][2], v[k][3], t1);
+#pragma unroll
+            for (int m = 0; m < 3; m++) xs[m][k * kThreads + threadIdx.x] = make_uint2(t0[m], t1[m]);
+        }
+        __syncthreads();
+        if (c + 1 < nci) fetch((c + 1) * 16);
+#pragma unroll 1
+        for (int kh = 0; kh < 3; kh++) {
+#pragma unroll
+            for (int k = 0; k < 3; k++) a[k] = an[k];
+            wp += 3 * 32;
+            if (c * 3 + kh + 1 < nci * 3) {
+#pragma unroll
+                for (int k = 0; k < 3; k++) an[k] = __ldg(wp + k * 32);
+            }
+            const int ik = il + kh * kPW * 4;
+#pragma unroll
+            for (int kw = 0; kw < 3; kw++)
+#pragma unroll
+                for (int t = 0; t < NT; t++) {
+                    const int i = ik + ((t / 2) * kPW + (t % 2) * 8 + kw) * 4;
+                    // the small terms in one sum, the large one (16-bit products: hardly a bit is cut
+                    // inside the unit) in another
+                    float d[4] = {0.f, 0.f, 0.f, 0.f}, z[4] = {0.f, 0.f, 0.f, 0.f};
+                    mma16816(d, a[kw], xs[2][i], d);
+                    mma16816(d, a[kw], xs[1][i], d);
+                    mma16816(z, a[kw], xs[0][i], z);
+#pragma unroll
+                    for (int q = 0; q < 4; q++) acc[t][q] = (acc[t][q] + d[q]) + z[q];
+                }
+        }
+    }
+    if (!live) return;
+    const bool even = (W & 1) == 0;  // else (the quarter-size images of some widths) a pair is not 8-byte aligned
+#pragma unroll
+    for (int hf = 0; hf < 2; hf++) {
+        const int co = co16 * 16 + (lane >> 2) + 8 * hf;
+        if (co >= Co) continue;
         const float bias = b ? b[co] : 0.f;
 #pragma unroll
-        for (int p = 0; p < 4; p++) {
-            const int ww = tw0 + px + p;
-            if (ww >= W) continue;
-            float v = acc[o][p] + bias;
-            if (RELU) v = v > 0.f ? v : 0.f;
-            y[((size_t(n) * Co + co) * H + hh) * W + ww] = v;
+        for (int t = 0; t < NT; t++) {
+            const int hh = h0 + rg * (NT / 2) + t / 2, ww = w0 + (t % 2) * 8 + (lane & 3) * 2;
+            if (hh >= H || ww >= W) continue;
+            const size_t o = (size_t(n) * Co + co) * HW + hh * W + ww;
+            float r0 = acc[t][2 * hf] + bias, r1 = acc[t][2 * hf + 1] + bias;
+            if (RELU) {
+                r0 = r0 > 0.f ? r0 : 0.f;
+                r1 = r1 > 0.f ? r1 : 0.f;
+            }
+            if (even) {
+                *reinterpret_cast<float2 *>(y + o) = make_float2(r0, r1);
+            } else {
+                y[o] = r0;
+                if (ww + 1 < W) y[o + 1] = r1;
+            }
         }
     }
 }
 
-// dw[co][ci][k] += sum over the block's pixels of dy[n][co][h][w] x[n][ci][h+kh-1][w+kw-1];
-// db[co] += sum of dy (blocks of the first input-channel tile only).
-__global__ void __launch_bounds__(256)
-k_conv_bwd_w(const float *__restrict__ x, const float *__restrict__ dy, float *__restrict__ dw,
+// The same convolution in FP32 multiply-adds: every output adds its products in
+// the order of the input channels, then the kernel's rows, then its columns. A
+// warp makes 8 output channels (their weights are one broadcast load for the
+// warp) of a tile of 8 G rows x 16 columns: a lane 4 G pixels of a row, 32 G
+// accumulators. Bound: the FP32 pipes (one operand load per 12 to 19
+// multiply-adds). Per step of 8 input channels the block stages the tile with
+// its halo and the step's weights, [ci][offset][co], by asynchronous copies into
+// one of two buffers while it works from the other.
+constexpr int kFmaCi = 8, kFmaPitch = 20;  // pitch: 8 rows of a quarter-warp's 16-byte loads fall in distinct banks
+
+template <int G, int WARPS>
+constexpr int kFmaStage = kFmaCi * (8 * G + 2) * kFmaPitch + kFmaCi * 9 * 8 * WARPS;  // floats
+
+__device__ __forceinline__ void copy4(float *dst, const float *src, bool valid)  // valid = false: zero, no read
+{
+    asm volatile("cp.async.ca.shared.global [%0], [%1], 4, %2;" ::"r"(uint32_t(__cvta_generic_to_shared(dst))),
+                 "l"(src), "r"(valid ? 4 : 0) : "memory");
+}
+__device__ __forceinline__ void copy16(float *dst, const float *src)
+{
+    asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(uint32_t(__cvta_generic_to_shared(dst))), "l"(src)
+                 : "memory");
+}
+
+template <int G, int WARPS, bool RELU, bool MASK>
+__global__ void __launch_bounds__(32 * WARPS, G == 2 ? 16 / WARPS : 20 / WARPS)
+k_conv_fma(const float *__restrict__ x, const float *__restrict__ wq, const float *__restrict__ b,
+           const float *__restrict__ mask, float *__restrict__ y, int Ci, int Co, int H, int W)
+{
+    constexpr int kThreads = 32 * WARPS, kRows = 8 * G, kCo = 8 * WARPS, kPix = (kRows + 2) * 18;
+    constexpr int kPlane = (kRows + 2) * kFmaPitch, kStage = kFmaStage<G, WARPS>;
+    constexpr int kItems = (kPix + kThreads - 1) / kThreads;
+    extern __shared__ __align__(16) float smf[];  // two stages: x [ci][row][20], then weights [ci 9 + offset][co]
+    const int tiles_w = (W + 15) / 16;
+    const int h0 = int(blockIdx.x) / tiles_w * kRows, w0 = int(blockIdx.x) % tiles_w * 16;
+    const int n = blockIdx.z, lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const int co0 = int(blockIdx.y) * kCo;
+    const int row = lane & (kRows - 1), c4 = lane / kRows * 4;  // first pixel; G = 2: and the one 8 columns on
+    const int HW = H * W;
+    const float *xn = x + size_t(n) * Ci * HW;
+    const int cop = (Co + 63) / 64 * 64;  // weights: output channels padded to 64
+    int off[kItems], dst[kItems];         // this thread's pixels of a channel: offset (-1: outside), place
+#pragma unroll
+    for (int k = 0; k < kItems; k++) {
+        const int p = k * kThreads + int(threadIdx.x);
+        const int yy = p / 18, xx = p % 18, gy = h0 + yy - 1, gx = w0 + xx - 1;
+        off[k] = (gy >= 0 && gy < H && gx >= 0 && gx < W) ? gy * W + gx : -1;
+        dst[k] = p < kPix ? yy * kFmaPitch + xx : -1;
+    }
+    auto stage = [&](int c0, float *to) {
+        const int nc = Ci - c0 < kFmaCi ? Ci - c0 : kFmaCi;
+        for (int c = 0; c < nc; c++) {
+            const float *xc = xn + size_t(c0 + c) * HW;
+#pragma unroll
+            for (int k = 0; k < kItems; k++)
+                if (dst[k] >= 0) copy4(to + c * kPlane + dst[k], off[k] >= 0 ? xc + off[k] : xc, off[k] >= 0);
+        }
+        const float *wc = wq + size_t(c0) * 9 * cop + co0;
+        float *tw = to + kFmaCi * kPlane;
+        for (int k = threadIdx.x; k < nc * 9 * (kCo / 4); k += kThreads)
+            copy16(tw + 4 * k, wc + size_t(k / (kCo / 4)) * cop + k % (kCo / 4) * 4);
+        asm volatile("cp.async.commit_group;" ::: "memory");
+    };
+    float acc[G][8][4];
+#pragma unroll
+    for (int g = 0; g < G; g++)
+#pragma unroll
+        for (int o = 0; o < 8; o++)
+#pragma unroll
+            for (int q = 0; q < 4; q++) acc[g][o][q] = 0.f;
+    stage(0, smf);
+    int buf = 0;
+#pragma unroll 1
+    for (int c0 = 0; c0 < Ci; c0 += kFmaCi) {
+        if (c0 + kFmaCi < Ci) {
+            stage(c0 + kFmaCi, smf + (buf ^ 1) * kStage);
+            asm volatile("cp.async.wait_group 1;" ::: "memory");
+        } else {
+            asm volatile("cp.async.wait_group 0;" ::: "memory");
+        }
+        __syncthreads();
+        const float *xb = smf + buf * kStage + row * kFmaPitch + c4;
+        const float *wb = smf + buf * kStage + kFmaCi * kPlane + 8 * warp;
+        const int nc = Ci - c0 < kFmaCi ? Ci - c0 : kFmaCi;
+#pragma unroll 1
+        for (int c = 0; c < nc; c++) {
+#pragma unroll
+            for (int kh = 0; kh < 3; kh++) {
+                float xv[G][6];
+#pragma unroll
+                for (int g = 0; g < G; g++) {
+                    const float *p = xb + c * kPlane + kh * kFmaPitch + 8 * g;
+                    const float4 v = *reinterpret_cast<const float4 *>(p);
+                    const float2 u = *reinterpret_cast<const float2 *>(p + 4);
+                    xv[g][0] = v.x; xv[g][1] = v.y; xv[g][2] = v.z; xv[g][3] = v.w;
+                    xv[g][4] = u.x; xv[g][5] = u.y;
+                }
+#pragma unroll
+                for (int kw = 0; kw < 3; kw++) {
+                    const float *p = wb + (c * 9 + kh * 3 + kw) * kCo;
+                    const float4 wa = *reinterpret_cast<const float4 *>(p), wd = *reinterpret_cast<const float4 *>(p + 4);
+                    const float wv[8] = {wa.x, wa.y, wa.z, wa.w, wd.x, wd.y, wd.z, wd.w};
+#pragma unroll
+                    for (int g = 0; g < G; g++)
+#pragma unroll
+                        for (int o = 0; o < 8; o++)
+#pragma unroll
+                            for (int q = 0; q < 4; q++) acc[g][o][q] = fmaf(wv[o], xv[g][q + kw], acc[g][o][q]);
+                }
+            }
+        }
+        __syncthreads();  // the next copies go over this buffer
+        buf ^= 1;
+    }
+    const int hh = h0 + row;
+    if (hh >= H) return;
+#pragma unroll
+    for (int o = 0; o < 8; o++) {
+        const int co = co0 + 8 * warp + o;
+        if (co >= Co) break;
+        const float bias = b ? b[co] : 0.f;
+#pragma unroll
+        for (int g = 0; g < G; g++) {
+            const int ww = w0 + c4 + 8 * g;
+            const size_t at = (size_t(n) * Co + co) * HW + hh * W + ww;
+            if ((W & 3) == 0) {  // a lane's four pixels are one aligned word
+                if (ww >= W) continue;
+                float r[4];
+#pragma unroll
+                for (int q = 0; q < 4; q++) {
+                    r[q] = acc[g][o][q] + bias;
+                    if (RELU) r[q] = r[q] > 0.f ? r[q] : 0.f;
+                }
+                if (MASK) {
+                    const float4 m = *reinterpret_cast<const float4 *>(mask + at);
+                    r[0] = m.x > 0.f ? r[0] : 0.f;
+                    r[1] = m.y > 0.f ? r[1] : 0.f;
+                    r[2] = m.z > 0.f ? r[2] : 0.f;
+                    r[3] = m.w > 0.f ? r[3] : 0.f;
+                }
+                *reinterpret_cast<float4 *>(y + at) = make_float4(r[0], r[1], r[2], r[3]);
+                continue;
+            }
+#pragma unroll
+            for (int q = 0; q < 4; q++) {
+                if (ww + q >= W) break;
+                float r = acc[g][o][q] + bias;
+                if (RELU) r = r > 0.f ? r : 0.f;
+                if (MASK) r = mask[at + q] > 0.f ? r : 0.f;
+                y[at + q] = r;
+            }
+        }
+    }
+}
+
+// Weight gradient: dw[co][ci][kh][kw] += sum over the block's pixels of
+// dy[n][co][h][w] x[n][ci][h + kh - 1][w + kw - 1]; db[co] += sum of dy (blocks
+// of the first input channels only). A block makes 64 output x 16 input
+// channels x 9 offsets of a band of 8 rows of one sample, 16 columns at a time,
+// and adds its sums to dw; a thread 2 x 4 x 9 of them, each one chain of FP32
+// multiply-adds over the band's pixels, column tile by column tile, row by row.
+// Both operands are staged with the channels innermost, so that a pixel costs a
+// thread one 8-byte and at most nine 16-byte loads, mostly broadcasts, for 72
+// multiply-adds. Bound: the FP32 pipes.
+constexpr int kWgRows = 8, kWgCo = 64, kWgCi = 16, kWgPitchX = kWgCi + 4, kWgPitchD = kWgCo + 4;
+constexpr int kWgSmem = 4 * ((kWgRows + 2) * 18 * kWgPitchX + kWgRows * 16 * kWgPitchD);
+
+__global__ void __launch_bounds__(128, 4)
+k_conv_wgrad(const float *__restrict__ x, const float *__restrict__ dy, float *__restrict__ dw,
              float *__restrict__ db, int Ci, int Co, int H, int W)
 {
-    __shared__ float dys[WC][TH * TW + 1];
-    __shared__ float xs[WI][(TH + 2) * (TW + 2) + 1];
-    const int co0 = blockIdx.x * WC, ci0 = blockIdx.y * WI;
-    const int tiles_h = (H + TH - 1) / TH;
-    const int n = blockIdx.z / tiles_h;
-    const int th0 = (blockIdx.z % tiles_h) * TH;
-    const int t = threadIdx.x;
-    const int col = t / WI, cil = t % WI;
-    float acc[9];
+    extern __shared__ __align__(16) float smw[];
+    float *const xs = smw, *const ds = smw + (kWgRows + 2) * 18 * kWgPitchX;  // [pixel with halo][ci], [pixel][co]
+    const int co0 = blockIdx.x * kWgCo, ci0 = blockIdx.y * kWgCi;
+    const int bands = (H + kWgRows - 1) / kWgRows;
+    const int n = int(blockIdx.z) / bands, h0 = int(blockIdx.z) % bands * kWgRows;
+    const int cq = threadIdx.x & 3, cp = threadIdx.x >> 2;  // input channels 4 cq .. + 3, output channels 2 cp, + 1
+    const int HW = H * W;
+    const float *xn = x + (size_t(n) * Ci + ci0) * HW, *dn = dy + (size_t(n) * Co + co0) * HW;
+    float acc[2][4][9];
 #pragma unroll
-    for (int k = 0; k < 9; k++) acc[k] = 0.f;
-    float dbacc = 0.f;
-    for (int tw0 = 0; tw0 < W; tw0 += TW) {
-        for (int k = t; k < WC * TH * TW; k += blockDim.x) {
-            const int c = k / (TH * TW), r = k % (TH * TW);
-            const int hh = th0 + r / TW, ww = tw0 + r % TW, gc = co0 + c;
-            float v = 0.f;
-            if (gc < Co && hh < H && ww < W) v = dy[((size_t(n) * Co + gc) * H + hh) * W + ww];
-            dys[c][r] = v;
+    for (int o = 0; o < 2; o++)
+#pragma unroll
+        for (int i = 0; i < 4; i++)
+#pragma unroll
+            for (int k = 0; k < 9; k++) acc[o][i][k] = 0.f;
+    float db0 = 0.f, db1 = 0.f;
+#pragma unroll 1
+    for (int w0 = 0; w0 < W; w0 += 16) {
+        __syncthreads();  // the last tile has been read
+        for (int k = threadIdx.x; k < (kWgRows + 2) * 18 * (kWgCi / 4); k += 128) {
+            const int q = k / ((kWgRows + 2) * 18), p = k % ((kWgRows + 2) * 18);
+            const int gy = h0 + p / 18 - 1, gx = w0 + p % 18 - 1;
+            const bool in = gy >= 0 && gy < H && gx >= 0 && gx < W;
+            float v[4];
+#pragma unroll
+            for (int m = 0; m < 4; m++)
+                v[m] = (in && ci0 + 4 * q + m < Ci) ? __ldg(xn + size_t(4 * q + m) * HW + gy * W + gx) : 0.f;
+            *reinterpret_cast<float4 *>(xs + p * kWgPitchX + 4 * q) = make_float4(v[0], v[1], v[2], v[3]);
         }
-        for (int k = t; k < WI * (TH + 2) * (TW + 2); k += blockDim.x) {
-            const int c = k / ((TH + 2) * (TW + 2)), r = k % ((TH + 2) * (TW + 2));
-            const int gy = th0 + r / (TW + 2) - 1, gx = tw0 + r % (TW + 2) - 1, gc = ci0 + c;
-            float v = 0.f;
-            if (gc < Ci && gy >= 0 && gy < H && gx >= 0 && gx < W) v = x[((size_t(n) * Ci + gc) * H + gy) * W + gx];
-            xs[c][r] = v;
+        for (int k = threadIdx.x; k < kWgRows * 16 * (kWgCo / 4); k += 128) {
+            const int q = k / (kWgRows * 16), p = k % (kWgRows * 16);
+            const int gy = h0 + p / 16, gx = w0 + p % 16;
+            const bool in = gy < H && gx < W;
+            float v[4];
+#pragma unroll
+            for (int m = 0; m < 4; m++)
+                v[m] = (in && co0 + 4 * q + m < Co) ? __ldg(dn + size_t(4 * q + m) * HW + gy * W + gx) : 0.f;
+            *reinterpret_cast<float4 *>(ds + p * kWgPitchD + 4 * q) = make_float4(v[0], v[1], v[2], v[3]);
         }
         __syncthreads();
-        for (int p = 0; p < TH * TW; p++) {
-            const float d = dys[col][p];
-            const int py = p / TW, px = p % TW;
-            dbacc += d;
+#pragma unroll 1
+        for (int r = 0; r < kWgRows; r++)
+#pragma unroll 4
+            for (int c = 0; c < 16; c++) {
+                const float2 d = *reinterpret_cast<const float2 *>(ds + (r * 16 + c) * kWgPitchD + 2 * cp);
+                db0 += d.x;
+                db1 += d.y;
 #pragma unroll
-            for (int kh = 0; kh < 3; kh++)
-#pragma unroll
-                for (int kw = 0; kw < 3; kw++) acc[kh * 3 + kw] = fmaf(d, xs[cil][(py + kh) * (TW + 2) + px + kw], acc[kh * 3 + kw]);
-        }
-        __syncthreads();
+                for (int k = 0; k < 9; k++) {
+                    const float4 v = *reinterpret_cast<const float4 *>(
+                        xs + ((r + k / 3) * 18 + c + k % 3) * kWgPitchX + 4 * cq);
+                    acc[0][0][k] = fmaf(d.x, v.x, acc[0][0][k]);
+                    acc[0][1][k] = fmaf(d.x, v.y, acc[0][1][k]);
+                    acc[0][2][k] = fmaf(d.x, v.z, acc[0][2][k]);
+                    acc[0][3][k] = fmaf(d.x, v.w, acc[0][3][k]);
+                    acc[1][0][k] = fmaf(d.y, v.x, acc[1][0][k]);
+                    acc[1][1][k] = fmaf(d.y, v.y, acc[1][1][k]);
+                    acc[1][2][k] = fmaf(d.y, v.z, acc[1][2][k]);
+                    acc[1][3][k] = fmaf(d.y, v.w, acc[1][3][k]);
+                }
+            }
     }
-    const int co = co0 + col, ci = ci0 + cil;
-    if (co < Co && ci < Ci)
+    // through shared memory, so that a warp's adds are contiguous in dw
+    __syncthreads();
+    float *const out = smw;  // [co][ci][9]
 #pragma unroll
-        for (int k = 0; k < 9; k++) atomicAdd(&dw[(size_t(co) * Ci + ci) * 9 + k], acc[k]);
-    if (cil == 0 && blockIdx.y == 0 && co < Co) atomicAdd(&db[co], dbacc);
+    for (int o = 0; o < 2; o++)
+#pragma unroll
+        for (int i = 0; i < 4; i++)
+#pragma unroll
+            for (int k = 0; k < 9; k++) out[((2 * cp + o) * kWgCi + 4 * cq + i) * 9 + k] = acc[o][i][k];
+    __syncthreads();
+    for (int k = threadIdx.x; k < kWgCo * kWgCi * 9; k += 128) {
+        const int co = k / (kWgCi * 9), r = k % (kWgCi * 9);
+        if (co0 + co < Co && ci0 + r / 9 < Ci) atomicAdd(dw + (size_t(co0 + co) * Ci + ci0) * 9 + r, out[k]);
+    }
+    if (blockIdx.y == 0 && cq == 0) {
+        if (co0 + 2 * cp < Co) atomicAdd(db + co0 + 2 * cp, db0);
+        if (co0 + 2 * cp + 1 < Co) atomicAdd(db + co0 + 2 * cp + 1, db1);
+    }
+}
+static_assert(kWgSmem >= 4 * kWgCo * kWgCi * 9, "the sums are turned in the staging buffer");
+
+// The weights of one layer as k_conv reads them: fragment (co / 16, ci / 16,
+// offset) of 32 lanes x 4 words; lane l's words hold rows l / 4 and l / 4 + 8,
+// columns 2 (l mod 4) and + 1, then the same 8 columns on; zeros past the
+// layer's channels.
+__device__ __forceinline__ uint32_t bf16_bits(float v)
+{
+    return uint32_t(__bfloat16_as_ushort(__float2bfloat16_rn(v)));
 }
 
-// wt[ci][co][kh][kw] = w[co][ci][2-kh][2-kw]: the data gradient as a forward convolution.
-__global__ void k_flip_weights(const __nv_bfloat16 *__restrict__ w, __nv_bfloat16 *__restrict__ wt, int Ci, int Co)
+__device__ __forceinline__ uint32_t frag_word(const float *__restrict__ w, int64_t k, int Ci, int Co)
 {
-    const int64_t n = int64_t(Ci) * Co * 9;
-    for (int64_t k = int64_t(blockIdx.x) * blockDim.x + threadIdx.x; k < n; k += int64_t(gridDim.x) * blockDim.x) {
-        const int kk = int(k % 9);
-        const int64_t r = k / 9;
-        const int co = int(r % Co), ci = int(r / Co);
-        wt[k] = w[(int64_t(co) * Ci + ci) * 9 + (8 - kk)];
+    const int nc = (Ci + 15) / 16;
+    const int q = int(k & 3), l = int(k >> 2) & 31;
+    const int64_t f = k >> 7;
+    const int tap = int(f % 9), c16 = int(f / 9 % nc), r16 = int(f / 9 / nc);
+    const int r = r16 * 16 + l / 4 + 8 * (q & 1), c = c16 * 16 + 2 * (l & 3) + 8 * (q >> 1);
+    uint32_t v = 0u;
+    for (int m = 0; m < 2; m++)
+        if (r < Co && c + m < Ci) v |= bf16_bits(w[(int64_t(r) * Ci + c + m) * 9 + tap]) << (16 * m);
+    return v;
+}
+
+// As k_conv_fma reads them: [ci][offset][co, padded to 64], rounded to BF16 and
+// widened again. FLIP: of the transposed layer with the offsets reversed (the
+// data gradient as a forward convolution).
+template <bool FLIP>
+__device__ __forceinline__ uint32_t row_word(const float *__restrict__ w, int64_t k, int Ci, int Co)
+{
+    const int R = FLIP ? Ci : Co;  // output channels of the convolution
+    const int cop = (R + 63) / 64 * 64;
+    const int r = int(k % cop), tap = int(k / cop % 9), c = int(k / cop / 9);
+    if (r >= R) return 0u;
+    return bf16_bits(FLIP ? w[(int64_t(c) * Ci + r) * 9 + (8 - tap)] : w[(int64_t(r) * Ci + c) * 9 + tap]) << 16;
+}
+
+struct PackTable {
+    int ci[9], co[9];
+    int64_t w[9];           // offsets of the layers' parameters
+    int64_t at[3][10];      // words: fragments, FP32 rows, FP32 rows of the flipped layers (the last: the form's end)
+};
+
+__global__ void k_pack_weights(const float *__restrict__ w, uint32_t *__restrict__ out, PackTable t)
+{
+    for (int64_t k = int64_t(blockIdx.x) * blockDim.x + threadIdx.x; k < t.at[2][9]; k += int64_t(gridDim.x) * blockDim.x) {
+        const int form = k < t.at[0][9] ? 0 : (k < t.at[1][9] ? 1 : 2);
+        int l = 0;
+        while (l < 8 && k >= t.at[form][l + 1]) l++;
+        const int64_t r = k - t.at[form][l];
+        const float *wl = w + t.w[l];
+        out[k] = form == 0 ? frag_word(wl, r, t.ci[l], t.co[l])
+                           : (form == 1 ? row_word<false>(wl, r, t.ci[l], t.co[l]) : row_word<true>(wl, r, t.ci[l], t.co[l]));
     }
 }
 
-__global__ void k_relu_bwd(float *__restrict__ g, const float *__restrict__ a, int64_t n)
-{
-    for (int64_t k = int64_t(blockIdx.x) * blockDim.x + threadIdx.x; k < n; k += int64_t(gridDim.x) * blockDim.x)
-        if (!(a[k] > 0.f)) g[k] = 0.f;
-}
+// The elementwise kernels below go over planes (sample, channel): blockIdx.y, +
+// gridDim.y, ..., with the place inside a plane in 32 bits, so that rows and
+// columns cost one 32-bit division each.
 
-// y [NC][H/2][W/2] = 2x2 average of x [NC][H][W]; with accumulate, the backward adds into dx.
+// y [NC][H/2][W/2] = 2x2 average of x [NC][H][W].
 __global__ void k_pool_fwd(const float *__restrict__ x, float *__restrict__ y, int64_t NC, int H, int W)
 {
-    const int h2 = H / 2, w2 = W / 2;
-    const int64_t n = NC * h2 * w2;
-    for (int64_t k = int64_t(blockIdx.x) * blockDim.x + threadIdx.x; k < n; k += int64_t(gridDim.x) * blockDim.x) {
-        const int ww = int(k % w2), hh = int((k / w2) % h2);
-        const int64_t c = k / (int64_t(w2) * h2);
-        const float *p = x + (c * H + 2 * hh) * W + 2 * ww;
-        y[k] = 0.25f * (p[0] + p[1] + p[W] + p[W + 1]);
-    }
+    const unsigned w2 = unsigned(W) / 2, n = unsigned(H) / 2 * w2;
+    for (int64_t c = blockIdx.y; c < NC; c += gridDim.y)
+        for (unsigned k = blockIdx.x * blockDim.x + threadIdx.x; k < n; k += gridDim.x * blockDim.x) {
+            const unsigned hh = k / w2, ww = k - hh * w2;
+            const float *p = x + (c * H + 2 * hh) * W + 2 * ww;
+            y[c * n + k] = 0.25f * (p[0] + p[1] + p[W] + p[W + 1]);
+        }
 }
 
-__global__ void k_pool_bwd_add(const float *__restrict__ dy, float *__restrict__ dx, int64_t NC, int H, int W)
+// The pooled layer's input gradient: dx = skip + dy / 4 of the cell (skip: the
+// gradient through the skip connection), zeroed where a <= 0 (the ReLU).
+__global__ void k_pool_bwd(const float *__restrict__ dy, const float *__restrict__ skip, const float *__restrict__ a,
+                           float *__restrict__ dx, int64_t NC, int H, int W)
 {
-    const int64_t n = NC * H * W;
-    for (int64_t k = int64_t(blockIdx.x) * blockDim.x + threadIdx.x; k < n; k += int64_t(gridDim.x) * blockDim.x) {
-        const int ww = int(k % W), hh = int((k / W) % H);
-        const int64_t c = k / (int64_t(W) * H);
-        dx[k] += 0.25f * dy[(c * (H / 2) + hh / 2) * (W / 2) + ww / 2];
-    }
+    const unsigned n = unsigned(H) * unsigned(W), w2 = unsigned(W) / 2;
+    for (int64_t c = blockIdx.y; c < NC; c += gridDim.y)
+        for (unsigned k = blockIdx.x * blockDim.x + threadIdx.x; k < n; k += gridDim.x * blockDim.x) {
+            const unsigned hh = k / unsigned(W), ww = k - hh * unsigned(W);
+            const float g = skip[c * n + k] + 0.25f * dy[c * (n / 4) + hh / 2 * w2 + ww / 2];
+            dx[c * n + k] = a[c * n + k] > 0.f ? g : 0.f;
+        }
 }
 
 // s [NC][2h][2w] = nearest upsample of a [NC][h][w] + skip.
 __global__ void k_up_add(const float *__restrict__ a, const float *__restrict__ skip, float *__restrict__ s, int64_t NC,
                          int h, int w)
 {
-    const int H = 2 * h, W = 2 * w;
-    const int64_t n = NC * H * W;
-    for (int64_t k = int64_t(blockIdx.x) * blockDim.x + threadIdx.x; k < n; k += int64_t(gridDim.x) * blockDim.x) {
-        const int ww = int(k % W), hh = int((k / W) % H);
-        const int64_t c = k / (int64_t(W) * H);
-        s[k] = a[(c * h + hh / 2) * w + ww / 2] + skip[k];
-    }
+    const unsigned W = 2 * unsigned(w), n = 4 * unsigned(h) * unsigned(w);
+    for (int64_t c = blockIdx.y; c < NC; c += gridDim.y)
+        for (unsigned k = blockIdx.x * blockDim.x + threadIdx.x; k < n; k += gridDim.x * blockDim.x) {
+            const unsigned hh = k / W, ww = k - hh * W;
+            s[c * n + k] = a[c * (n / 4) + hh / 2 * unsigned(w) + ww / 2] + skip[c * n + k];
+        }
 }
 
-// da [NC][h][w] = sum of the 4 gradients of its upsampled copies.
-__global__ void k_up_bwd(const float *__restrict__ ds, float *__restrict__ da, int64_t NC, int h, int w)
+// da [NC][h][w] = sum of the 4 gradients of its upsampled copies, zeroed where a <= 0.
+__global__ void k_up_bwd(const float *__restrict__ ds, const float *__restrict__ a, float *__restrict__ da, int64_t NC,
+                         int h, int w)
 {
+    const unsigned n = unsigned(h) * unsigned(w);
     const int W = 2 * w;
-    const int64_t n = NC * h * w;
-    for (int64_t k = int64_t(blockIdx.x) * blockDim.x + threadIdx.x; k < n; k += int64_t(gridDim.x) * blockDim.x) {
-        const int ww = int(k % w), hh = int((k / w) % h);
-        const int64_t c = k / (int64_t(w) * h);
-        const float *p = ds + (c * (2 * h) + 2 * hh) * W + 2 * ww;
-        da[k] = p[0] + p[1] + p[W] + p[W + 1];
-    }
+    for (int64_t c = blockIdx.y; c < NC; c += gridDim.y)
+        for (unsigned k = blockIdx.x * blockDim.x + threadIdx.x; k < n; k += gridDim.x * blockDim.x) {
+            const unsigned hh = k / unsigned(w), ww = k - hh * unsigned(w);
+            const float *p = ds + (c * (2 * h) + 2 * hh) * W + 2 * ww;
+            da[c * n + k] = a[c * n + k] > 0.f ? p[0] + p[1] + p[W] + p[W + 1] : 0.f;
+        }
 }
 
 __device__ __forceinline__ float softplus(float z) { return z > 20.f ? z : log1pf(expf(z)); }
 
-// Output head: channel ch of a sample (ch = (k / HW) % Co) is the image's
-// softplus(z) for ch < Q and z itself for the dual channels ch >= Q.
-__global__ void k_head(const float *__restrict__ z, float *__restrict__ o, int64_t n, int64_t HW, int Co, int Q)
+// Output head: channel c mod Co of a sample is the image's softplus(z) below Q
+// and z itself for the dual channels from Q on.
+__global__ void k_head(const float *__restrict__ z, float *__restrict__ o, int64_t NC, int HW, int Co, int Q)
 {
-    for (int64_t k = int64_t(blockIdx.x) * blockDim.x + threadIdx.x; k < n; k += int64_t(gridDim.x) * blockDim.x) {
-        const int ch = int((k / HW) % Co);
-        o[k] = ch < Q ? softplus(z[k]) : z[k];
+    for (int64_t c = blockIdx.y; c < NC; c += gridDim.y) {
+        const bool img = int(c % Co) < Q;
+        for (int k = blockIdx.x * blockDim.x + threadIdx.x; k < HW; k += gridDim.x * blockDim.x) {
+            const float zz = z[c * HW + k];
+            o[c * HW + k] = img ? softplus(zz) : zz;
+        }
     }
 }
 
+// |v| as FP64 by integer instructions (the FP64 unit, which a conversion also
+// occupies, does about 2 lanes per clock and multiprocessor): the exponent moved
+// to its new bias; below FP32's normal range 0 (its square is below 2^-252);
+// infinities and NaNs by a real conversion.
+__device__ __forceinline__ double abs_f64(float v)
+{
+    const uint32_t u = __float_as_uint(v) & 0x7FFFFFFFu;
+    if (u >= 0x7F800000u) return fabs(double(v));
+    return u >= 0x00800000u ? __hiloint2double(int((u >> 3) + 0x38000000u), int(u << 29)) : 0.0;
+}
+
 // loss += sum (head(z) - t)^2 / n (FP64); dz = 2 (head(z) - t) head'(z) / n with
-// head' = sigmoid on the image channels and 1 on the dual channels.
-__global__ void k_mse_head(const float *__restrict__ z, const float *__restrict__ tgt, float *__restrict__ dz,
-                           int64_t n, int64_t HW, int Co, int Q, double *__restrict__ loss)
+// head' = sigmoid on the image channels and 1 on the dual channels. One plane
+// at a time per block, one FP64 add to the loss per block.
+__global__ void __launch_bounds__(256)
+k_mse_head(const float *__restrict__ z, const float *__restrict__ tgt, float *__restrict__ dz, int64_t NC, int HW,
+           int Co, int Q, double *__restrict__ loss)
 {
     __shared__ double sh[32];
     double acc = 0.0;
+    const int64_t n = NC * HW;
     const float inv = 1.0f / float(n);
-    for (int64_t k = int64_t(blockIdx.x) * blockDim.x + threadIdx.x; k < n; k += int64_t(gridDim.x) * blockDim.x) {
-        const float zz = z[k];
-        const bool img = int((k / HW) % Co) < Q;
-        const float diff = (img ? softplus(zz) : zz) - tgt[k];
-        acc += double(diff) * double(diff);
-        dz[k] = img ? 2.f * diff * inv / (1.f + expf(-zz)) : 2.f * diff * inv;
+    for (int64_t c = blockIdx.x; c < NC; c += gridDim.x) {
+        const bool img = int(c % Co) < Q;
+        for (int k = threadIdx.x; k < HW; k += blockDim.x) {
+            const float zz = z[c * HW + k];
+            const float diff = (img ? softplus(zz) : zz) - tgt[c * HW + k];
+            const double a = abs_f64(diff);
+            acc = fma(a, a, acc);
+            dz[c * HW + k] = img ? 2.f * diff * inv / (1.f + expf(-zz)) : 2.f * diff * inv;
+        }
     }
     for (int o = 16; o > 0; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
     if ((threadIdx.x & 31) == 0) sh[threadIdx.x >> 5] = acc;
@@ -265,8 +619,7 @@ __global__ void k_mse_head(const float *__restrict__ z, const float *__restrict_
 }
 
 __global__ void k_adam(float *__restrict__ w, const float *__restrict__ g, float *__restrict__ m, float *__restrict__ v,
-                       __nv_bfloat16 *__restrict__ wb, int64_t n, float lr, float b1, float b2, float eps, float c1,
-                       float c2)
+                       int64_t n, float lr, float b1, float b2, float eps, float c1, float c2)
 {
     for (int64_t k = int64_t(blockIdx.x) * blockDim.x + threadIdx.x; k < n; k += int64_t(gridDim.x) * blockDim.x) {
         const float gk = g[k];
@@ -274,16 +627,8 @@ __global__ void k_adam(float *__restrict__ w, const float *__restrict__ g, float
         const float vk = b2 * v[k] + (1.f - b2) * gk * gk;
         m[k] = mk;
         v[k] = vk;
-        const float wk = w[k] - lr * (mk / c1) / (sqrtf(vk / c2) + eps);
-        w[k] = wk;
-        wb[k] = __float2bfloat16_rn(wk);
+        w[k] -= lr * (mk / c1) / (sqrtf(vk / c2) + eps);
     }
-}
-
-__global__ void k_to_bf16(const float *__restrict__ w, __nv_bfloat16 *__restrict__ wb, int64_t n)
-{
-    for (int64_t k = int64_t(blockIdx.x) * blockDim.x + threadIdx.x; k < n; k += int64_t(gridDim.x) * blockDim.x)
-        wb[k] = __float2bfloat16_rn(w[k]);
 }
 
 __global__ void k_pack_input(const float *__restrict__ bp, int Nx, int Nz, int Nq, float inv_scale, float level,
@@ -339,7 +684,9 @@ struct wsnet_ctx {
     Layer L[9];
     int64_t P = 0;
     float *w = nullptr, *g = nullptr, *m = nullptr, *v = nullptr;
-    __nv_bfloat16 *wb = nullptr, *wt = nullptr;  // BF16 weights, flipped scratch
+    uint32_t *wp = nullptr;  // BF16 weights in the orders that the convolutions read them (PackTable)
+    PackTable pack{};
+    int sms = 1;
     // activations and gradients
     float *a1, *a2, *p1, *a3, *a4, *p2, *a5, *a6, *s1, *a7, *s2, *a8, *z;
     float *gz, *g8, *gs2, *g7, *gs1, *g6, *g5, *gp2, *g4, *g3, *gp1, *g2, *g1;
@@ -370,52 +717,100 @@ void *walloc(wsnet_t h, size_t bytes)
     return p;
 }
 
-void conv_fwd(wsnet_t h, const float *x, int l, float *y, int N, int Hh, int Ww, bool relu)
+// Inference: the larger block where it leaves every multiprocessor one of them,
+// the smaller one (a quarter of the work) otherwise.
+template <bool RELU>
+void conv_tc(wsnet_t h, const float *x, int l, float *y, int N, int Hh, int Ww)
 {
     const Layer &L = h->L[l];
-    dim3 grid(unsigned(((Hh + TH - 1) / TH) * ((Ww + TW - 1) / TW)), unsigned((L.co + TC - 1) / TC), unsigned(N));
-    if (relu)
-        k_conv_fwd<true><<<grid, kT, 0, h->stream>>>(x, h->wb + L.woff, h->w + L.boff, y, L.ci, L.co, Hh, Ww);
-    else
-        k_conv_fwd<false><<<grid, kT, 0, h->stream>>>(x, h->wb + L.woff, h->w + L.boff, y, L.ci, L.co, Hh, Ww);
+    const unsigned tw = unsigned((Ww + 15) / 16), c16 = unsigned((L.co + 15) / 16);
+    const uint4 *w = reinterpret_cast<const uint4 *>(h->wp + h->pack.at[0][l]);
+    const float *b = h->w + L.boff;
+    const dim3 big(tw * unsigned((Hh + 7) / 8), (c16 + 3) / 4, unsigned(N));
+    if (uint64_t(big.x) * big.y * big.z >= unsigned(h->sms)) {
+        k_conv<4, 2, 8, RELU><<<big, 256, 0, h->stream>>>(x, w, b, y, L.ci, L.co, Hh, Ww);
+        return;
+    }
+    const dim3 small(tw * unsigned((Hh + 3) / 4), (c16 + 1) / 2, unsigned(N));
+    k_conv<2, 2, 4, RELU><<<small, 128, 0, h->stream>>>(x, w, b, y, L.ci, L.co, Hh, Ww);
 }
 
-// dy -> weight and bias gradients, and (if dx) the data gradient.
-void conv_bwd(wsnet_t h, const float *x, const float *dy, int l, float *dx, int N, int Hh, int Ww)
+// Training: 64 channels of 16 x 16 pixels a block where that gives every
+// multiprocessor about one, else 32 channels of 8 x 16.
+template <bool RELU, bool MASK>
+void conv_fma(wsnet_t h, const float *x, const uint32_t *w, const float *b, const float *mask, float *y, int Ci, int Co,
+              int N, int Hh, int Ww)
+{
+    const unsigned tw = unsigned((Ww + 15) / 16);
+    const float *wf = reinterpret_cast<const float *>(w);
+    const dim3 big(tw * unsigned((Hh + 15) / 16), unsigned((Co + 63) / 64), unsigned(N));
+    if (4 * uint64_t(big.x) * big.y * big.z >= 3 * unsigned(h->sms)) {
+        k_conv_fma<2, 8, RELU, MASK>
+            <<<big, 256, 2 * 4 * kFmaStage<2, 8>, h->stream>>>(x, wf, b, mask, y, Ci, Co, Hh, Ww);
+        return;
+    }
+    const dim3 small(tw * unsigned((Hh + 7) / 8), unsigned((Co + 31) / 32), unsigned(N));
+    k_conv_fma<1, 4, RELU, MASK>
+        <<<small, 128, 2 * 4 * kFmaStage<1, 4>, h->stream>>>(x, wf, b, mask, y, Ci, Co, Hh, Ww);
+}
+
+void conv_fwd(wsnet_t h, const float *x, int l, float *y, int N, int Hh, int Ww, bool relu, bool training)
 {
     const Layer &L = h->L[l];
-    dim3 gw(unsigned((L.co + WC - 1) / WC), unsigned((L.ci + WI - 1) / WI), unsigned(N * ((Hh + TH - 1) / TH)));
-    k_conv_bwd_w<<<gw, kT, 0, h->stream>>>(x, dy, h->g + L.woff, h->g + L.boff, L.ci, L.co, Hh, Ww);
-    if (dx) {
-        k_flip_weights<<<blocks_for(int64_t(L.ci) * L.co * 9), kT, 0, h->stream>>>(h->wb + L.woff, h->wt, L.ci, L.co);
-        dim3 grid(unsigned(((Hh + TH - 1) / TH) * ((Ww + TW - 1) / TW)), unsigned((L.ci + TC - 1) / TC), unsigned(N));
-        k_conv_fwd<false><<<grid, kT, 0, h->stream>>>(dy, h->wt, nullptr, dx, L.co, L.ci, Hh, Ww);
+    const uint32_t *w = h->wp + h->pack.at[1][l];
+    if (!training) {
+        if (relu) conv_tc<true>(h, x, l, y, N, Hh, Ww);
+        else conv_tc<false>(h, x, l, y, N, Hh, Ww);
+    } else if (relu) {
+        conv_fma<true, false>(h, x, w, h->w + L.boff, nullptr, y, L.ci, L.co, N, Hh, Ww);
+    } else {
+        conv_fma<false, false>(h, x, w, h->w + L.boff, nullptr, y, L.ci, L.co, N, Hh, Ww);
     }
 }
 
-void relu_bwd(wsnet_t h, float *g, const float *a, int64_t n)
+// dy -> weight and bias gradients, and (if dx) the data gradient, zeroed where
+// mask <= 0 (if mask: the activation that the layer's input is, after its ReLU).
+void conv_bwd(wsnet_t h, const float *x, const float *dy, int l, float *dx, const float *mask, int N, int Hh, int Ww)
 {
-    k_relu_bwd<<<blocks_for(n), kT, 0, h->stream>>>(g, a, n);
+    const Layer &L = h->L[l];
+    const dim3 gw(unsigned((L.co + kWgCo - 1) / kWgCo), unsigned((L.ci + kWgCi - 1) / kWgCi),
+                  unsigned(N * ((Hh + kWgRows - 1) / kWgRows)));
+    k_conv_wgrad<<<gw, 128, kWgSmem, h->stream>>>(x, dy, h->g + L.woff, h->g + L.boff, L.ci, L.co, Hh, Ww);
+    if (!dx) return;
+    const uint32_t *w = h->wp + h->pack.at[2][l];
+    if (mask) conv_fma<false, true>(h, dy, w, nullptr, mask, dx, L.co, L.ci, N, Hh, Ww);
+    else conv_fma<false, false>(h, dy, w, nullptr, nullptr, dx, L.co, L.ci, N, Hh, Ww);
+}
+
+void pack_weights(wsnet_t h)
+{
+    k_pack_weights<<<blocks_for(h->pack.at[2][9]), kT, 0, h->stream>>>(h->w, h->wp, h->pack);
+}
+
+// Blocks over NC planes of n elements each.
+dim3 planes(int64_t NC, int64_t n)
+{
+    return dim3(unsigned((n + kT - 1) / kT), unsigned(NC < 65535 ? NC : 65535));
 }
 
 // The forward pass up to z (pre-softplus output).
-void forward_to_z(wsnet_t h, const float *x, int N)
+void forward_to_z(wsnet_t h, const float *x, int N, bool training)
 {
     const int H = h->H, W = h->W, H2 = H / 2, W2 = W / 2, H4 = H / 4, W4 = W / 4;
     cudaStream_t st = h->stream;
-    conv_fwd(h, x, 0, h->a1, N, H, W, true);
-    conv_fwd(h, h->a1, 1, h->a2, N, H, W, true);
-    k_pool_fwd<<<blocks_for(int64_t(N) * 64 * H2 * W2), kT, 0, st>>>(h->a2, h->p1, int64_t(N) * 64, H, W);
-    conv_fwd(h, h->p1, 2, h->a3, N, H2, W2, true);
-    conv_fwd(h, h->a3, 3, h->a4, N, H2, W2, true);
-    k_pool_fwd<<<blocks_for(int64_t(N) * 128 * H4 * W4), kT, 0, st>>>(h->a4, h->p2, int64_t(N) * 128, H2, W2);
-    conv_fwd(h, h->p2, 4, h->a5, N, H4, W4, true);
-    conv_fwd(h, h->a5, 5, h->a6, N, H4, W4, true);
-    k_up_add<<<blocks_for(int64_t(N) * 128 * H2 * W2), kT, 0, st>>>(h->a6, h->a4, h->s1, int64_t(N) * 128, H4, W4);
-    conv_fwd(h, h->s1, 6, h->a7, N, H2, W2, true);
-    k_up_add<<<blocks_for(int64_t(N) * 64 * H * W), kT, 0, st>>>(h->a7, h->a2, h->s2, int64_t(N) * 64, H2, W2);
-    conv_fwd(h, h->s2, 7, h->a8, N, H, W, true);
-    conv_fwd(h, h->a8, 8, h->z, N, H, W, false);
+    conv_fwd(h, x, 0, h->a1, N, H, W, true, training);
+    conv_fwd(h, h->a1, 1, h->a2, N, H, W, true, training);
+    k_pool_fwd<<<planes(int64_t(N) * 64, int64_t(H2) * W2), kT, 0, st>>>(h->a2, h->p1, int64_t(N) * 64, H, W);
+    conv_fwd(h, h->p1, 2, h->a3, N, H2, W2, true, training);
+    conv_fwd(h, h->a3, 3, h->a4, N, H2, W2, true, training);
+    k_pool_fwd<<<planes(int64_t(N) * 128, int64_t(H4) * W4), kT, 0, st>>>(h->a4, h->p2, int64_t(N) * 128, H2, W2);
+    conv_fwd(h, h->p2, 4, h->a5, N, H4, W4, true, training);
+    conv_fwd(h, h->a5, 5, h->a6, N, H4, W4, true, training);
+    k_up_add<<<planes(int64_t(N) * 128, int64_t(H2) * W2), kT, 0, st>>>(h->a6, h->a4, h->s1, int64_t(N) * 128, H4, W4);
+    conv_fwd(h, h->s1, 6, h->a7, N, H2, W2, true, training);
+    k_up_add<<<planes(int64_t(N) * 64, int64_t(H) * W), kT, 0, st>>>(h->a7, h->a2, h->s2, int64_t(N) * 64, H2, W2);
+    conv_fwd(h, h->s2, 7, h->a8, N, H, W, true, training);
+    conv_fwd(h, h->a8, 8, h->z, N, H, W, false, training);
 }
 
 }  // namespace
@@ -461,13 +856,37 @@ int wsnet_create(wsnet_t *out, int32_t H, int32_t W, int32_t Q, int32_t n_dual, 
         if (cudaStreamCreateWithFlags(&h->stream, cudaStreamNonBlocking) != cudaSuccess) return fail_create(SGTV_ERR_CUDA);
         h->own_stream = true;
     }
+    int dev = 0;
+    if (cudaGetDevice(&dev) != cudaSuccess ||
+        cudaDeviceGetAttribute(&h->sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess)
+        return fail_create(SGTV_ERR_CUDA);
+    auto opt_in = [](auto *kernel, int bytes) {
+        return cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes) == cudaSuccess;
+    };
+    constexpr int big = 2 * 4 * kFmaStage<2, 8>;
+    if (!opt_in(k_conv_wgrad, kWgSmem) || !opt_in(k_conv_fma<2, 8, true, false>, big) ||
+        !opt_in(k_conv_fma<2, 8, false, true>, big) || !opt_in(k_conv_fma<2, 8, false, false>, big))
+        return fail_create(SGTV_ERR_CUDA);
     const size_t P = size_t(h->P);
     h->w = static_cast<float *>(walloc(h, 4 * P));
     h->g = static_cast<float *>(walloc(h, 4 * P));
     h->m = static_cast<float *>(walloc(h, 4 * P));
     h->v = static_cast<float *>(walloc(h, 4 * P));
-    h->wb = static_cast<__nv_bfloat16 *>(walloc(h, 2 * P));
-    h->wt = static_cast<__nv_bfloat16 *>(walloc(h, 2 * size_t(256) * (h->Co > 256 ? h->Co : 256) * 9));
+    for (int l = 0; l < 9; l++) {
+        h->pack.ci[l] = h->L[l].ci;
+        h->pack.co[l] = h->L[l].co;
+        h->pack.w[l] = h->L[l].woff;
+    }
+    int64_t words = 0;
+    for (int form = 0; form < 3; form++)
+        for (int l = 0; l < 9; l++) {
+            const int64_t ci = h->L[l].ci, co = h->L[l].co;
+            h->pack.at[form][l] = words;
+            words += form == 0 ? (ci + 15) / 16 * ((co + 15) / 16) * 9 * 128
+                               : (form == 1 ? ci * 9 * ((co + 63) / 64 * 64) : co * 9 * ((ci + 63) / 64 * 64));
+            h->pack.at[form][l + 1] = words;
+        }
+    h->wp = static_cast<uint32_t *>(walloc(h, 4 * size_t(words)));
     h->loss = static_cast<double *>(walloc(h, sizeof(double)));
     const size_t N = size_t(max_batch);
     const size_t f1 = N * H * W, f2 = N * (H / 2) * (W / 2), f4 = N * (H / 4) * (W / 4);
@@ -486,7 +905,7 @@ int wsnet_create(wsnet_t *out, int32_t H, int32_t W, int32_t Q, int32_t n_dual, 
     h->g5 = static_cast<float *>(walloc(h, 4 * f4 * 256));
     for (void *p : h->blocks)
         if (!p) return fail_create(SGTV_ERR_OOM);
-    if (h->blocks.size() != 7 + 8 + 2 + 4 + 6 + 4 + 2) return fail_create(SGTV_ERR_OOM);
+    if (h->blocks.size() != 6 + 8 + 2 + 4 + 6 + 4 + 2) return fail_create(SGTV_ERR_OOM);
     // He initialisation (normal, std sqrt(2 / fan_in)), deterministic from seed; biases 0
     std::vector<float> hw(P, 0.f);
     std::mt19937_64 rng(seed);
@@ -519,7 +938,7 @@ int wsnet_set_params(wsnet_t h, const float *host)
     WK(h, cudaMemsetAsync(h->m, 0, 4 * P, h->stream));
     WK(h, cudaMemsetAsync(h->v, 0, 4 * P, h->stream));
     WK(h, cudaMemsetAsync(h->g, 0, 4 * P, h->stream));
-    k_to_bf16<<<blocks_for(h->P), kT, 0, h->stream>>>(h->w, h->wb, h->P);
+    pack_weights(h);
     WK(h, cudaGetLastError());
     WK(h, cudaStreamSynchronize(h->stream));
     h->step = 0;
@@ -546,10 +965,10 @@ int wsnet_forward(wsnet_t h, const float *x, int32_t N, float *out)
 {
     if (!h || !x || !out) return SGTV_ERR_ARG;
     if (N < 1 || N > h->maxN) return wfail(h, SGTV_ERR_ARG, "N must be in [1, max_batch]");
-    forward_to_z(h, x, N);
-    const int64_t HW = int64_t(h->H) * h->W;
-    const int64_t n = int64_t(N) * h->Co * HW;
-    k_head<<<blocks_for(n), kT, 0, h->stream>>>(h->z, out, n, HW, h->Co, h->C);
+    forward_to_z(h, x, N, false);
+    const int HW = h->H * h->W;
+    const int64_t NC = int64_t(N) * h->Co;
+    k_head<<<planes(NC, HW), kT, 0, h->stream>>>(h->z, out, NC, HW, h->Co, h->C);
     WK(h, cudaGetLastError());
     return SGTV_OK;
 }
@@ -560,38 +979,28 @@ int wsnet_loss_grad(wsnet_t h, const float *x, const float *target, int32_t N, d
     if (N < 1 || N > h->maxN) return wfail(h, SGTV_ERR_ARG, "N must be in [1, max_batch]");
     const int H = h->H, W = h->W, H2 = H / 2, W2 = W / 2, H4 = H / 4, W4 = W / 4;
     cudaStream_t st = h->stream;
-    forward_to_z(h, x, N);
+    forward_to_z(h, x, N, true);
     WK(h, cudaMemsetAsync(h->g, 0, 4 * size_t(h->P), st));
     WK(h, cudaMemsetAsync(h->loss, 0, sizeof(double), st));
-    const int64_t nz = int64_t(N) * h->Co * H * W;
-    k_mse_head<<<blocks_for(nz), kT, 0, st>>>(h->z, target, h->gz, nz, int64_t(H) * W, h->Co, h->C, h->loss);
-    const int64_t n64 = int64_t(N) * 64 * H * W, n64h = int64_t(N) * 64 * H2 * W2, n128h = int64_t(N) * 128 * H2 * W2;
-    const int64_t n128q = int64_t(N) * 128 * H4 * W4, n256q = int64_t(N) * 256 * H4 * W4;
-    conv_bwd(h, h->a8, h->gz, 8, h->g8, N, H, W);
-    relu_bwd(h, h->g8, h->a8, n64);
-    conv_bwd(h, h->s2, h->g8, 7, h->gs2, N, H, W);
+    const int64_t nz = int64_t(N) * h->Co, n64 = int64_t(N) * 64, n128 = int64_t(N) * 128;
+    const int64_t full = int64_t(H) * W, half = int64_t(H2) * W2, quarter = int64_t(H4) * W4;
+    k_mse_head<<<unsigned(nz < 8 * int64_t(h->sms) ? nz : 8 * int64_t(h->sms)), kT, 0, st>>>(h->z, target, h->gz, nz,
+                                                                                            H * W, h->Co, h->C, h->loss);
+    conv_bwd(h, h->a8, h->gz, 8, h->g8, h->a8, N, H, W);
+    conv_bwd(h, h->s2, h->g8, 7, h->gs2, nullptr, N, H, W);
     // s2 = up(a7) + a2
-    WK(h, cudaMemcpyAsync(h->g2, h->gs2, 4 * size_t(n64), cudaMemcpyDeviceToDevice, st));
-    k_up_bwd<<<blocks_for(n64h), kT, 0, st>>>(h->gs2, h->g7, int64_t(N) * 64, H2, W2);
-    relu_bwd(h, h->g7, h->a7, n64h);
-    conv_bwd(h, h->s1, h->g7, 6, h->gs1, N, H2, W2);
+    k_up_bwd<<<planes(n64, half), kT, 0, st>>>(h->gs2, h->a7, h->g7, n64, H2, W2);
+    conv_bwd(h, h->s1, h->g7, 6, h->gs1, nullptr, N, H2, W2);
     // s1 = up(a6) + a4
-    WK(h, cudaMemcpyAsync(h->g4, h->gs1, 4 * size_t(n128h), cudaMemcpyDeviceToDevice, st));
-    k_up_bwd<<<blocks_for(n128q), kT, 0, st>>>(h->gs1, h->g6, int64_t(N) * 128, H4, W4);
-    relu_bwd(h, h->g6, h->a6, n128q);
-    conv_bwd(h, h->a5, h->g6, 5, h->g5, N, H4, W4);
-    relu_bwd(h, h->g5, h->a5, n256q);
-    conv_bwd(h, h->p2, h->g5, 4, h->gp2, N, H4, W4);
-    k_pool_bwd_add<<<blocks_for(n128h), kT, 0, st>>>(h->gp2, h->g4, int64_t(N) * 128, H2, W2);
-    relu_bwd(h, h->g4, h->a4, n128h);
-    conv_bwd(h, h->a3, h->g4, 3, h->g3, N, H2, W2);
-    relu_bwd(h, h->g3, h->a3, n128h);
-    conv_bwd(h, h->p1, h->g3, 2, h->gp1, N, H2, W2);
-    k_pool_bwd_add<<<blocks_for(n64), kT, 0, st>>>(h->gp1, h->g2, int64_t(N) * 64, H, W);
-    relu_bwd(h, h->g2, h->a2, n64);
-    conv_bwd(h, h->a1, h->g2, 1, h->g1, N, H, W);
-    relu_bwd(h, h->g1, h->a1, n64);
-    conv_bwd(h, x, h->g1, 0, nullptr, N, H, W);
+    k_up_bwd<<<planes(n128, quarter), kT, 0, st>>>(h->gs1, h->a6, h->g6, n128, H4, W4);
+    conv_bwd(h, h->a5, h->g6, 5, h->g5, h->a5, N, H4, W4);
+    conv_bwd(h, h->p2, h->g5, 4, h->gp2, nullptr, N, H4, W4);
+    k_pool_bwd<<<planes(n128, half), kT, 0, st>>>(h->gp2, h->gs1, h->a4, h->g4, n128, H2, W2);
+    conv_bwd(h, h->a3, h->g4, 3, h->g3, h->a3, N, H2, W2);
+    conv_bwd(h, h->p1, h->g3, 2, h->gp1, nullptr, N, H2, W2);
+    k_pool_bwd<<<planes(n64, full), kT, 0, st>>>(h->gp1, h->gs2, h->a2, h->g2, n64, H, W);
+    conv_bwd(h, h->a1, h->g2, 1, h->g1, h->a1, N, H, W);
+    conv_bwd(h, x, h->g1, 0, nullptr, nullptr, N, H, W);
     WK(h, cudaGetLastError());
     if (loss) {
         WK(h, cudaMemcpyAsync(loss, h->loss, sizeof(double), cudaMemcpyDeviceToHost, st));
@@ -605,7 +1014,8 @@ int wsnet_adam_step(wsnet_t h, float lr, float beta1, float beta2, float eps)
     if (!h) return SGTV_ERR_ARG;
     h->step += 1;
     const float c1 = 1.f - powf(beta1, float(h->step)), c2 = 1.f - powf(beta2, float(h->step));
-    k_adam<<<blocks_for(h->P), kT, 0, h->stream>>>(h->w, h->g, h->m, h->v, h->wb, h->P, lr, beta1, beta2, eps, c1, c2);
+    k_adam<<<blocks_for(h->P), kT, 0, h->stream>>>(h->w, h->g, h->m, h->v, h->P, lr, beta1, beta2, eps, c1, c2);
+    pack_weights(h);
     WK(h, cudaGetLastError());
     return SGTV_OK;
 }
