@@ -590,7 +590,7 @@ def time_form(sgtv, P, args, form, stream, torch, barrier, ws, sample_clocks=Fal
     if pin_sc:
         h.set_variant(sgtv.K_SCATTER, names["k_scatter"].index(args.scatter_variant))
     if form == "single_pass":
-        tuning = {"k_scatter": names["k_scatter"][h.get_variant(sgtv.K_SCATTER)], "k_fupdate": "per site",
+        tuning = {"k_scatter": names["k_scatter"][h.get_variant(sgtv.K_SCATTER)], "k_fupdate": "per voxel",
                   "k_shrink": "per site"}
     else:
         vf, vb = h.get_variants()

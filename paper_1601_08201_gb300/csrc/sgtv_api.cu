@@ -955,6 +955,8 @@ static int setup_impl(sgtv_t *out, int32_t nscans, const sgtv_scan *sc, const sg
             tab[k].beta = sc[k].lambda;
             tab[k].rhof = float(tab[k].rho);
             tab[k].tauf = float(tab[k].tau);
+            set_divisor(uint32_t(sc[k].Nq), tab[k].q_mul, tab[k].q_shift);
+            set_divisor(uint32_t(sc[k].Nz), tab[k].z_mul, tab[k].z_shift);
         }
         h->scan_tab = tab;
         SK(cudaMemcpyAsync(p_scans, h->scan_tab.data(), sizeof(Scan) * nscans, cudaMemcpyHostToDevice, st));

@@ -15,7 +15,16 @@ struct Scan {
     int32_t Nx, Nz, Nq, pad_;
     double rho, tau, beta;      // ADMM penalty, shrink threshold beta / rho, regularisation weight
     float rhof, tauf;           // rho and tau rounded to FP32 once (the FP32 kernels' operands)
+    // n / Nq and n / Nz for n < 2^31: (umulhi(mul, n) + n) >> shift (Granlund and Montgomery, PLDI 1994)
+    uint32_t q_mul, q_shift, z_mul, z_shift;
 };
+
+inline void set_divisor(uint32_t d, uint32_t &mul, uint32_t &shift)
+{
+    shift = 0;
+    while ((uint64_t(1) << shift) < d) shift++;
+    mul = uint32_t(((uint64_t(1) << 32) * ((uint64_t(1) << shift) - d)) / d + 1);
+}
 
 // The group-TV stencil (Eq. 2): direction p moves (dx[p], dz[p]) in (x, z)
 // with weight w[p]; plus the per-scan geometry (device tables).

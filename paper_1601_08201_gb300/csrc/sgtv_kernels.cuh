@@ -1604,110 +1604,108 @@ k_scatter_sp(int64_t I, int64_t J, const int64_t *__restrict__ rp, const uint16_
     for (int k = threadIdx.x + 256 * kU; k < nstage; k += blockDim.x) flush(k, wl > 0 ? 0 : tl.uidx[u0 + k]);
 }
 
-// The f-update (Eq. 5 closed form) from the accumulated e, which it clears
-// for the next scatter: one warp per spatial site, lanes over q. It reads
-// u = d - c as the shrink left it (one load per direction and position
-// instead of two), the site's stencil (which neighbours exist, their
-// offsets) is found once per warp, and QB q-steps of every lane issue all
-// their loads before any arithmetic, which is that of voxel_update_at in the
-// same order.
+// The f-update (Eq. 5 closed form) from e and u = d - c as the shrink left it:
+// a thread per hyper-voxel, B of them 256 apart, every load before any
+// arithmetic, which is that of voxel_update_at in the same order. Voxels in
+// storage order fill the lanes for any number of q-bins (a warp per site left
+// half of them idle at 16 and went through its sites one after the other: 22 us
+// at 16384 sites of 16 or 32 q-bins), and the place in the image costs two
+// multiplications with the scan's precomputed divisors. The four neighbours'
+// f serve both the forward and the backward terms: the directions are the
+// library's own (+x, -x, +z, -z or +x, +z).
 //
-// poff = NULL: e is the accumulated vector, cleared here. Else e holds
+// PART = false: e is the accumulated vector, cleared here. PART = true: e holds
 // partial sums (k_rows_stack), those of hyper-voxel j at poff[j] .. poff[j+1],
 // added up in that order.
 template <typename T>
 __device__ __forceinline__ T sum_parts(const T *__restrict__ part, const int32_t *__restrict__ poff, int64_t j)
 {
     T a = T(0);
-    for (int k = poff[j], k1 = poff[j + 1]; k < k1; k++) a += part[k];
+    int k = poff[j];
+    const int k1 = poff[j + 1];
+    for (; k + 4 <= k1; k += 4) {  // four loads in flight, added in order
+        const T v0 = part[k], v1 = part[k + 1], v2 = part[k + 2], v3 = part[k + 3];
+        a = (((a + v0) + v1) + v2) + v3;
+    }
+    for (; k < k1; k++) a += part[k];
     return a;
 }
 
-template <typename T, int QB, bool PART = false>
-__global__ void __launch_bounds__(256, QB == 1 ? 4 : 3)
-k_fupdate_site(Geom g, T *__restrict__ e, const T *__restrict__ s, const T *__restrict__ f,
-               const T *__restrict__ u, T *__restrict__ f_new, const int32_t *__restrict__ poff = nullptr)
+template <typename T, int ND, int B, bool ONE, bool PART>
+__global__ void __launch_bounds__(256)
+k_fupdate(Geom g, T *__restrict__ e, const T *__restrict__ s, const T *__restrict__ f, const T *__restrict__ u,
+          T *__restrict__ f_new, const int32_t *__restrict__ poff)
 {
-    const int lane = threadIdx.x & 31;
-    const int64_t nwarps = (int64_t(gridDim.x) * blockDim.x) >> 5;
-#pragma unroll 1
-    for (int64_t site = (int64_t(blockIdx.x) * blockDim.x + threadIdx.x) >> 5; site < g.S; site += nwarps) {
-        int64_t v0;
-        const Loc L = locate_site(g, site, v0);
-        int32_t stF[4], stB[4];  // offsets of the existing neighbours (0 for a ghost: the voxel itself, unused)
-        bool inF[4], inB[4];
+    const int64_t j0 = int64_t(blockIdx.x) * (256 * B) + threadIdx.x;
+    T ej[B], fj[B], sj[B], fp[B], fm[B], fu[B], fd[B], uF[B][ND], uB[B][ND], rho[B];
+    bool xp[B], xm[B], zp[B], zm[B];
 #pragma unroll
-        for (int p = 0; p < 4; p++) {
-            const int32_t step = p < g.n_dirs ? int32_t(step_of(g, L, p)) : 0;
-            inF[p] = p < g.n_dirs && inside(L, L.x + g.dx[p], L.z + g.dz[p]);
-            inB[p] = p < g.n_dirs && inside(L, L.x - g.dx[p], L.z - g.dz[p]);
-            stF[p] = inF[p] ? step : 0;
-            stB[p] = inB[p] ? step : 0;
-        }
-        const T rho = lrho<T>(L);
-        const int nd = g.n_dirs;
-#pragma unroll 1
-        for (int q0 = 0; q0 < L.Nq; q0 += 32 * QB) {
-            T ej[QB], fj[QB], sj[QB], fF[QB][4], fB[QB][4], uF[QB][4], uB[QB][4];
+    for (int b = 0; b < B; b++) {
+        const int64_t j = j0 + 256 * b < g.J ? j0 + 256 * b : g.J - 1;  // past the end: the last voxel, not written
+        const Scan &sc = g.scans[ONE ? 0 : scan_of(g.vox_off, g.nscans, j)];
+        const uint32_t v = uint32_t(j - sc.vox0);  // J < 2^31
+        const uint32_t site = (__umulhi(sc.q_mul, v) + v) >> sc.q_shift;
+        const int32_t x = int32_t((__umulhi(sc.z_mul, site) + site) >> sc.z_shift);
+        const int32_t z = int32_t(site) - x * sc.Nz;
+        Loc L;
+        L.rho = sc.rho;
+        L.rhof = sc.rhof;
+        rho[b] = lrho<T>(L);
+        xp[b] = x + 1 < sc.Nx;
+        xm[b] = x > 0;
+        zp[b] = z + 1 < sc.Nz;
+        zm[b] = z > 0;
+        const int64_t sx = int64_t(sc.Nz) * sc.Nq, sz = sc.Nq;
+        const int64_t up = xp[b] ? sx : 0, um = xm[b] ? sx : 0, vp = zp[b] ? sz : 0, vm = zm[b] ? sz : 0;
+        ej[b] = PART ? sum_parts<T>(e, poff, j) : e[j];
+        fj[b] = f[j];
+        sj[b] = s[j];
+        fp[b] = f[j + up];  // a ghost's operand is not used
+        fm[b] = f[j - um];
+        fu[b] = f[j + vp];
+        fd[b] = f[j - vm];
 #pragma unroll
-            for (int b = 0; b < QB; b++) {
-                const int q = q0 + 32 * b + lane;
-                const bool act = q < L.Nq;
-                const int64_t j = v0 + (act ? q : 0);
-                ej[b] = PART ? sum_parts<T>(e, poff, j) : e[j];
-                fj[b] = f[j];
-                sj[b] = s[j];
-#pragma unroll
-                for (int p = 0; p < 4; p++) {
-                    const int64_t pj = int64_t(p < nd ? p : 0) * g.J + j;
-                    fF[b][p] = f[j + stF[p]];
-                    fB[b][p] = f[j - stB[p]];
-                    uF[b][p] = u[pj];
-                    uB[b][p] = u[pj - stB[p]];
-                }
-            }
-#pragma unroll
-            for (int b = 0; b < QB; b++) {
-                const int q = q0 + 32 * b + lane;
-                if (q >= L.Nq) continue;
-                const int64_t j = v0 + q;
-                if (!PART) e[j] = T(0);
-                T alpha = T(0), gamma = T(0);
-#pragma unroll
-                for (int p = 0; p < 4; p++) {
-                    if (p >= nd) break;
-                    const T w = wgt<T>(g, p);
-                    const T w2 = w * w;
-                    if (inF[p]) {
-                        alpha += w2;
-                        gamma += w * (w * (fj[b] + fF[b][p]) + uF[b][p]);
-                    } else {
-                        alpha += T(0.5) * w2;
-                        gamma += w * uF[b][p];
-                    }
-                    if (inB[p]) {
-                        alpha += w2;
-                        gamma += w * (w * (fB[b][p] + fj[b]) - uB[b][p]);
-                    }
-                }
-                alpha *= rho;
-                gamma *= rho;
-                f_new[j] = sgtv_root<T>(alpha, sj[b] - gamma, fj[b] * ej[b], sj[b]);
-            }
+        for (int p = 0; p < ND; p++) uF[b][p] = u[int64_t(p) * g.J + j];
+        if (ND == 4) {
+            uB[b][0] = u[j - um];
+            uB[b][1] = u[g.J + j + up];
+            uB[b][2] = u[2 * g.J + j - vm];
+            uB[b][ND - 1] = u[3 * g.J + j + vp];
+        } else {
+            uB[b][0] = u[j - um];
+            uB[b][1] = u[g.J + j - vm];
         }
     }
-}
-
-// Same update, one thread per hyper-voxel.
-template <typename T, bool PART = false>
-__global__ void __launch_bounds__(256)
-k_fupdate(Geom g, T *__restrict__ e, const T *__restrict__ s, const T *__restrict__ f, const T *__restrict__ d,
-          const T *__restrict__ c, T *__restrict__ f_new, const int32_t *__restrict__ poff = nullptr)
-{
-    for (int64_t j = int64_t(blockIdx.x) * blockDim.x + threadIdx.x; j < g.J; j += int64_t(gridDim.x) * blockDim.x) {
-        const T ej = PART ? sum_parts<T>(e, poff, j) : e[j];
+#pragma unroll
+    for (int b = 0; b < B; b++) {
+        const int64_t j = j0 + 256 * b;
+        if (j >= g.J) break;
         if (!PART) e[j] = T(0);
-        f_new[j] = voxel_update<T, true>(g, j, ej, s, f, d, c);
+        T alpha = T(0), gamma = T(0);
+#pragma unroll
+        for (int p = 0; p < ND; p++) {
+            const T w = wgt<T>(g, p);
+            const T w2 = w * w;
+            const int d = ND == 4 ? p : 2 * p;  // direction: +x, -x, +z, -z
+            const bool inF = d == 0 ? xp[b] : (d == 1 ? xm[b] : (d == 2 ? zp[b] : zm[b]));
+            const bool inB = d == 0 ? xm[b] : (d == 1 ? xp[b] : (d == 2 ? zm[b] : zp[b]));
+            const T fF = d == 0 ? fp[b] : (d == 1 ? fm[b] : (d == 2 ? fu[b] : fd[b]));
+            const T fB = d == 0 ? fm[b] : (d == 1 ? fp[b] : (d == 2 ? fd[b] : fu[b]));
+            if (inF) {
+                alpha += w2;
+                gamma += w * (w * (fj[b] + fF) + uF[b][p]);
+            } else {
+                alpha += T(0.5) * w2;
+                gamma += w * uF[b][p];
+            }
+            if (inB) {
+                alpha += w2;
+                gamma += w * (w * (fB + fj[b]) - uB[b][p]);
+            }
+        }
+        alpha *= rho[b];
+        gamma *= rho[b];
+        f_new[j] = sgtv_root<T>(alpha, sj[b] - gamma, fj[b] * ej[b], sj[b]);
     }
 }
 

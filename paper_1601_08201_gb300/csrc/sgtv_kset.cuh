@@ -377,13 +377,22 @@ struct Impl {
         k_dual_rule<T><<<grid_for(g.S, d.sm_count * 8), kThreads, 0, st>>>(
             g, static_cast<const T *>(d.d), static_cast<T *>(d.c), theta);
     }
-    template <int QB>
-    static void fupdate_site(const Dev &d, const Geom &g, void *e, const void *f, void *f_new, cudaStream_t st)
+    // Two voxels a thread where that still leaves four blocks a multiprocessor, else one.
+    template <int ND, bool PART>
+    static void fupdate_nd(const Dev &d, const Geom &g, void *e, const void *f, void *f_new, const int32_t *poff,
+                           cudaStream_t st)
     {
-        static const int nb = resident_blocks(k_fupdate_site<T, QB>);
-        k_fupdate_site<T, QB><<<grid_for(g.S, d.sm_count * nb), kThreads, 0, st>>>(
-            g, static_cast<T *>(e), static_cast<const T *>(d.s), static_cast<const T *>(f),
-            static_cast<const T *>(d.u), static_cast<T *>(f_new));
+        T *ee = static_cast<T *>(e), *fn = static_cast<T *>(f_new);
+        const T *s = static_cast<const T *>(d.s), *ff = static_cast<const T *>(f), *u = static_cast<const T *>(d.u);
+        const int64_t one = (g.J + 255) / 256;
+        if (one >= 8 * int64_t(d.sm_count)) {
+            const unsigned blocks = unsigned((g.J + 511) / 512);
+            if (g.nscans == 1) k_fupdate<T, ND, 2, true, PART><<<blocks, 256, 0, st>>>(g, ee, s, ff, u, fn, poff);
+            else k_fupdate<T, ND, 2, false, PART><<<blocks, 256, 0, st>>>(g, ee, s, ff, u, fn, poff);
+        } else {
+            if (g.nscans == 1) k_fupdate<T, ND, 1, true, PART><<<unsigned(one), 256, 0, st>>>(g, ee, s, ff, u, fn, poff);
+            else k_fupdate<T, ND, 1, false, PART><<<unsigned(one), 256, 0, st>>>(g, ee, s, ff, u, fn, poff);
+        }
     }
     static void sub(int64_t n, const void *a, const void *b, void *out, cudaStream_t st)
     {
@@ -394,37 +403,14 @@ struct Impl {
     }
     static void fupdate(const Dev &d, const Geom &g, void *e, const void *f, void *f_new, cudaStream_t st)
     {
-        if (g.max_nq >= 16 && d.u) {  // a warp per site: lanes over q-bins
-            if (g.max_nq <= 32) fupdate_site<1>(d, g, e, f, f_new, st);
-            else fupdate_site<2>(d, g, e, f, f_new, st);
-            return;
-        }
-        int64_t blocks = (d.J + kThreads - 1) / kThreads;  // one hyper-voxel per thread
-        blocks = blocks > (int64_t(1) << 30) ? (int64_t(1) << 30) : (blocks < 1 ? 1 : blocks);
-        k_fupdate<T><<<unsigned(blocks), kThreads, 0, st>>>(g, static_cast<T *>(e), static_cast<const T *>(d.s),
-                                                  static_cast<const T *>(f), static_cast<const T *>(d.d),
-                                                  static_cast<const T *>(d.c), static_cast<T *>(f_new));
+        if (g.n_dirs == 4) fupdate_nd<4, false>(d, g, e, f, f_new, nullptr, st);
+        else fupdate_nd<2, false>(d, g, e, f, f_new, nullptr, st);
     }
     // The f-update from the partial sums that the stacked forward pass left.
-    template <int QB>
-    static void back_stack_site(const Dev &d, const Geom &g, const void *f, void *f_new, cudaStream_t st)
-    {
-        static const int nb = resident_blocks(k_fupdate_site<T, QB, true>);
-        k_fupdate_site<T, QB, true><<<grid_for(g.S, d.sm_count * nb), kThreads, 0, st>>>(
-            g, static_cast<T *>(d.st.part), static_cast<const T *>(d.s), static_cast<const T *>(f),
-            static_cast<const T *>(d.u), static_cast<T *>(f_new), d.st.poff);
-    }
     static void back_stack(const Dev &d, const Geom &g, const void *f, void *f_new, cudaStream_t st)
     {
-        if (g.max_nq >= 16) {
-            if (g.max_nq <= 32) back_stack_site<1>(d, g, f, f_new, st);
-            else back_stack_site<2>(d, g, f, f_new, st);
-            return;
-        }
-        int64_t blocks = (d.J + kThreads - 1) / kThreads;
-        k_fupdate<T, true><<<unsigned(blocks), kThreads, 0, st>>>(
-            g, static_cast<T *>(d.st.part), static_cast<const T *>(d.s), static_cast<const T *>(f),
-            static_cast<const T *>(d.d), static_cast<const T *>(d.c), static_cast<T *>(f_new), d.st.poff);
+        if (g.n_dirs == 4) fupdate_nd<4, true>(d, g, d.st.part, f, f_new, d.st.poff, st);
+        else fupdate_nd<2, true>(d, g, d.st.part, f, f_new, d.st.poff, st);
     }
     static void backproject(const Dev &d, const void *v, void *out, cudaStream_t st)
     {
