@@ -477,12 +477,16 @@ struct Impl {
         }
         finalize(d.part, blocks, 1, 0u, d.red + slot, st);
     }
+    // Up to twice the blocks of the other reductions: two partial fields fit twice in Dev::part.
     static void tv(const Dev &d, const Geom &g, const void *f, const void *dsplit, int64_t s0, int64_t s1, int slot,
                    cudaStream_t st)
     {
-        k_tv_partials<T><<<d.red_blocks, kThreads, 0, st>>>(g, static_cast<const T *>(f),
-                                                            static_cast<const T *>(dsplit), s0, s1, d.part);
-        finalize(d.part, d.red_blocks, 2, 0u, d.red + slot, st);
+        const T *ff = static_cast<const T *>(f), *dd = static_cast<const T *>(dsplit);
+        const int blocks = grid_for(s1 - s0, 2 * d.red_blocks);
+        if (dd) k_tv_partials<T, true, false><<<blocks, kThreads, 0, st>>>(g, ff, dd, s0, s1, d.part);
+        else if (g.per_bin) k_tv_partials<T, false, true><<<blocks, kThreads, 0, st>>>(g, ff, dd, s0, s1, d.part);
+        else k_tv_partials<T, false, false><<<blocks, kThreads, 0, st>>>(g, ff, dd, s0, s1, d.part);
+        finalize(d.part, blocks, 2, 0u, d.red + slot, st);
     }
     static void kkt(const Dev &d, const Geom &g, const void *f, int slot, cudaStream_t st)
     {

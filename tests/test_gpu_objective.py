@@ -60,3 +60,22 @@ def test_objective_of_scans_that_end_inside_a_tile():
         ref = O.objective(O.from_problem(P), np.ascontiguousarray(f[off[k]:off[k + 1]]))
         assert each[k] == pytest.approx(ref, rel=1e-12), k
     assert total[1] == pytest.approx(sum(e[1] for e in each), rel=1e-12)
+
+
+# sites of one bin, of a warp's 32 less and more one, with edges on every side; fewer and more sites than
+# a block's warps. The TV terms are FP64 sums of one differenced value each: the same 1e-12.
+@pytest.mark.parametrize("per_bin", [False, True])
+@pytest.mark.parametrize("n_dirs,w", [(2, [0.7, 1.4]), (4, [0.5, 1.3, 2.0, 0.7])])
+@pytest.mark.parametrize("shape", [(1, 3, 1), (3, 5, 31), (9, 7, 33), (40, 33, 65)])
+def test_tv_terms_at_site_and_bin_edges(shape, n_dirs, w, per_bin):
+    J = shape[0] * shape[1] * shape[2]
+    P = scan(max(4, J // 3), 3, shape)
+    op = O.from_problem(P, n_dirs=n_dirs, w=w, per_bin=per_bin)
+    flags = sgtv.FLAG_NO_AUTOTUNE | (sgtv.FLAG_STANDARD_TV if per_bin else 0)
+    with sgtv.Handle(P, n_dirs=n_dirs, w=w, flags=flags) as h:
+        h.iterate(3)
+        f, d, c = h.get_state_f64()
+        tv = h.objective()[2]
+        primal = h.residuals()[0]
+    assert tv == pytest.approx(O.objective(op, f)[2], rel=1e-12)
+    assert primal == pytest.approx(O.residuals(op, f, d, c)[0], rel=1e-12)
