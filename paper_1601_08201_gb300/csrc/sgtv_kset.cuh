@@ -54,6 +54,26 @@ struct Back {
     }
 };
 
+// Both products with eight lanes per segment (FP64).
+template <typename V>
+struct Group8 {
+    static constexpr int kSegs = kG8Threads / 8;
+    static void forward(const Dev &d, const void *f, void *ratio, cudaStream_t st)
+    {
+        k_forward_g8<V><<<unsigned((d.I + kSegs - 1) / kSegs), kG8Threads, 0, st>>>(
+            d.I, d.rowptr, d.col, static_cast<const V *>(d.rval), static_cast<const double *>(f),
+            static_cast<const double *>(d.r), d.r_scalar, static_cast<const double *>(d.y),
+            static_cast<double *>(ratio));
+    }
+    static void back(const Dev &d, const Geom &g, const void *f, void *f_new, cudaStream_t st)
+    {
+        k_back_update_g8<V><<<unsigned((d.J + kSegs - 1) / kSegs), kG8Threads, 0, st>>>(
+            g, d.colptr, d.row, static_cast<const V *>(d.cval), static_cast<const double *>(d.ratio),
+            static_cast<const double *>(d.s), static_cast<const double *>(f), static_cast<const double *>(d.d),
+            static_cast<const double *>(d.c), static_cast<double *>(f_new));
+    }
+};
+
 // Launch a TLI kernel with `smem` bytes of dynamic shared memory, raising the
 // kernel's opt-in limit the first time a launch needs more than 48 KB.
 template <typename K>
@@ -525,6 +545,8 @@ struct Impl {
         k.fwd[n] = FwdTma<T, V, 4, 16>::launch;  k.fwd_name[n] = "tma_ns4_w16"; k.fwd_need[n++] = 4;
         if constexpr (sizeof(T) == 4) {
             k.fwd[n] = RowsStack<V, true>::forward; k.fwd_name[n] = "stack_v4"; k.fwd_need[n++] = 2;
+        } else {
+            k.fwd[n] = Group8<V>::forward; k.fwd_name[n++] = "lanes8";
         }
         k.n_fwd = n;
         n = 0;
@@ -547,6 +569,8 @@ struct Impl {
         k.back[n] = BackTma<T, V, 4, 16>::launch;  k.back_name[n] = "tma_ns4_w16"; k.back_need[n++] = 4;
         if constexpr (sizeof(T) == 4) {
             k.back[n] = back_stack; k.back_name[n] = "stack_v4"; k.back_need[n++] = 2;
+        } else {
+            k.back[n] = Group8<V>::back; k.back_name[n++] = "lanes8";
         }
         k.n_back = n;
         // index = 4 * (register cap) + 2 * (forward 4-wide) + (back 4-wide)
