@@ -490,9 +490,9 @@ k_back_update(Geom g, const int64_t *__restrict__ colptr, const int32_t *__restr
 // segments. The tasks are small and each is one pass through its loads, so
 // that a scan of a few thousand measurements reaches every multiprocessor.
 // 13 x 7 x 37, 3001 measurements (1.7e5 nonzeros): forward 9.7 (the best of the
-// tiled forms) -> 6.0 us, backprojection with f-update 14.3 -> 5.5 us. The
-// set-up's timing chooses: on large scans the FP64 forms that stream through
-// shared memory can still win.
+// tiled forms) -> 6.0 us, backprojection with f-update 14.3 -> 5.5 us; 64^3,
+// 65,536 measurements (3.4e7 nonzeros) 120 -> 108 and 348 -> 239 us. The
+// set-up's timing chooses among these and the tiled forms.
 constexpr int kG8Threads = 64;  // eight segments a block
 
 __device__ __forceinline__ double g8_sum(double v)
