@@ -221,6 +221,26 @@ __device__ __forceinline__ void copy16(float *dst, const float *src)
                  : "memory");
 }
 
+// Two FP32 multiply-adds in one instruction, each rounded as fmaf rounds.
+__device__ __forceinline__ uint64_t fma2(uint64_t a, uint64_t b, uint64_t c)
+{
+    uint64_t d;
+    asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(d) : "l"(a), "l"(b), "l"(c));
+    return d;
+}
+__device__ __forceinline__ uint64_t twice(float x)
+{
+    uint64_t d;
+    asm("mov.b64 %0, {%1, %1};" : "=l"(d) : "f"(x));
+    return d;
+}
+__device__ __forceinline__ float2 halves(uint64_t a)
+{
+    float2 v;
+    asm("mov.b64 {%0, %1}, %2;" : "=f"(v.x), "=f"(v.y) : "l"(a));
+    return v;
+}
+
 template <int G, int WARPS, bool RELU, bool MASK>
 __global__ void __launch_bounds__(32 * WARPS, G == 2 ? 16 / WARPS : 20 / WARPS)
 k_conv_fma(const float *__restrict__ x, const float *__restrict__ wq, const float *__restrict__ b,
@@ -260,13 +280,13 @@ k_conv_fma(const float *__restrict__ x, const float *__restrict__ wq, const floa
             copy16(tw + 4 * k, wc + size_t(k / (kCo / 4)) * cop + k % (kCo / 4) * 4);
         asm volatile("cp.async.commit_group;" ::: "memory");
     };
-    float acc[G][8][4];
+    uint64_t acc[G][4][4];  // output channels 2 o and 2 o + 1
 #pragma unroll
     for (int g = 0; g < G; g++)
 #pragma unroll
-        for (int o = 0; o < 8; o++)
+        for (int o = 0; o < 4; o++)
 #pragma unroll
-            for (int q = 0; q < 4; q++) acc[g][o][q] = 0.f;
+            for (int q = 0; q < 4; q++) acc[g][o][q] = 0;
     stage(0, smf);
     int buf = 0;
 #pragma unroll 1
@@ -285,26 +305,27 @@ k_conv_fma(const float *__restrict__ x, const float *__restrict__ wq, const floa
         for (int c = 0; c < nc; c++) {
 #pragma unroll
             for (int kh = 0; kh < 3; kh++) {
-                float xv[G][6];
+                uint64_t xv[G][6];
 #pragma unroll
                 for (int g = 0; g < G; g++) {
                     const float *p = xb + c * kPlane + kh * kFmaPitch + 8 * g;
                     const float4 v = *reinterpret_cast<const float4 *>(p);
                     const float2 u = *reinterpret_cast<const float2 *>(p + 4);
-                    xv[g][0] = v.x; xv[g][1] = v.y; xv[g][2] = v.z; xv[g][3] = v.w;
-                    xv[g][4] = u.x; xv[g][5] = u.y;
+                    xv[g][0] = twice(v.x); xv[g][1] = twice(v.y); xv[g][2] = twice(v.z); xv[g][3] = twice(v.w);
+                    xv[g][4] = twice(u.x); xv[g][5] = twice(u.y);
                 }
 #pragma unroll
                 for (int kw = 0; kw < 3; kw++) {
                     const float *p = wb + (c * 9 + kh * 3 + kw) * kCo;
-                    const float4 wa = *reinterpret_cast<const float4 *>(p), wd = *reinterpret_cast<const float4 *>(p + 4);
-                    const float wv[8] = {wa.x, wa.y, wa.z, wa.w, wd.x, wd.y, wd.z, wd.w};
+                    const ulonglong2 wa = *reinterpret_cast<const ulonglong2 *>(p);
+                    const ulonglong2 wd = *reinterpret_cast<const ulonglong2 *>(p + 4);
+                    const uint64_t wv[4] = {wa.x, wa.y, wd.x, wd.y};
 #pragma unroll
                     for (int g = 0; g < G; g++)
 #pragma unroll
-                        for (int o = 0; o < 8; o++)
+                        for (int o = 0; o < 4; o++)
 #pragma unroll
-                            for (int q = 0; q < 4; q++) acc[g][o][q] = fmaf(wv[o], xv[g][q + kw], acc[g][o][q]);
+                            for (int q = 0; q < 4; q++) acc[g][o][q] = fma2(wv[o], xv[g][q + kw], acc[g][o][q]);
                 }
             }
         }
@@ -322,12 +343,15 @@ k_conv_fma(const float *__restrict__ x, const float *__restrict__ wq, const floa
         for (int g = 0; g < G; g++) {
             const int ww = w0 + c4 + 8 * g;
             const size_t at = (size_t(n) * Co + co) * HW + hh * W + ww;
+            float sum[4];
+#pragma unroll
+            for (int q = 0; q < 4; q++) sum[q] = (o & 1) ? halves(acc[g][o / 2][q]).y : halves(acc[g][o / 2][q]).x;
             if ((W & 3) == 0) {  // a lane's four pixels are one aligned word
                 if (ww >= W) continue;
                 float r[4];
 #pragma unroll
                 for (int q = 0; q < 4; q++) {
-                    r[q] = acc[g][o][q] + bias;
+                    r[q] = sum[q] + bias;
                     if (RELU) r[q] = r[q] > 0.f ? r[q] : 0.f;
                 }
                 if (MASK) {
@@ -343,7 +367,7 @@ k_conv_fma(const float *__restrict__ x, const float *__restrict__ wq, const floa
 #pragma unroll
             for (int q = 0; q < 4; q++) {
                 if (ww + q >= W) break;
-                float r = acc[g][o][q] + bias;
+                float r = sum[q] + bias;
                 if (RELU) r = r > 0.f ? r : 0.f;
                 if (MASK) r = mask[at + q] > 0.f ? r : 0.f;
                 y[at + q] = r;
@@ -362,83 +386,107 @@ k_conv_fma(const float *__restrict__ x, const float *__restrict__ wq, const floa
 // thread one 8-byte and at most nine 16-byte loads, mostly broadcasts, for 72
 // multiply-adds. Bound: the FP32 pipes.
 constexpr int kWgRows = 8, kWgCo = 64, kWgCi = 16, kWgPitchX = kWgCi + 4, kWgPitchD = kWgCo + 4;
-constexpr int kWgSmem = 4 * ((kWgRows + 2) * 18 * kWgPitchX + kWgRows * 16 * kWgPitchD);
+constexpr int kWgStage = (kWgRows + 2) * 18 * kWgPitchX + kWgRows * 16 * kWgPitchD;  // floats
 
-__global__ void __launch_bounds__(128, 4)
+__global__ void __launch_bounds__(128, 2)
 k_conv_wgrad(const float *__restrict__ x, const float *__restrict__ dy, float *__restrict__ dw,
              float *__restrict__ db, int Ci, int Co, int H, int W)
 {
-    extern __shared__ __align__(16) float smw[];
-    float *const xs = smw, *const ds = smw + (kWgRows + 2) * 18 * kWgPitchX;  // [pixel with halo][ci], [pixel][co]
+    extern __shared__ __align__(16) float smw[];  // one or two stages: x [pixel with halo][ci], dy [pixel][co]
+    constexpr int kPix = (kWgRows + 2) * 18, kXs = kPix * kWgPitchX;
     const int co0 = blockIdx.x * kWgCo, ci0 = blockIdx.y * kWgCi;
     const int bands = (H + kWgRows - 1) / kWgRows;
     const int n = int(blockIdx.z) / bands, h0 = int(blockIdx.z) % bands * kWgRows;
     const int cq = threadIdx.x & 3, cp = threadIdx.x >> 2;  // input channels 4 cq .. + 3, output channels 2 cp, + 1
     const int HW = H * W;
     const float *xn = x + (size_t(n) * Ci + ci0) * HW, *dn = dy + (size_t(n) * Co + co0) * HW;
-    float acc[2][4][9];
+    // a warp copies 8 pixels x 4 channels at a time: 32-byte runs, every bank once
+    const int pl = threadIdx.x & 7, ch = threadIdx.x >> 5 << 2 | ((threadIdx.x >> 3) & 3);
+    auto stage = [&](int w0, float *to) {
+        const bool live = ci0 + ch < Ci;
+        const float *xc = live ? xn + size_t(ch) * HW : x;
+#pragma unroll 4
+        for (int p = pl; p < kPix; p += 8) {
+            const int gy = h0 + p / 18 - 1, gx = w0 + p % 18 - 1;
+            const bool in = live && gy >= 0 && gy < H && gx >= 0 && gx < W;
+            copy4(to + p * kWgPitchX + ch, in ? xc + gy * W + gx : x, in);
+        }
+#pragma unroll 4
+        for (int p = pl; p < kWgRows * 16; p += 8) {
+            const int gy = h0 + p / 16, gx = w0 + p % 16;
+            const bool in = gy < H && gx < W;
+#pragma unroll
+            for (int c = ch; c < ch + kWgCo; c += 16) {
+                const bool ok = in && co0 + c < Co;
+                copy4(to + kXs + p * kWgPitchD + c, ok ? dn + size_t(c) * HW + gy * W + gx : dy, ok);
+            }
+        }
+        asm volatile("cp.async.commit_group;" ::: "memory");
+    };
+    uint64_t acc[2][2][9];  // input channels 2 i and 2 i + 1 of the four
 #pragma unroll
     for (int o = 0; o < 2; o++)
 #pragma unroll
-        for (int i = 0; i < 4; i++)
+        for (int i = 0; i < 2; i++)
 #pragma unroll
-            for (int k = 0; k < 9; k++) acc[o][i][k] = 0.f;
+            for (int k = 0; k < 9; k++) acc[o][i][k] = 0;
     float db0 = 0.f, db1 = 0.f;
+    stage(0, smw);
+    int buf = 0;
 #pragma unroll 1
     for (int w0 = 0; w0 < W; w0 += 16) {
-        __syncthreads();  // the last tile has been read
-        for (int k = threadIdx.x; k < (kWgRows + 2) * 18 * (kWgCi / 4); k += 128) {
-            const int q = k / ((kWgRows + 2) * 18), p = k % ((kWgRows + 2) * 18);
-            const int gy = h0 + p / 18 - 1, gx = w0 + p % 18 - 1;
-            const bool in = gy >= 0 && gy < H && gx >= 0 && gx < W;
-            float v[4];
-#pragma unroll
-            for (int m = 0; m < 4; m++)
-                v[m] = (in && ci0 + 4 * q + m < Ci) ? __ldg(xn + size_t(4 * q + m) * HW + gy * W + gx) : 0.f;
-            *reinterpret_cast<float4 *>(xs + p * kWgPitchX + 4 * q) = make_float4(v[0], v[1], v[2], v[3]);
-        }
-        for (int k = threadIdx.x; k < kWgRows * 16 * (kWgCo / 4); k += 128) {
-            const int q = k / (kWgRows * 16), p = k % (kWgRows * 16);
-            const int gy = h0 + p / 16, gx = w0 + p % 16;
-            const bool in = gy < H && gx < W;
-            float v[4];
-#pragma unroll
-            for (int m = 0; m < 4; m++)
-                v[m] = (in && co0 + 4 * q + m < Co) ? __ldg(dn + size_t(4 * q + m) * HW + gy * W + gx) : 0.f;
-            *reinterpret_cast<float4 *>(ds + p * kWgPitchD + 4 * q) = make_float4(v[0], v[1], v[2], v[3]);
+        if (w0 + 16 < W) {
+            stage(w0 + 16, smw + (buf ^ 1) * kWgStage);
+            asm volatile("cp.async.wait_group 1;" ::: "memory");
+        } else {
+            asm volatile("cp.async.wait_group 0;" ::: "memory");
         }
         __syncthreads();
+        const float *const xs = smw + buf * kWgStage + 4 * cq, *const ds = smw + buf * kWgStage + kXs + 2 * cp;
 #pragma unroll 1
-        for (int r = 0; r < kWgRows; r++)
-#pragma unroll 4
+        for (int r = 0; r < kWgRows; r++) {
+            const float *const xr = xs + r * 18 * kWgPitchX, *const dr = ds + r * 16 * kWgPitchD;
+            ulonglong2 win[3][3];  // [row][column mod 3] around the pixel
+#pragma unroll
+            for (int c = 0; c < 2; c++)
+#pragma unroll
+                for (int kh = 0; kh < 3; kh++)
+                    win[kh][c] = *reinterpret_cast<const ulonglong2 *>(xr + (kh * 18 + c) * kWgPitchX);
+#pragma unroll
             for (int c = 0; c < 16; c++) {
-                const float2 d = *reinterpret_cast<const float2 *>(ds + (r * 16 + c) * kWgPitchD + 2 * cp);
+                const float2 d = *reinterpret_cast<const float2 *>(dr + c * kWgPitchD);
+#pragma unroll
+                for (int kh = 0; kh < 3; kh++)
+                    win[kh][(c + 2) % 3] = *reinterpret_cast<const ulonglong2 *>(xr + (kh * 18 + c + 2) * kWgPitchX);
                 db0 += d.x;
                 db1 += d.y;
+                const uint64_t d0 = twice(d.x), d1 = twice(d.y);
 #pragma unroll
                 for (int k = 0; k < 9; k++) {
-                    const float4 v = *reinterpret_cast<const float4 *>(
-                        xs + ((r + k / 3) * 18 + c + k % 3) * kWgPitchX + 4 * cq);
-                    acc[0][0][k] = fmaf(d.x, v.x, acc[0][0][k]);
-                    acc[0][1][k] = fmaf(d.x, v.y, acc[0][1][k]);
-                    acc[0][2][k] = fmaf(d.x, v.z, acc[0][2][k]);
-                    acc[0][3][k] = fmaf(d.x, v.w, acc[0][3][k]);
-                    acc[1][0][k] = fmaf(d.y, v.x, acc[1][0][k]);
-                    acc[1][1][k] = fmaf(d.y, v.y, acc[1][1][k]);
-                    acc[1][2][k] = fmaf(d.y, v.z, acc[1][2][k]);
-                    acc[1][3][k] = fmaf(d.y, v.w, acc[1][3][k]);
+                    const ulonglong2 v = win[k / 3][(c + k % 3) % 3];
+                    acc[0][0][k] = fma2(d0, v.x, acc[0][0][k]);
+                    acc[0][1][k] = fma2(d0, v.y, acc[0][1][k]);
+                    acc[1][0][k] = fma2(d1, v.x, acc[1][0][k]);
+                    acc[1][1][k] = fma2(d1, v.y, acc[1][1][k]);
                 }
             }
+        }
+        __syncthreads();  // the next copies go over this buffer
+        buf ^= 1;
     }
     // through shared memory, so that a warp's adds are contiguous in dw
-    __syncthreads();
     float *const out = smw;  // [co][ci][9]
 #pragma unroll
     for (int o = 0; o < 2; o++)
 #pragma unroll
-        for (int i = 0; i < 4; i++)
+        for (int i = 0; i < 2; i++)
 #pragma unroll
-            for (int k = 0; k < 9; k++) out[((2 * cp + o) * kWgCi + 4 * cq + i) * 9 + k] = acc[o][i][k];
+            for (int k = 0; k < 9; k++) {
+                const float2 v = halves(acc[o][i][k]);
+                float *const to = out + ((2 * cp + o) * kWgCi + 4 * cq + 2 * i) * 9 + k;
+                to[0] = v.x;
+                to[9] = v.y;
+            }
     __syncthreads();
     for (int k = threadIdx.x; k < kWgCo * kWgCi * 9; k += 128) {
         const int co = k / (kWgCi * 9), r = k % (kWgCi * 9);
@@ -449,7 +497,7 @@ k_conv_wgrad(const float *__restrict__ x, const float *__restrict__ dy, float *_
         if (co0 + 2 * cp + 1 < Co) atomicAdd(db + co0 + 2 * cp + 1, db1);
     }
 }
-static_assert(kWgSmem >= 4 * kWgCo * kWgCi * 9, "the sums are turned in the staging buffer");
+static_assert(kWgStage >= kWgCo * kWgCi * 9, "the sums are turned in the staging buffer");
 
 // The weights of one layer as k_conv reads them: fragment (co / 16, ci / 16,
 // offset) of 32 lanes x 4 words; lane l's words hold rows l / 4 and l / 4 + 8,
@@ -775,7 +823,7 @@ void conv_bwd(wsnet_t h, const float *x, const float *dy, int l, float *dx, cons
     const Layer &L = h->L[l];
     const dim3 gw(unsigned((L.co + kWgCo - 1) / kWgCo), unsigned((L.ci + kWgCi - 1) / kWgCi),
                   unsigned(N * ((Hh + kWgRows - 1) / kWgRows)));
-    k_conv_wgrad<<<gw, 128, kWgSmem, h->stream>>>(x, dy, h->g + L.woff, h->g + L.boff, L.ci, L.co, Hh, Ww);
+    k_conv_wgrad<<<gw, 128, (Ww > 16 ? 2 : 1) * 4 * kWgStage, h->stream>>>(x, dy, h->g + L.woff, h->g + L.boff, L.ci, L.co, Hh, Ww);
     if (!dx) return;
     const uint32_t *w = h->wp + h->pack.at[2][l];
     if (mask) conv_fma<false, true>(h, dy, w, nullptr, mask, dx, L.co, L.ci, N, Hh, Ww);
@@ -864,7 +912,7 @@ int wsnet_create(wsnet_t *out, int32_t H, int32_t W, int32_t Q, int32_t n_dual, 
         return cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes) == cudaSuccess;
     };
     constexpr int big = 2 * 4 * kFmaStage<2, 8>;
-    if (!opt_in(k_conv_wgrad, kWgSmem) || !opt_in(k_conv_fma<2, 8, true, false>, big) ||
+    if (!opt_in(k_conv_wgrad, 2 * 4 * kWgStage) || !opt_in(k_conv_fma<2, 8, true, false>, big) ||
         !opt_in(k_conv_fma<2, 8, false, true>, big) || !opt_in(k_conv_fma<2, 8, false, false>, big))
         return fail_create(SGTV_ERR_CUDA);
     const size_t P = size_t(h->P);
