@@ -648,12 +648,24 @@ k_mse_head(const float *__restrict__ z, const float *__restrict__ tgt, float *__
     const float inv = 1.0f / float(n);
     for (int64_t c = blockIdx.x; c < NC; c += gridDim.x) {
         const bool img = int(c % Co) < Q;
-        for (int k = threadIdx.x; k < HW; k += blockDim.x) {
-            const float zz = z[c * HW + k];
-            const float diff = (img ? softplus(zz) : zz) - tgt[c * HW + k];
-            const double a = abs_f64(diff);
-            acc = fma(a, a, acc);
-            dz[c * HW + k] = img ? 2.f * diff * inv / (1.f + expf(-zz)) : 2.f * diff * inv;
+        const float *const zc = z + c * HW, *const tc = tgt + c * HW;
+        for (int k0 = threadIdx.x; k0 < HW; k0 += 4 * kT) {
+            float zz[4], tt[4];  // all loads first
+#pragma unroll
+            for (int u = 0; u < 4; u++) {
+                const int k = k0 + u * kT;
+                zz[u] = k < HW ? zc[k] : 0.f;
+                tt[u] = k < HW ? tc[k] : 0.f;
+            }
+#pragma unroll
+            for (int u = 0; u < 4; u++) {
+                const int k = k0 + u * kT;
+                if (k >= HW) break;
+                const float diff = (img ? softplus(zz[u]) : zz[u]) - tt[u];
+                const double a = abs_f64(diff);
+                acc = fma(a, a, acc);
+                dz[c * HW + k] = img ? 2.f * diff * inv / (1.f + expf(-zz[u])) : 2.f * diff * inv;
+            }
         }
     }
     for (int o = 16; o > 0; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
