@@ -404,7 +404,9 @@ struct Impl {
         k_dual_rule<T><<<grid_for(g.S, d.sm_count * 8), kThreads, 0, st>>>(
             g, static_cast<const T *>(d.d), static_cast<T *>(d.c), theta);
     }
-    // Two voxels a thread where that still leaves four blocks a multiprocessor, else one.
+    // Two voxels a thread (their loads in flight together) where that still leaves four blocks a
+    // multiprocessor, else one: 41 x 9 x 54 2.1 us with one and 2.4 with two, 64^3 (262144) 3.9 either way,
+    // 128 x 128 x 64 9.8 and 9.2.
     template <int ND, bool PART>
     static void fupdate_nd(const Dev &d, const Geom &g, void *e, const void *f, void *f_new, const int32_t *poff,
                            cudaStream_t st)
@@ -484,15 +486,16 @@ struct Impl {
         k_sum_partials<T><<<d.red_blocks, kThreads, 0, st>>>(n, static_cast<const T *>(a), d.part);
         finalize(d.part, d.red_blocks, 1, 0u, d.red + slot, st);
     }
-    // Tiled wherever the largest tile's f fits in 24 KB as FP64 (two blocks' worth of staging next
-    // to the row sums keeps at least 4 blocks on an SM): list tiles and short windows. Wide windows
-    // (small problems whose tiles span most of the image) read f from L2 in the plain form.
+    // Tiled wherever the largest tile's f fits in 31 KB as FP64 (with 16.75 KB of row sums within the 48 KB
+    // that a block has without asking): list tiles and short windows. 60,000 rows, staging 20 KB: 38 us, plain 59; 27 KB:
+    // 42 and 59; 31 KB: 40 and 59; 64^3 (2 KB) 150 and 459. Wide windows (small problems whose tiles span most of the image)
+    // read f from L2 in the plain form.
     static void deviance(const Dev &d, const void *f, int64_t i0, int64_t i1, int slot, cudaStream_t st)
     {
         const T *ff = static_cast<const T *>(f), *r = static_cast<const T *>(d.r), *y = static_cast<const T *>(d.y);
         const V *val = static_cast<const V *>(d.rval);
         int blocks = d.red_blocks;
-        if (d.tr.fmt != 0 && d.tr.max_stage * int(sizeof(double)) <= 24 * 1024) {
+        if (d.tr.fmt != 0 && d.tr.max_stage * int(sizeof(double)) <= 31 * 1024) {
             // one partial field is free for up to 4 red_blocks blocks (Dev::part)
             const int64_t tiles = (i1 + kTliTile - 1) / kTliTile - i0 / kTliTile;
             blocks = int(tiles < 4 * int64_t(d.red_blocks) ? (tiles > 0 ? tiles : 1) : 4 * int64_t(d.red_blocks));

@@ -778,7 +778,9 @@ void *walloc(wsnet_t h, size_t bytes)
 }
 
 // Inference: the larger block where it leaves every multiprocessor one of them,
-// the smaller one (a quarter of the work) otherwise.
+// the smaller one (a quarter of the work) otherwise: one sample of 64 x 64 (32
+// larger blocks a layer at full size) 241 us for the nine layers with the
+// larger block, 114 with the smaller; eight samples (256) 29.2 and 29.5 a layer.
 template <bool RELU>
 void conv_tc(wsnet_t h, const float *x, int l, float *y, int N, int Hh, int Ww)
 {
@@ -795,8 +797,12 @@ void conv_tc(wsnet_t h, const float *x, int l, float *y, int N, int Hh, int Ww)
     k_conv<2, 2, 4, RELU><<<small, 128, 0, h->stream>>>(x, w, b, y, L.ci, L.co, Hh, Ww);
 }
 
-// Training: 64 channels of 16 x 16 pixels a block where that gives every
-// multiprocessor about one, else 32 channels of 8 x 16.
+// Training: 64 channels of 16 x 16 pixels a block, or 32 channels of 8 x 16. A
+// multiprocessor takes about 51 us for one of the larger blocks at 64 input
+// channels and 14 us for one of the smaller (more staging for a product), so
+// the form whose fullest multiprocessor is done first: 128 larger blocks or
+// 512 smaller 51 or 56 us, 160 or 640 97 or 69, 320 or 1280 143 or 120, 640 or
+// 2560 235 or 222.
 template <bool RELU, bool MASK>
 void conv_fma(wsnet_t h, const float *x, const uint32_t *w, const float *b, const float *mask, float *y, int Ci, int Co,
               int N, int Hh, int Ww)
@@ -804,12 +810,13 @@ void conv_fma(wsnet_t h, const float *x, const uint32_t *w, const float *b, cons
     const unsigned tw = unsigned((Ww + 15) / 16);
     const float *wf = reinterpret_cast<const float *>(w);
     const dim3 big(tw * unsigned((Hh + 15) / 16), unsigned((Co + 63) / 64), unsigned(N));
-    if (4 * uint64_t(big.x) * big.y * big.z >= 3 * unsigned(h->sms)) {
+    const dim3 small(tw * unsigned((Hh + 7) / 8), unsigned((Co + 31) / 32), unsigned(N));
+    auto fullest = [&](const dim3 &g) { return (uint64_t(g.x) * g.y * g.z + h->sms - 1) / h->sms; };
+    if (51 * fullest(big) <= 14 * fullest(small)) {
         k_conv_fma<2, 8, RELU, MASK>
             <<<big, 256, 2 * 4 * kFmaStage<2, 8>, h->stream>>>(x, wf, b, mask, y, Ci, Co, Hh, Ww);
         return;
     }
-    const dim3 small(tw * unsigned((Hh + 7) / 8), unsigned((Co + 31) / 32), unsigned(N));
     k_conv_fma<1, 4, RELU, MASK>
         <<<small, 128, 2 * 4 * kFmaStage<1, 4>, h->stream>>>(x, wf, b, mask, y, Ci, Co, Hh, Ww);
 }

@@ -79,3 +79,15 @@ def test_tv_terms_at_site_and_bin_edges(shape, n_dirs, w, per_bin):
         primal = h.residuals()[0]
     assert tv == pytest.approx(O.objective(op, f)[2], rel=1e-12)
     assert primal == pytest.approx(O.residuals(op, f, d, c)[0], rel=1e-12)
+
+
+# one window that is the image: 3913 columns still staged as FP64, 4004 not
+@pytest.mark.parametrize("precision", ["fp32", "fp64"])
+@pytest.mark.parametrize("Nq", [43, 44])
+def test_objective_at_the_staging_limit(Nq, precision):
+    P = scan(2000, 40, (13, 7, Nq))
+    with sgtv.Handle(P, precision=precision, flags=sgtv.FLAG_NO_AUTOTUNE) as h:
+        h.iterate(2)
+        f = h.get_state_f64()[0]
+        dev = h.objective()[1]
+    assert dev == pytest.approx(O.objective(oracle_of(P, precision), f)[1], rel=1e-12)
