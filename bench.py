@@ -564,8 +564,10 @@ def run_batched(args):
 
 
 FORMS = {
-    "single_pass": "single pass: CSR forward + scatter into e (bank-dealt row stream), elementwise f-update, shrink",
-    "two_pass": "two passes: CSR forward, CSC backprojection fused with the f-update, shrink",
+    "single_pass": "single pass: both products from one read of A by rows (form: k_scatter in tuning), elementwise "
+                   "f-update, shrink",
+    "two_pass": "two-pass handle: CSR forward, CSC backprojection fused with the f-update, shrink (form stack_v4: one "
+                "read of A by rows, partial sums added up by the f-update)",
 }
 
 
@@ -693,7 +695,8 @@ def main():
     it_survey = sum(sb[k] * v[1] for k, v in prof.items()) / args.steps
     roofline = {"bound": "hbm", "kernel": dom, "achieved": achieved, "peak": peak, "unit": "GB/s",
                 "frac": achieved / peak, "peak_source": peak_kind,
-                "bytes_basis": "the kernel's stored format (16-bit local indices, padded rows)",
+                "bytes_basis": "the kernel's stored format (stack: values, bit records, tiles' columns; others: 16-bit local "
+                               "indices, padded rows)",
                 "survey_basis": {"kernel_bytes": sb[dom], "achieved": sb[dom] / (dom_ms / 1e3) / 1e9,
                                  "frac": sb[dom] / (dom_ms / 1e3) / 1e9 / peak,
                                  "iteration_bytes": it_survey,
