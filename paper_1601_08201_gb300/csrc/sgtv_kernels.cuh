@@ -2506,32 +2506,6 @@ __device__ __forceinline__ double dev_term(double yb, double yi)
     return t;
 }
 
-// A value of A as an FP64 factor scaled by 2^-kF64Shift, and that factor's
-// partner, a dense operand scaled by 2^+kF64Shift: their product is the
-// unscaled one, rounded alike. The bits of a nonnegative FP32 (or BF16) value
-// shifted into an FP64 pattern read as that value times 2^(127 - 1023)
-// (subnormals included), so the conversion is two integer instructions. The
-// device's FP64 unit, which a real conversion also occupies, does about 2
-// lanes per clock and SM (0.5 T/s measured for the conversion as for the
-// multiply-add), so the deviance below is bound by it.
-constexpr double kF64Up = 0x1p896;
-__device__ __forceinline__ double f64_scaled(float v)
-{
-    const uint32_t u = __float_as_uint(v);
-    return __hiloint2double(int(u >> 3), int(u << 29));
-}
-// BF16 rounding can reach infinity: it stays one.
-__device__ __forceinline__ double f64_scaled_bf16(float v)
-{
-    const uint32_t u = __float_as_uint(v);
-    return __hiloint2double((u >> 23) == 0xFFu ? int(0x7FF00000u | (u & 0x7FFFFFu) >> 3) : int(u >> 3), 0);
-}
-template <typename V> __device__ __forceinline__ double val_scaled(float v) { return f64_scaled(v); }
-template <> __device__ __forceinline__ double val_scaled<__nv_bfloat16>(float v) { return f64_scaled_bf16(v); }
-template <typename V> __device__ __forceinline__ double val_scaled(double v) { return v; }
-template <typename T> __device__ __forceinline__ double dense_scaled(T x) { return double(x) * kF64Up; }
-template <> __device__ __forceinline__ double dense_scaled<double>(double x) { return x; }
-
 // Deviance partials over the measurements [i0, i1), from the plain CSR form
 // (matrices without tiles, and tiles whose staging would fill an SM): ybar
 // accumulated in FP64 from the stored A values and f. A warp takes 8 rows in
@@ -2566,28 +2540,25 @@ k_dev_partials(int64_t i0, int64_t i1, const int64_t *__restrict__ rowptr, const
     if (threadIdx.x == 0) part[blockIdx.x] = tot;
 }
 
-// The same from the tiled form (16-bit local indices): a block takes tiles
-// blockIdx.x, + gridDim.x, ... that meet [i0, i1), stages the tile's f in
-// shared memory as scaled FP64, and each warp forms 8 rows' products with one
-// FP64 multiply-add per nonzero and no other FP64 work in the loop. The lanes'
-// sums are folded by all 256 threads (a warp-wide tree would take 5 FP64
-// additions per row and lane, as much again as 5/8 of the products), and the
-// 64 terms are formed by 64 threads side by side. The lanes take consecutive
-// elements because an FP64 instruction costs a warp the same for any number
-// of active lanes (4-wide chunks, whose last chunk is mostly empty, took a
-// third more). Bound: the FP64 unit (2^28 nonzeros at 0.5 T/s: 0.53 ms).
-// Measured on that problem: 0.85 ms, against 5.11 ms for the plain form with
-// one row and one lane's term at a time.
-template <typename T, typename V>
+// The same from the tiled form (16-bit local indices), T = double: a block takes
+// tiles blockIdx.x, + gridDim.x, ... that meet [i0, i1), stages the tile's f in
+// shared memory, and each warp forms 8 rows' products with one FP64
+// multiply-add per nonzero and no other FP64 work in the loop. The lanes' sums
+// are folded by all 256 threads (a warp-wide tree would take 5 FP64 additions
+// per row and lane, as much again as 5/8 of the products), and the 64 terms
+// are formed by 64 threads side by side. The lanes take consecutive elements
+// because an FP64 instruction costs a warp the same for any number of active
+// lanes. Bound: the FP64 unit, about 2 lanes per clock and SM.
+template <typename T>
 __global__ void __launch_bounds__(256, 4)
 k_dev_partials_tli(int64_t i0, int64_t i1, int64_t ntiles, const int64_t *__restrict__ rowptr, TliTiles tl,
-                   const V *__restrict__ val, const T *__restrict__ f, const T *__restrict__ r, int r_scalar,
+                   const T *__restrict__ val, const T *__restrict__ f, const T *__restrict__ r, int r_scalar,
                    const T *__restrict__ y, double *__restrict__ part)
 {
     extern __shared__ __align__(128) unsigned char smem_raw[];
     __shared__ double rows[kTliTile][33];
     __shared__ double sh[32];
-    double *xs = reinterpret_cast<double *>(smem_raw);
+    T *xs = reinterpret_cast<T *>(smem_raw);
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     constexpr int R = kTliTile / 8;
     double mine = 0.0;
@@ -2599,7 +2570,7 @@ k_dev_partials_tli(int64_t i0, int64_t i1, int64_t ntiles, const int64_t *__rest
         const int nstage = wl > 0 ? wl : int(tl.uoff[t + 1] - u0);
         const int64_t wb = tl.wbase[t];
         for (int k = threadIdx.x; k < nstage; k += blockDim.x)
-            xs[k] = dense_scaled<T>(f[wl > 0 ? wb + k : int64_t(tl.uidx[u0 + k])]);
+            xs[k] = f[wl > 0 ? wb + k : int64_t(tl.uidx[u0 + k])];
         __syncthreads();
         const int64_t w0 = t0 + warp * R;
         const int n = w0 < t1 ? int(t1 - w0 < R ? t1 - w0 : R) : 0;
@@ -2610,24 +2581,24 @@ k_dev_partials_tli(int64_t i0, int64_t i1, int64_t ntiles, const int64_t *__rest
             double a0 = 0.0, a1 = 0.0;
             const int n_el = int(e - s);  // a row holds at most J < 2^31 nonzeros
             const uint16_t *__restrict__ li = tl.lidx + s;
-            const V *__restrict__ va = val + s;
+            const T *__restrict__ va = val + s;
             for (int p = 0; p < n_el; p += 256) {
                 int32_t c[8];
                 T v[8];
 #pragma unroll
                 for (int u = 0; u < 8; u++) {
                     c[u] = 0;
-                    v[u] = T(0);
+                    v[u] = 0.0;
                     if (p + 32 * u + lane < n_el) {
                         c[u] = ld_idx(li + p + 32 * u + lane);
-                        v[u] = T(ld_val(va + p + 32 * u + lane));
+                        v[u] = ld_val(va + p + 32 * u + lane);
                     }
                 }
 #pragma unroll
                 for (int u = 0; u < 8; u++)
                     if (p + 32 * u < n_el) {  // warp-uniform: no FP64 instruction past the row's end
                         double &a = (u & 1) ? a1 : a0;
-                        if (p + 32 * u + lane < n_el) a = fma(val_scaled<V>(v[u]), xs[c[u]], a);
+                        if (p + 32 * u + lane < n_el) a = fma(v[u], xs[c[u]], a);
                     }
             }
             rows[warp * R + k][lane] = a0 + a1;
@@ -2646,6 +2617,162 @@ k_dev_partials_tli(int64_t i0, int64_t i1, int64_t ntiles, const int64_t *__rest
         const int64_t i = t0 + threadIdx.x;
         if (threadIdx.x < kTliTile && i >= i0 && i < t1)
             mine += dev_term(rows[threadIdx.x][0] + double(r_scalar ? r[0] : r[i]), double(y[i]));
+        __syncthreads();  // rows and xs are rewritten by the next tile
+    }
+    double tot = block_reduce<false>(mine, sh);
+    if (threadIdx.x == 0) part[blockIdx.x] = tot;
+}
+
+// Packed FP32 sums with their rounding errors (Knuth's two-sum): hi + lo is the
+// exact sum, on each half.
+__device__ __forceinline__ uint64_t add2(uint64_t a, uint64_t b)
+{
+    uint64_t d;
+    asm("add.rn.f32x2 %0, %1, %2;" : "=l"(d) : "l"(a), "l"(b));
+    return d;
+}
+__device__ __forceinline__ uint64_t sub2(uint64_t a, uint64_t b)
+{
+    return fma2(b, pack2(-1.f, -1.f), a);  // exact product: rounds as a - b
+}
+__device__ __forceinline__ uint64_t two_sum2(uint64_t a, uint64_t b, uint64_t &lo)
+{
+    const uint64_t t = add2(a, b), bb = sub2(t, a);
+    lo = add2(sub2(a, sub2(t, bb)), sub2(b, bb));
+    return t;
+}
+__device__ __forceinline__ float two_sum(float a, float b, float &lo)
+{
+    const float t = __fadd_rn(a, b), bb = __fsub_rn(t, a);
+    lo = __fadd_rn(__fsub_rn(a, __fsub_rn(t, bb)), __fsub_rn(b, bb));
+    return t;
+}
+
+// The same for FP32 images, without the FP64 unit in the loop: a product is
+// the exact sum of two FP32 numbers (a multiplication and a multiply-add), and
+// a row's sum three FP32 numbers, each taking the rounding errors of the one
+// before; what is lost is about 2^-70 of it, where a chain of FP64 sums loses
+// 2^-53 per step. Two rows at a time, one in each half of the packed
+// instructions: 23 of them for two products, at 64 times the FP64 unit's rate.
+// A row for which that may not be so (a product that overflows FP32, or may have
+// underflowed next to a ybar as small) is summed again in FP64. Bound:
+// issue in the loop (2^28 nonzeros: 0.2 ms) and the 64 divisions and logarithms
+// a tile, which are FP64 (0.1 to 0.2 ms beside it). Against the loop with one
+// FP64 multiply-add per nonzero (and a plain one with a row at a time): 2^28
+// nonzeros, 256 a row, 0.86 -> 0.62 ms (5.11), 64^3 with 128 a row 168 -> 112
+// us; the same error against extended precision (at most 2e-16 of the sum).
+template <typename V>
+__global__ void __launch_bounds__(256, 4)
+k_dev_partials_tl3(int64_t i0, int64_t i1, int64_t ntiles, const int64_t *__restrict__ rowptr, TliTiles tl,
+                   const V *__restrict__ val, const float *__restrict__ f, const float *__restrict__ r, int r_scalar,
+                   const float *__restrict__ y, double *__restrict__ part)
+{
+    extern __shared__ __align__(128) unsigned char smem_raw[];
+    __shared__ float rows[3][kTliTile][33];
+    __shared__ double sum[kTliTile];
+    __shared__ double sh[32];
+    float *xs = reinterpret_cast<float *>(smem_raw);
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    constexpr int R = kTliTile / 8;
+    double mine = 0.0;
+    for (int64_t t = i0 / kTliTile + blockIdx.x; t < ntiles && t * kTliTile < i1; t += gridDim.x) {
+        const int64_t t0 = t * kTliTile, t1 = t0 + kTliTile < i1 ? t0 + kTliTile : i1;
+        if (threadIdx.x == 0) prefetch_segments_l2(rowptr, t0, t1, tl.lidx, val);
+        const int wl = tl.wlen[t];
+        const int64_t u0 = tl.uoff[t];
+        const int nstage = wl > 0 ? wl : int(tl.uoff[t + 1] - u0);
+        const int64_t wb = tl.wbase[t];
+        for (int k = threadIdx.x; k < nstage; k += blockDim.x)
+            xs[k] = f[wl > 0 ? wb + k : int64_t(tl.uidx[u0 + k])];
+        __syncthreads();
+        const int64_t w0 = t0 + warp * R;
+        const int n = w0 < t1 ? int(t1 - w0 < R ? t1 - w0 : R) : 0;
+        const int64_t bound = lane <= n && n > 0 ? rowptr[w0 + lane] : 0;
+#pragma unroll 1
+        for (int k = 0; k < n; k += 2) {
+            const int64_t sa = __shfl_sync(0xffffffffu, bound, k), sb = __shfl_sync(0xffffffffu, bound, k + 1);
+            const int64_t se = __shfl_sync(0xffffffffu, bound, k + 2 <= n ? k + 2 : k + 1);
+            const int na = int(sb - sa), nb = int(se - sb);  // the second row: none at an odd end
+            const uint16_t *__restrict__ la = tl.lidx + sa, *__restrict__ lb = tl.lidx + sb;
+            const V *__restrict__ va = val + sa, *__restrict__ vb = val + sb;
+            uint64_t s0 = 0, s1 = 0, s2 = 0;
+            for (int p = 0; p < na || p < nb; p += 128) {
+                int32_t ca[4], cb[4];
+                float x[4], z[4];
+#pragma unroll
+                for (int u = 0; u < 4; u++) {
+                    const int q = p + 32 * u + lane;
+                    ca[u] = cb[u] = 0;
+                    x[u] = z[u] = 0.f;
+                    if (q < na) {
+                        ca[u] = ld_idx(la + q);
+                        x[u] = ld_val(va + q);
+                    }
+                    if (q < nb) {
+                        cb[u] = ld_idx(lb + q);
+                        z[u] = ld_val(vb + q);
+                    }
+                }
+#pragma unroll
+                for (int u = 0; u < 4; u++) {
+                    const int q0 = p + 32 * u;
+                    if (q0 >= na && q0 >= nb) break;  // warp-uniform
+                    const int q = q0 + lane;
+                    const uint64_t a = pack2(x[u], z[u]);
+                    const uint64_t b = pack2(q < na ? xs[ca[u]] : 0.f, q < nb ? xs[cb[u]] : 0.f);
+                    const uint64_t w = fma2(a, b, pack2(-0.f, -0.f));
+                    const uint64_t e = fma2(a, b, sub2(pack2(-0.f, -0.f), w));  // a b = w + e
+                    uint64_t l0, l1, l2;
+                    s0 = two_sum2(s0, w, l0);
+                    s1 = two_sum2(s1, l0, l1);
+                    s1 = two_sum2(s1, e, l2);
+                    s2 = add2(s2, add2(l1, l2));
+                }
+            }
+            const uint64_t s[3] = {s0, s1, s2};
+#pragma unroll
+            for (int m = 0; m < 3; m++) {
+                float u, v;
+                asm("mov.b64 {%0, %1}, %2;" : "=f"(u), "=f"(v) : "l"(s[m]));
+                rows[m][warp * R + k][lane] = u;
+                if (k + 1 < n) rows[m][warp * R + k + 1][lane] = v;
+            }
+        }
+        __syncthreads();
+        // 4 threads per row: 8 lanes' sums each, then the quad's total
+        const int rr = threadIdx.x >> 2, qd = threadIdx.x & 3;
+        float a0 = 0.f, a1 = 0.f, a2 = 0.f;
+#pragma unroll
+        for (int m = 0; m < 8; m++) {
+            float l0, l1, l2;
+            a0 = two_sum(a0, rows[0][rr][qd + 4 * m], l0);
+            a1 = two_sum(a1, l0, l1);
+            a1 = two_sum(a1, rows[1][rr][qd + 4 * m], l2);
+            a2 += (l1 + l2) + rows[2][rr][qd + 4 * m];
+        }
+        double yb = double(a0) + (double(a1) + double(a2));
+        yb += __shfl_xor_sync(0xffffffffu, yb, 1);
+        yb += __shfl_xor_sync(0xffffffffu, yb, 2);
+        if (qd == 0) sum[rr] = yb;
+        __syncthreads();
+        const int64_t i = t0 + threadIdx.x;
+        if (threadIdx.x < kTliTile) {  // whole warps
+            const bool in = i >= i0 && i < t1;
+            const double ri = in ? double(r_scalar ? r[0] : r[i]) : 1.0;
+            double ab = in ? sum[threadIdx.x] : 0.0;
+            // what underflowed is below 2^-149 a product; NaN fails too
+            uint32_t again = __ballot_sync(0xffffffffu, !(fabs(ab + ri) > 0x1p-60 && fabs(ab) < 0x1p100));
+            for (; again != 0u; again &= again - 1u) {
+                const int k = __ffs(again) - 1;
+                const int64_t row = t0 + 32 * warp + k;
+                double acc = 0.0;
+                for (int64_t p = rowptr[row] + lane; p < rowptr[row + 1]; p += 32)
+                    acc = fma(double(ld_val(val + p)), double(xs[ld_idx(tl.lidx + p)]), acc);
+                acc = warp_sum_d(acc);
+                if (lane == k) ab = acc;
+            }
+            if (in) mine += dev_term(ab + ri, double(y[i]));
+        }
         __syncthreads();  // rows and xs are rewritten by the next tile
     }
     double tot = block_reduce<false>(mine, sh);

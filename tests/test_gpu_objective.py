@@ -91,3 +91,21 @@ def test_objective_at_the_staging_limit(Nq, precision):
         f = h.get_state_f64()[0]
         dev = h.objective()[1]
     assert dev == pytest.approx(O.objective(oracle_of(P, precision), f)[1], rel=1e-12)
+
+
+# images whose products with A leave FP32's range (some rows, or all), or are subnormal, and ordinary ones;
+# odd numbers of rows per warp and rows of more than 128 nonzeros
+@pytest.mark.parametrize("precision", ["fp32", "bf16"])
+@pytest.mark.parametrize("scale", [1e-44, 1e-38, 1e-22, 1.0, 1e28, 1e36])
+@pytest.mark.parametrize("mixed", [False, True])
+def test_deviance_of_images_at_the_ends_of_fp32(scale, mixed, precision):
+    P = scan(331, 90, (8, 6, 16))
+    rng = np.random.default_rng(3)
+    f = (rng.uniform(0.5, 2.0, P.J) * scale).astype(np.float32)
+    if mixed:
+        f[::2] = rng.uniform(0.5, 2.0, f[::2].size)
+    f = f.astype(np.float64)
+    with sgtv.Handle(P, precision=precision, flags=sgtv.FLAG_NO_AUTOTUNE) as h:
+        h.set_state_f64(f)
+        dev = h.objective()[1]
+    assert dev == pytest.approx(O.objective(oracle_of(P, precision), f)[1], rel=1e-12)
