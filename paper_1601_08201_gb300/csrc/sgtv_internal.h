@@ -90,6 +90,14 @@ constexpr int stk_rec_bytes(int words) { return words <= kStkShortWords ? 4 : 8;
 // 20 words 16 blocks without spills and 18 with a few take the same time, 22
 // half as much again).
 constexpr int stk_min_blocks(int words) { return words <= 8 ? 28 : (words <= 12 ? 24 : (words <= 20 ? 18 : 16)); }
+// What the kernel is compiled for: up to 12 words the 28 blocks that it reaches without spills or nearly so (left to
+// itself the allocator takes 3 registers more in some instantiations, which costs 4 blocks: 64^3 with 160 a row 52.4
+// -> 55.8 us); with partial sums and 19 words or more 16 blocks without spills (2^28 nonzeros 278 -> 263 us; without
+// partial sums 79 -> 83 on 2^26, so not there).
+constexpr int stk_resident(int words, bool part)
+{
+    return words <= 12 ? 28 : (part && words > 18 ? 16 : stk_min_blocks(words));
+}
 struct StackMat {
     int built;
     int tr;               // rows per tile

@@ -16,6 +16,7 @@
 
 #include <cuda_bf16.h>
 #include <cuda_runtime.h>
+#include <float.h>
 #include <stdint.h>
 
 #include <type_traits>
@@ -2100,7 +2101,14 @@ k_back_update_tma(TmaMat m, TmaLayout L, Geom g, const V *__restrict__ val, cons
 // nonzero costs neither a gather nor a scatter: per row and word a lane tests
 // its bit, reads the next value of its stack from the ring if it is set, and
 // two packed FP32 multiply-adds (one per word pair in the product, one in the
-// sums) take two words at once; words without a nonzero add 0.
+// sums) take two words at once; words without a nonzero add 0 times the image
+// in the product and 0 times the ratio in the sums. That is 0 only for finite
+// factors: an infinite ratio (a count where A f + r is 0, or y / ybar past FP32)
+// or image value has to reach the row's own columns and no other. The loop does
+// not look: a ratio that is not finite, which an image value that is not finite
+// makes of every row of the tile with a count, leaves every sum of the tile
+// infinite or NaN, so one sum a lane is looked at when the tile is done, and such
+// a tile is done again over its nonzeros alone (stk_redo).
 //
 // The row stream it replaces as the first choice (k_scatter_sp) is bound by
 // instruction issue: 12.4 warp instructions per 32 nonzeros for the gather,
@@ -2195,8 +2203,91 @@ __device__ __forceinline__ bool mbar_try(uint32_t bar, uint32_t parity)
     return done != 0;
 }
 
+// Tile t again, nonzero by nonzero from global memory, its sums in the ring's
+// place (at least 2 W + kStkMirror levels of 32 V: room for W of 32 floats). Bound
+// by the latency of its loads, kRedo words of them in flight, some
+// 1.3 us a row of 20 words: a pass over 2^26 nonzeros takes 80 us, 164 where one
+// tile is done again, 565 where all are.
+template <typename V, typename M, int W, bool PART>
+__device__ __forceinline__ void stk_redo(int64_t I, int64_t t, const StackMat &m, float *sum,
+                                         const float *__restrict__ f, const float *__restrict__ r, int r_scalar,
+                                         const float *__restrict__ y, float *__restrict__ out,
+                                         float *__restrict__ ratio)
+{
+    static_assert((2 * W + kStkMirror) * sizeof(V) >= W * sizeof(float), "the sums are kept in the ring's place");
+    static_assert(kStkMaxRows <= 64, "a lane per pair of rows");
+    constexpr int kRedo = W % 5 == 0 ? 5 : (W % 6 == 0 ? 6 : (W % 4 == 0 ? 4 : 2));
+    const int lane = threadIdx.x;
+    const int64_t r0 = t * m.tr;
+    const int n = int(I - r0 < m.tr ? I - r0 : m.tr);
+    const V *__restrict__ val = static_cast<const V *>(m.val) + m.lvl[t] * 32;
+    const M *__restrict__ rec = static_cast<const M *>(m.rec) + (r0 >> 1) * 32 + lane;
+    const int32_t *__restrict__ cols = m.uidx + (t * W) * 32 + lane;
+    const int32_t *__restrict__ dst = PART ? m.ppos + (t * W) * 32 + lane : cols;
+    int top = 2 * lane < n ? int((m.ctl[(r0 >> 1) + lane] >> 7) & 63u) : 0;  // of pair `lane`: levels up to its last
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+        const int below = __shfl_up_sync(0xffffffffu, top, o);
+        if (lane >= o) top += below;
+    }
+    __syncwarp();
+#pragma unroll 1
+    for (int w = 0; w < W; w++) sum[32 * w + lane] = 0.f;
+    M next = rec[0];
+#pragma unroll 1
+    for (int k = 0; k < n; k++) {
+        const int first = __shfl_sync(0xffffffffu, top, k >> 1) - m.ring;  // the pair's values lie from here on
+        const M now = next;
+        if (k + 1 < n) next = rec[((k + 1) >> 1) * 32];
+        const float yi = y[r0 + k], ri = r[r_scalar ? 0 : r0 + k];
+        uint32_t a, b, at;
+        stk_split(now, a, b, at);
+        const uint32_t all = (1u << W) - 1u, mk = (k & 1 ? b : a) & all;
+        const int place = int(at >> 5);
+        const int level = first + ((place - first) % m.ring + m.ring) % m.ring + (k & 1 ? __popc(a & all) : 0);
+        // a lane without values in the row reads the tile's first ones and drops them
+        const V *__restrict__ v = val + (mk != 0u ? int64_t(level) * 32 + (at & 31u) : 0);
+        float s = 0.f;
+#pragma unroll 1
+        for (int w0 = 0; w0 < W; w0 += kRedo) {
+            float x[kRedo], z[kRedo];
+#pragma unroll
+            for (int u = 0; u < kRedo; u++) {
+                const bool in = (mk >> (w0 + u)) & 1u;
+                x[u] = float(v[in ? 32 * __popc(mk & ((1u << (w0 + u)) - 1u)) : 0]);
+                z[u] = f[in ? cols[32 * (w0 + u)] : 0];
+            }
+#pragma unroll
+            for (int u = 0; u < kRedo; u++)
+                if ((mk >> (w0 + u)) & 1u) s = fmaf(x[u], z[u], s);
+        }
+        const float q = yi != 0.f ? yi / (warp_sum(s) + ri) : 0.f;
+        if (PART && lane == 0) ratio[r0 + k] = q;
+#pragma unroll 1
+        for (int w0 = 0; w0 < W && q != 0.f; w0 += kRedo) {  // warp-uniform
+            float x[kRedo], z[kRedo];
+#pragma unroll
+            for (int u = 0; u < kRedo; u++) {
+                x[u] = float(v[(mk >> (w0 + u)) & 1u ? 32 * __popc(mk & ((1u << (w0 + u)) - 1u)) : 0]);
+                z[u] = sum[32 * (w0 + u) + lane];
+            }
+#pragma unroll
+            for (int u = 0; u < kRedo; u++)
+                if ((mk >> (w0 + u)) & 1u) sum[32 * (w0 + u) + lane] = fmaf(x[u], q, z[u]);
+        }
+    }
+#pragma unroll 1
+    for (int w = 0; w < W; w++) {
+        const int32_t to = dst[32 * w];
+        const float a = sum[32 * w + lane];
+        if (to < 0) continue;
+        if (PART) out[to] = a;
+        else if (a != 0.f) atomicAdd(out + to, a);
+    }
+}
+
 template <typename V, int W, bool PART>
-__global__ void __launch_bounds__(32, stk_min_blocks(W))
+__global__ void __launch_bounds__(32, stk_resident(W, PART))
 k_rows_stack(int64_t I, StackMat m, const float *__restrict__ f, const float *__restrict__ r, int r_scalar,
              const float *__restrict__ y, float *__restrict__ out, float *__restrict__ ratio, int *__restrict__ flag)
 {
@@ -2345,7 +2436,12 @@ k_rows_stack(int64_t I, StackMat m, const float *__restrict__ f, const float *__
         }
         return;
     }
-    const int32_t *__restrict__ dst = PART ? m.ppos + (t * W) * 32 + lane : cols;
+    uint32_t tile;  // read anew: no address is kept through the loop for what follows
+    asm volatile("mov.u32 %0, %%ctaid.x;" : "=r"(tile));
+    float sum0, sum1;
+    unpack2(acc[0], sum0, sum1);
+    if (__builtin_expect(__all_sync(0xffffffffu, sum0 <= FLT_MAX), 1)) {  // the sums are >= 0 or NaN
+    const int32_t *__restrict__ dst = (PART ? m.ppos : m.uidx) + (int64_t(tile) * W) * 32 + lane;
 #pragma unroll
     for (int w = 0; w < W / 2; w++) {
         float a, b;
@@ -2358,6 +2454,9 @@ k_rows_stack(int64_t I, StackMat m, const float *__restrict__ f, const float *__
             if (ia >= 0 && a != 0.f) atomicAdd(out + ia, a);
             if (ib >= 0 && b != 0.f) atomicAdd(out + ib, b);
         }
+    }
+    } else {
+        stk_redo<V, M, W, PART>(I, tile, m, reinterpret_cast<float *>(smem_raw), f, r, r_scalar, y, out, ratio);
     }
 }
 
