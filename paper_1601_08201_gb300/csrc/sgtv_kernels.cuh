@@ -2441,20 +2441,20 @@ k_rows_stack(int64_t I, StackMat m, const float *__restrict__ f, const float *__
     float sum0, sum1;
     unpack2(acc[0], sum0, sum1);
     if (__builtin_expect(__all_sync(0xffffffffu, sum0 <= FLT_MAX), 1)) {  // the sums are >= 0 or NaN
-    const int32_t *__restrict__ dst = (PART ? m.ppos : m.uidx) + (int64_t(tile) * W) * 32 + lane;
+        const int32_t *__restrict__ dst = (PART ? m.ppos : m.uidx) + (int64_t(tile) * W) * 32 + lane;
 #pragma unroll
-    for (int w = 0; w < W / 2; w++) {
-        float a, b;
-        unpack2(acc[w], a, b);
-        const int32_t ia = __ldg(dst + 64 * w), ib = __ldg(dst + 64 * w + 32);
-        if (PART) {
-            if (ia >= 0) out[ia] = a;
-            if (ib >= 0) out[ib] = b;
-        } else {
-            if (ia >= 0 && a != 0.f) atomicAdd(out + ia, a);
-            if (ib >= 0 && b != 0.f) atomicAdd(out + ib, b);
+        for (int w = 0; w < W / 2; w++) {
+            float a, b;
+            unpack2(acc[w], a, b);
+            const int32_t ia = __ldg(dst + 64 * w), ib = __ldg(dst + 64 * w + 32);
+            if (PART) {
+                if (ia >= 0) out[ia] = a;
+                if (ib >= 0) out[ib] = b;
+            } else {
+                if (ia >= 0 && a != 0.f) atomicAdd(out + ia, a);
+                if (ib >= 0 && b != 0.f) atomicAdd(out + ib, b);
+            }
         }
-    }
     } else {
         stk_redo<V, M, W, PART>(I, tile, m, reinterpret_cast<float *>(smem_raw), f, r, r_scalar, y, out, ratio);
     }
