@@ -371,7 +371,8 @@ k_stk_check(int64_t I, int64_t J, int tr, int words_per_tile, int ring, int64_t 
                 const int at = int(Rec<M>::place(v));
                 stack = at & 31;
                 level = top - ring + (((at >> 5) - (top - ring)) % ring + ring) % ring;
-                bad |= (at >> 5) >= ring || __popc(__match_any_sync(0xffffffffu, stack)) != 1;
+                const uint32_t same = __match_any_sync(0xffffffffu, stack);  // by every lane, also one out of the ring
+                bad |= (at >> 5) >= ring || __popc(same) != 1;
                 // a lane without values in the pair may stand at the top of the highest stack
                 if ((Rec<M>::first(v) | Rec<M>::second(v)) == 0u && level < low) level = top;
                 bad |= level < low;
