@@ -251,7 +251,9 @@ int sgtv_set_state_f64(sgtv_t h, const double *f, const double *d, const double 
  * summed in a fixed order; prefetch depth; register cap; "stack": sums in
  * registers) that fit in shared memory. kernel is SGTV_K_FORWARD, SGTV_K_BACK_UPDATE or SGTV_K_SCATTER (the
  * latter in sgtv_variant_count / _name and sgtv_get_variant / sgtv_set_variant
- * only). The set functions return SGTV_ERR_ARG (not sticky) for an index out
+ * only). Where sgtv_set_variant takes one product into or out of the stacked
+ * pair, the other goes with it: into the pair, or back to the form it was last
+ * set to or timed best in. The set functions return SGTV_ERR_ARG (not sticky) for an index out
  * of range or a form that does not fit; sgtv_variant_name returns "" for one. */
 int sgtv_autotune(sgtv_t h, int32_t reps);
 int sgtv_get_variants(sgtv_t h, int32_t *fwd, int32_t *back);

@@ -60,6 +60,7 @@ struct sgtv_ctx {
     std::vector<int64_t> I_off, J_off, S_off;  // per-scan offsets (nscans + 1)
     std::vector<Scan> scan_tab;
     int v_fwd = 0, v_back = 0;  // chosen SpMV variants (see sgtv_autotune)
+    int alone_fwd = 0, alone_back = 0;  // the last chosen (or best timed) ones that are no pair, for leaving the stacked pair
     bool persistent = false;    // one cooperative launch per iteration
     int v_pers = 0;             // its variant (KernelSet::pers)
     bool use_graph = false;     // iterations replayed from captured CUDA graphs
@@ -1584,6 +1585,8 @@ int sgtv_autotune(sgtv_t h, int32_t reps)
         if (ms < best) { best = ms; best_v = v; }
     }
     h->v_back = best_v;
+    h->alone_fwd = h->v_fwd;
+    h->alone_back = h->v_back;
     if (!h->single_pass && !h->persistent && stk_f >= 0 && stk_b >= 0) {
         void *const u = d.u;
         d.u = h->u_buf;
@@ -1675,6 +1678,10 @@ int sgtv_set_variants(sgtv_t h, int32_t fwd, int32_t back)
     if (h->persistent) h->v_pers = (h->v_pers & 4) | pers_index(h, fwd, back);
     h->v_fwd = fwd;
     h->v_back = back;
+    if (h->ks->fwd_need[fwd] != 2) {
+        h->alone_fwd = fwd;
+        h->alone_back = back;
+    }
     drop_graphs(h);
     CK(h, follow_variants(h));
     return SGTV_OK;
@@ -1712,8 +1719,21 @@ int sgtv_set_variant(sgtv_t h, int32_t kernel, int32_t v)
 {
     int rc = check_live(h);
     if (rc) return rc;
-    if (kernel == SGTV_K_FORWARD) return sgtv_set_variants(h, v, h->v_back);
-    if (kernel == SGTV_K_BACK_UPDATE) return sgtv_set_variants(h, h->v_fwd, v);
+    if (kernel == SGTV_K_FORWARD || kernel == SGTV_K_BACK_UPDATE) {
+        // The stacked products go together: the other one comes along into the pair, and back to its own form out
+        // of it.
+        const KernelSet *ks = h->ks;
+        const bool fwd = kernel == SGTV_K_FORWARD;
+        const int n = fwd ? ks->n_fwd : ks->n_back, n_other = fwd ? ks->n_back : ks->n_fwd;
+        const int *need = fwd ? ks->fwd_need : ks->back_need, *need_other = fwd ? ks->back_need : ks->fwd_need;
+        if (v < 0 || v >= n) return SGTV_ERR_ARG;
+        int other = fwd ? h->v_back : h->v_fwd;
+        if (need[v] == 2)
+            while (other = (other + 1) % n_other, need_other[other] != 2) {}
+        else if (need_other[other] == 2)
+            other = fwd ? h->alone_back : h->alone_fwd;
+        return fwd ? sgtv_set_variants(h, v, other) : sgtv_set_variants(h, other, v);
+    }
     if (kernel != SGTV_K_SCATTER || v < 0 || v >= h->ks->n_scatter) return SGTV_ERR_ARG;
     if (!h->single_pass || !scatter_fits(h, v)) return SGTV_ERR_ARG;
     h->v_scatter = v;
