@@ -29,6 +29,7 @@
 
 #include "../../include/sgtv.h"
 #include "../../include/wsnet.h"
+#include "sgtv_rules.h"
 
 namespace {
 
@@ -645,31 +646,34 @@ __device__ __forceinline__ double abs_f64(float v)
 }
 
 // loss += sum (head(z) - t)^2 / n (FP64); dz = 2 (head(z) - t) head'(z) / n with
-// head' = sigmoid on the image channels and 1 on the dual channels. One plane
-// at a time per block, one FP64 add to the loss per block.
+// head' = sigmoid on the image channels and 1 on the dual channels. A block takes
+// `len` consecutive elements of a plane at a time (`pieces` of them a plane), and
+// adds to the loss once.
 __global__ void __launch_bounds__(256)
 k_mse_head(const float *__restrict__ z, const float *__restrict__ tgt, float *__restrict__ dz, int64_t NC, int HW,
-           int Co, int Q, double *__restrict__ loss)
+           int Co, int Q, int pieces, int len, double *__restrict__ loss)
 {
     __shared__ double sh[32];
     double acc = 0.0;
     const int64_t n = NC * HW;
     const float inv = 1.0f / float(n);
-    for (int64_t c = blockIdx.x; c < NC; c += gridDim.x) {
+    for (int64_t t = blockIdx.x; t < NC * pieces; t += gridDim.x) {
+        const int64_t c = t / pieces;
         const bool img = int(c % Co) < Q;
         const float *const zc = z + c * HW, *const tc = tgt + c * HW;
-        for (int k0 = threadIdx.x; k0 < HW; k0 += 4 * kT) {
+        const int k1 = int(t - c * pieces) * len, k2 = len < HW - k1 ? k1 + len : HW;
+        for (int k0 = k1 + int(threadIdx.x); k0 < k2; k0 += 4 * kT) {
             float zz[4], tt[4];  // all loads first
 #pragma unroll
             for (int u = 0; u < 4; u++) {
                 const int k = k0 + u * kT;
-                zz[u] = k < HW ? zc[k] : 0.f;
-                tt[u] = k < HW ? tc[k] : 0.f;
+                zz[u] = k < k2 ? zc[k] : 0.f;
+                tt[u] = k < k2 ? tc[k] : 0.f;
             }
 #pragma unroll
             for (int u = 0; u < 4; u++) {
                 const int k = k0 + u * kT;
-                if (k >= HW) break;
+                if (k >= k2) break;
                 const float diff = (img ? softplus(zz[u]) : zz[u]) - tt[u];
                 const double a = abs_f64(diff);
                 acc = fma(a, a, acc);
@@ -1060,8 +1064,10 @@ int wsnet_loss_grad(wsnet_t h, const float *x, const float *target, int32_t N, d
     WK(h, cudaMemsetAsync(h->loss, 0, sizeof(double), st));
     const int64_t nz = int64_t(N) * h->Co, n64 = int64_t(N) * 64, n128 = int64_t(N) * 128;
     const int64_t full = int64_t(H) * W, half = int64_t(H2) * W2, quarter = int64_t(H4) * W4;
-    k_mse_head<<<unsigned(nz < 8 * int64_t(h->sms) ? nz : 8 * int64_t(h->sms)), kT, 0, st>>>(h->z, target, h->gz, nz,
-                                                                                            H * W, h->Co, h->C, h->loss);
+    const int64_t blocks = 8 * int64_t(h->sms);
+    const int pieces = int(sgtv::mse_pieces(nz, full, blocks)), len = int((full + pieces - 1) / pieces);
+    k_mse_head<<<unsigned(nz * pieces < blocks ? nz * pieces : blocks), kT, 0, st>>>(
+        h->z, target, h->gz, nz, H * W, h->Co, h->C, pieces, len, h->loss);
     conv_bwd(h, h->a8, h->gz, 8, h->g8, h->a8, N, H, W);
     conv_bwd(h, h->s2, h->g8, 7, h->gs2, nullptr, N, H, W);
     // s2 = up(a7) + a2
