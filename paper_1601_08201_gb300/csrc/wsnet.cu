@@ -636,13 +636,13 @@ __global__ void k_head(const float *__restrict__ z, float *__restrict__ o, int64
 
 // |v| as FP64 by integer instructions (the FP64 unit, which a conversion also
 // occupies, does about 2 lanes per clock and multiprocessor): the exponent moved
-// to its new bias; below FP32's normal range 0 (its square is below 2^-252);
-// infinities and NaNs by a real conversion.
+// to its new bias; outside FP32's normal range by a real conversion (a loss may
+// consist of subnormal differences alone).
 __device__ __forceinline__ double abs_f64(float v)
 {
     const uint32_t u = __float_as_uint(v) & 0x7FFFFFFFu;
-    if (u >= 0x7F800000u) return fabs(double(v));
-    return u >= 0x00800000u ? __hiloint2double(int((u >> 3) + 0x38000000u), int(u << 29)) : 0.0;
+    if (u - 0x00800000u >= 0x7F000000u) return u == 0u ? 0.0 : fabs(double(v));
+    return __hiloint2double(int((u >> 3) + 0x38000000u), int(u << 29));
 }
 
 // loss += sum (head(z) - t)^2 / n (FP64); dz = 2 (head(z) - t) head'(z) / n with

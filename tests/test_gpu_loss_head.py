@@ -47,6 +47,17 @@ def test_loss_and_its_derivative(H, W, Q, N, n_dual):
     assert (np.abs(db - dz.sum((0, 2, 3))) <= 1e-5 * np.abs(dz).sum((0, 2, 3))).all()
 
 
+@pytest.mark.parametrize("size", [1e-39, 3e-45, 1e-38, 1e-37])
+def test_differences_below_the_normal_range_count(size):
+    net, x, out = zero_net(8, 12, 3, 2, 2)
+    t = out.clone()
+    t[:, 3:] = size
+    torch.cuda.synchronize()
+    loss = net.loss_grad(x.data_ptr(), t.data_ptr(), 2)
+    d = float(np.float32(size))
+    assert d > 0 and abs(loss / (d * d * 2 / 3) - 1) <= 1e-12
+
+
 @pytest.mark.parametrize("bad", [np.inf, -np.inf, np.nan])
 def test_infinite_and_nan_targets_show_in_the_loss(bad):
     net, x, out = zero_net(8, 12, 3, 1, 0)
