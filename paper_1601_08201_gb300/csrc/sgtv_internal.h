@@ -5,6 +5,8 @@
 #include <cuda_runtime.h>
 #include <stdint.h>
 
+#include "sgtv_rules.h"
+
 namespace sgtv {
 
 // One scan of a batch. A handle holds one or more independent scans stored

@@ -2605,31 +2605,50 @@ __device__ __forceinline__ double dev_term(double yb, double yi)
     return t;
 }
 
+// acc += N of a lane's products, 32 nonzeros apart from p on.
+template <int N, typename T, typename V>
+__device__ __forceinline__ void dev_chunk(const V *__restrict__ val, const T *__restrict__ f,
+                                          const int32_t *__restrict__ col, int64_t p, double &acc)
+{
+    V v[N];
+    T x[N];
+#pragma unroll
+    for (int u = 0; u < N; u++) {
+        v[u] = val[p + 32 * u];
+        x[u] = f[col[p + 32 * u]];
+    }
+#pragma unroll
+    for (int u = 0; u < N; u++) acc = fma(to_f64(v[u]), double(x[u]), acc);
+}
+
 // Deviance partials over the measurements [i0, i1), from the plain CSR form
-// (matrices without tiles, and tiles whose staging would fill an SM): ybar
-// accumulated in FP64 from the stored A values and f. A warp takes 8 rows in
-// turn, lane k keeps row k's ybar, and the 8 terms (a division and a
-// logarithm in FP64, which cost a warp the same for one lane as for 32) are
-// formed side by side.
+// (matrices without tiles, tiles whose staging would fill an SM, few rows): ybar
+// accumulated in FP64 from the stored A values and f. A warp takes R rows (at
+// most 32) in turn, lane k keeps row k's ybar, and their terms (a
+// division and a logarithm in FP64, which cost a warp the same for one lane as
+// for 32) are formed side by side.
 template <typename T, typename V>
 __global__ void __launch_bounds__(256)
 k_dev_partials(int64_t i0, int64_t i1, const int64_t *__restrict__ rowptr, const int32_t *__restrict__ col,
                const V *__restrict__ val, const T *__restrict__ f, const T *__restrict__ r,
-               int r_scalar, const T *__restrict__ y, double *__restrict__ part)
+               int r_scalar, const T *__restrict__ y, int R, double *__restrict__ part)
 {
     __shared__ double sh[32];
-    constexpr int R = 8;
     const int lane = threadIdx.x & 31;
     const int64_t nwarps = (int64_t(gridDim.x) * blockDim.x) >> 5;
     double mine = 0.0;
-    for (int64_t k0 = i0 + R * ((int64_t(blockIdx.x) * blockDim.x + threadIdx.x) >> 5); k0 < i1; k0 += R * nwarps) {
+    // tasks are dealt to the blocks in turn, so that few rows have an FP64 unit each
+    for (int64_t k0 = i0 + R * (int64_t(threadIdx.x >> 5) * gridDim.x + blockIdx.x); k0 < i1; k0 += R * nwarps) {
         const int n = int(i1 - k0 < R ? i1 - k0 : R);
         double yb = 0.0;
         for (int k = 0; k < n; k++) {
             double acc = 0.0;
             const int64_t start = rowptr[k0 + k], end = rowptr[k0 + k + 1];
-            for (int64_t p = start + lane; p < end; p += 32)
-                acc = fma(to_f64(val[p]), double(f[col[p]]), acc);
+            int64_t p = start + lane;
+            // loads ahead, eight of them in the long rows; added in order
+            for (; p + 224 < end; p += 256) dev_chunk<8>(val, f, col, p, acc);
+            for (; p + 96 < end; p += 128) dev_chunk<4>(val, f, col, p, acc);
+            for (; p < end; p += 32) dev_chunk<1>(val, f, col, p, acc);
             acc = warp_sum_d(acc);
             if (lane == k) yb = acc;
         }

@@ -486,16 +486,19 @@ struct Impl {
         k_sum_partials<T><<<d.red_blocks, kThreads, 0, st>>>(n, static_cast<const T *>(a), d.part);
         finalize(d.part, d.red_blocks, 1, 0u, d.red + slot, st);
     }
-    // Tiled wherever the largest tile has at most 3968 columns (31 KB as FP64, 15.5 as FP32: with the row
-    // sums within the 48 KB that a block has without asking): list tiles and short windows. FP32, 60,000
+    // The tiled form is there where the largest tile has at most 3968 columns (31 KB as FP64, 15.5 as FP32: with
+    // the row sums within the 48 KB that a block has without asking): list tiles and short windows. FP32, 60,000
     // rows, tiles of 2460 columns: 24 us, plain 59; 3368: 25 and 59; 3916: 25 and 59; 64^3 (293) 108 and 459.
-    // Wide windows (small problems whose tiles span most of the image) read f from L2 in the plain form.
+    // Wide windows (small problems whose tiles span most of the image) read f from L2 in the plain form, and so do
+    // few rows, which would leave most of the chip without a tile (dev_rows_per_warp).
     static void deviance(const Dev &d, const void *f, int64_t i0, int64_t i1, int slot, cudaStream_t st)
     {
         const T *ff = static_cast<const T *>(f), *r = static_cast<const T *>(d.r), *y = static_cast<const T *>(d.y);
         const V *val = static_cast<const V *>(d.rval);
         int blocks = d.red_blocks;
-        if (d.tr.fmt != 0 && d.tr.max_stage * int(sizeof(double)) <= 31 * 1024) {
+        const bool tiled = d.tr.fmt != 0 && d.tr.max_stage * int(sizeof(double)) <= 31 * 1024;
+        const int in_turn = dev_rows_per_warp(i1 - i0, d.nnz / d.I, d.sm_count, tiled);
+        if (in_turn == 0) {
             // one partial field is free for up to 4 red_blocks blocks (Dev::part)
             const int64_t tiles = (i1 + kTliTile - 1) / kTliTile - i0 / kTliTile;
             blocks = int(tiles < 4 * int64_t(d.red_blocks) ? (tiles > 0 ? tiles : 1) : 4 * int64_t(d.red_blocks));
@@ -507,7 +510,7 @@ struct Impl {
                     i0, i1, d.tr.ntiles, d.rowptr, tiles_of(d.tr), val, ff, r, d.r_scalar, y, d.part);
         } else {
             k_dev_partials<T, V><<<blocks, kThreads, 0, st>>>(i0, i1, d.rowptr, d.col, val, ff, r, d.r_scalar, y,
-                                                              d.part);
+                                                              in_turn, d.part);
         }
         finalize(d.part, blocks, 1, 0u, d.red + slot, st);
     }

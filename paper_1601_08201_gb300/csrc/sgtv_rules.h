@@ -11,6 +11,26 @@
 
 namespace sgtv {
 
+// The deviance's form for `rows` measurements of `mean` nonzeros on average: 0 the
+// tiled one (where there is one), else the rows that a warp of the plain one takes
+// in turn. The plain form has 16 warps a multiprocessor (two blocks of 8). What
+// counts is how many rows lie behind one another in a warp (8 in the tiled form),
+// and from some rows a multiprocessor on the FP64 terms, a division and a
+// logarithm, which cost a warp the same for one row as for 8 side by side. So a warp
+// each while there is one for every row, then the tiled form, and without it 8
+// rows in turn unless they are long. Measured, microseconds, tiled / plain with 1 /
+// 2 / 8 rows (FP32, 152 multiprocessors): 640 rows of 64 nonzeros 10.1 / 5.8 / 6.6 /
+// 14.2, of 1400 40 / 12 / 18 / 60; 2000 rows of 64 10.4 / 10.2 / 8.5 / 14.4, of 1400 45 /
+// 26 / 24 / 60; 6000 rows of 64 10.4 / 24 / 18 / 15, of 1400 54 / 69 / 67 / 71; 20,000 rows
+// of 300 24 / 100 / 77 / 70, of 700 42 / 145 / 126 / 143, of 1400 75 / 232 / 217 / 260;
+// 60,000 rows of 64 27 / 206 / 132 / 81.
+SGTV_RULE int dev_rows_per_warp(int64_t rows, int64_t mean, int sms, bool tiled)
+{
+    if (rows <= 16 * int64_t(sms)) return 1;
+    if (tiled) return 0;
+    return mean <= 512 ? 8 : 1;
+}
+
 // Pieces that a plane (sample, channel) of n elements is cut into for the loss
 // head: one where the planes alone fill `blocks` blocks, else enough to, of at
 // least 1024 elements (four a thread). A sample of one channel, 256 x 256: 87 us with

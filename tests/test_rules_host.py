@@ -26,3 +26,16 @@ def test_loss_head_fills_the_chip_whatever_the_planes(tmp_path):
         assert planes * pieces >= 1216 or length <= 1024, (planes, n, pieces)
         # no more pieces than that takes
         assert pieces == 1 or (planes * (pieces - 1) < 1216 and length > 512), (planes, n, pieces)
+
+
+def test_deviance_form(tmp_path):
+    sms, rows = 152, (1, 64, 1216, 1217, 2432, 2433, 20000, 1 << 20)
+    cases = [(r, mean, tiled) for r in rows for mean in (0, 64, 256, 257, 512, 513, 5000) for tiled in (0, 1)]
+    body = "".join('printf("%%d\\n", dev_rows_per_warp(%d, %d, %d, %d));\n' % (r, m, sms, t) for r, m, t in cases)
+    for (r, mean, tiled), (form,) in zip(cases, run(tmp_path, body)):
+        form = int(form)
+        assert form in (0, 1, 8) and (form != 0 or tiled)
+        if r <= 16 * sms:  # a warp for each row: none has two
+            assert form == 1, (r, mean, tiled)
+        if r > 16 * sms and tiled:
+            assert form == 0, (r, mean)
