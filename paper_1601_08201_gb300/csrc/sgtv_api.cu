@@ -1534,25 +1534,19 @@ int sgtv_autotune(sgtv_t h, int32_t reps)
     cudaEvent_t a, b;
     CK(h, cudaEventCreate(&a));
     CK(h, cudaEventCreate(&b));
-    // Mean time of `reps` launches. Where a launch is long (50 us, so that one
-    // more wait for the stream counts for little), a form whose first launch
-    // after the warm-up takes over 1.5 times the best so far is out of the
-    // running at once.
+    // The time of a form by the autotuner's rule (sgtv_rules.h); the first launch warms up (and asks for its occupancy).
     auto time_it = [&](auto &&launch, float *ms, float so_far) -> cudaError_t {
-        launch();  // warm-up (also the first-launch occupancy query)
-        cudaError_t e = cudaSuccess;
-        for (int pass = so_far > 0.05f ? 0 : 1; pass < 2 && e == cudaSuccess; pass++) {
-            const int n = pass == 0 ? 1 : reps;
-            e = cudaEventRecord(a, st);
-            for (int k = 0; k < n; k++) launch();
-            if (e == cudaSuccess) e = cudaEventRecord(b, st);
-            if (e == cudaSuccess) e = cudaEventSynchronize(b);
-            if (e == cudaSuccess) e = cudaEventElapsedTime(ms, a, b);
-            if (e == cudaSuccess) e = cudaGetLastError();
-            *ms /= float(n);
-            if (*ms > 1.5f * so_far) break;
-        }
-        return e;
+        launch();
+        return tuned_time(
+            [&](int n, float *all) {
+                cudaError_t e = cudaEventRecord(a, st);
+                for (int k = 0; k < n; k++) launch();
+                if (e == cudaSuccess) e = cudaEventRecord(b, st);
+                if (e == cudaSuccess) e = cudaEventSynchronize(b);
+                if (e == cudaSuccess) e = cudaEventElapsedTime(all, a, b);
+                return e == cudaSuccess ? cudaGetLastError() : e;
+            },
+            reps, so_far, ms);
     };
     // Only scratch is written (ratio, f_next): the ADMM state is untouched.
     // The single-pass form times only its scatter forms (the two-pass

@@ -42,4 +42,29 @@ SGTV_RULE int64_t mse_pieces(int64_t planes, int64_t n, int64_t blocks)
     return want < most ? want : most;
 }
 
+// The autotuner's time of one launch of a form: the mean of `reps`, where
+// timed(n, &ms) launches n times, gives the time of all and returns 0 or an error.
+// Where a launch is long (50 us, so that one more wait for the stream counts for
+// little), a form over 1.5 times the best so far is out of the running without
+// them, if two launches by themselves say so: one alone may have been disturbed,
+// and the choice is for the life of the handle.
+template <typename Timed>
+auto tuned_time(Timed &&timed, int reps, float so_far, float *ms) -> decltype(timed(1, ms))
+{
+    if (so_far > 0.05f) {
+        float least = 0.f;
+        for (int k = 0; k < 2; k++) {
+            const auto e = timed(1, ms);
+            if (e != decltype(e)(0)) return e;
+            least = k == 0 || *ms < least ? *ms : least;
+            if (least <= 1.5f * so_far) break;
+        }
+        *ms = least;
+        if (least > 1.5f * so_far) return decltype(timed(1, ms))(0);
+    }
+    const auto e = timed(reps, ms);
+    *ms /= float(reps);
+    return e;
+}
+
 }  // namespace sgtv
