@@ -367,11 +367,8 @@ struct Impl {
     static void shrink_lean(const Dev &d, const Geom &g, const void *f, void *d_out, cudaStream_t st)
     {
         static const int nb = resident_blocks(k_shrink_lean<T, QPL, ONE>);
-        // A warp per site. FP64 sites of a small image are spread over the multiprocessors in blocks of a warp,
-        // since a block of eight waits for one FP64 unit: 13 x 7 x 37 6.6 -> 4.8 us. Not in FP32, where the
-        // spread blocks stand in the way of the row pass that runs beside them (41 x 9 x 54: shrink 2.6 -> 2.3
-        // us, but the row pass 6.1 -> 7.9).
-        const bool spread = sizeof(T) == 8 && g.S < 8 * int64_t(d.sm_count);
+        // A warp per site; Dev::u is set in the single-pass form (FP64 has no stacked one).
+        const bool spread = shrink_spread(sizeof(T), d.u != nullptr, g.S, d.sm_count);
         const int threads = spread ? 32 : kThreads;
         const int blocks = spread ? int(g.S) : grid_for(g.S, d.sm_count * nb);
         k_shrink_lean<T, QPL, ONE><<<blocks, threads, 0, st>>>(

@@ -42,6 +42,21 @@ SGTV_RULE int64_t mse_pieces(int64_t planes, int64_t n, int64_t blocks)
     return want < most ? want : most;
 }
 
+// Whether the shrink of `sites` sites goes out in blocks of a warp, one a site,
+// instead of eight: FP64 sites of a small image, where a block of eight waits for
+// one FP64 unit (13 x 7 x 37, the shrink alone 6.6 -> 4.8 us; an iteration of two
+// passes 12.9 -> 11.3). Not in the single-pass form (`staged`: a row pass that stages
+// tiles in shared memory runs beside the shrink): blocks on every multiprocessor
+// are in the way of its start on those with room for its tiles, and replayed from
+// graphs an iteration of 41 x 9 x 54 took 78 us instead of 44, 20 x 20 x 40 64 instead
+// of 37, 2000 rows of 1500 nonzeros 214 instead of 137. Nor in FP32, where they stand
+// in the way of the stacked row pass (41 x 9 x 54: shrink 2.6 -> 2.3 us, but the row
+// pass 6.1 -> 7.9).
+SGTV_RULE bool shrink_spread(int elem_size, bool staged, int64_t sites, int sms)
+{
+    return elem_size == 8 && !staged && sites < 8 * int64_t(sms);
+}
+
 // The autotuner's time of one launch of a form: the mean of `reps`, where
 // timed(n, &ms) launches n times, gives the time of all and returns 0 or an error.
 // Where a launch is long (50 us, so that one more wait for the stream counts for

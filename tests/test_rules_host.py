@@ -86,3 +86,10 @@ def test_deviance_form(tmp_path):
             assert form == 1, (r, mean, tiled)
         if r > 16 * sms and tiled:
             assert form == 0, (r, mean)
+
+
+def test_shrink_is_spread_beside_kernels_without_staging_only(tmp_path):
+    cases = [(e, st, s) for e in (4, 8) for st in (0, 1) for s in (1, 369, 1215, 1216, 1 << 20)]
+    body = "".join('printf("%%d\\n", int(shrink_spread(%d, %d, %d, 152)));\n' % c for c in cases)
+    for (elem, staged, sites), (spread,) in zip(cases, run(tmp_path, body)):
+        assert int(spread) == (elem == 8 and not staged and sites < 1216)
