@@ -46,6 +46,9 @@ struct sgtv_ctx {
     sgtv_free_fn free_ = nullptr;
     void *alloc_user = nullptr;
     std::vector<void *> blocks;
+    std::vector<size_t> block_bytes;  // of blocks[k]
+    // forms of A beside the CSR, CSC and tiled ones: held only while a chosen or pinned variant reads them
+    std::vector<void *> sp_blocks, st_blocks;
     int64_t bytes = 0;
 
     Geom g{};
@@ -127,6 +130,7 @@ void *dev_alloc(sgtv_t h, size_t bytes, cudaError_t *err)
     }
     if (p) {
         h->blocks.push_back(p);
+        h->block_bytes.push_back(bytes);
         h->bytes += int64_t(bytes);
     }
     return p;
@@ -137,7 +141,9 @@ void dev_free(sgtv_t h, void *p)
     if (!p) return;
     for (size_t k = 0; k < h->blocks.size(); k++)
         if (h->blocks[k] == p) {
+            h->bytes -= int64_t(h->block_bytes[k]);
             h->blocks.erase(h->blocks.begin() + k);
+            h->block_bytes.erase(h->block_bytes.begin() + k);
             break;
         }
     if (h->free_) h->free_(p, h->alloc_user);
@@ -195,7 +201,7 @@ int check_live(sgtv_t h)
 bool variant_ok(const Dev &d, const TliMat &m, int need)
 {
     if (need == 0) return true;
-    if (need == 2) return d.st.built && d.st.part;
+    if (need == 2) return d.st.built && d.st.part;  // need_forms builds it
     if (m.fmt == 0) return false;
     if (need == 1) return true;
     return m.tma_stage_bytes > 0 && int64_t(need) * m.tma_stage_bytes <= m.smem_optin - 1024;
@@ -269,7 +275,8 @@ int validate_ptr(sgtv_t h, const int64_t *ptr, int64_t n, int64_t nnz, const cha
 }
 
 // A single-pass scatter form fits when its staging-sized buffers (f and the
-// accumulators) fit in the opt-in shared memory of one block.
+// accumulators) fit in the opt-in shared memory of one block, and the form of A
+// that it reads is there (need_forms builds them).
 bool scatter_fits(sgtv_t h, int v)
 {
     const TliMat &m = h->d.tr;
@@ -529,6 +536,55 @@ int build_tli(sgtv_t h, const int64_t *ptr, const int64_t *host_ptr, const int32
     return SGTV_OK;
 }
 
+// Build the bank-dealt row stream of the single-pass scatter (sgtv_sp.cu). Where
+// its memory is refused, the handle runs without it: d.sp.built stays 0.
+int build_sp(sgtv_t h)
+{
+    Dev &d = h->d;
+    cudaStream_t st = h->stream;
+    const int64_t I = d.I;
+    const size_t V = h->ks->val_size;
+    std::vector<int64_t> rp(I + 1), srp(I + 1);
+    CK(h, cudaMemcpyAsync(rp.data(), d.rowptr, sizeof(int64_t) * (I + 1), cudaMemcpyDeviceToHost, st));
+    CK(h, cudaStreamSynchronize(st));
+    srp[0] = 0;
+    for (int64_t i = 0; i < I; i++) srp[i + 1] = srp[i] + ((rp[i + 1] - rp[i] + 3) & ~int64_t(3));
+    h->max_sp_span = 0;
+    for (int64_t i0 = 0; i0 < I; i0 += kTliTile / 8) {
+        const int64_t span = srp[i0 + kTliTile / 8 < I ? i0 + kTliTile / 8 : I] - srp[i0];
+        if (span > h->max_sp_span) h->max_sp_span = span;
+    }
+    const int64_t nsp = srp[I] + 16;
+    const size_t bytes[3] = {sizeof(int64_t) * (I + 1), sizeof(uint16_t) * nsp, V * nsp};
+    void *p[3];
+    for (int k = 0; k < 3; k++) {
+        cudaError_t ae;
+        p[k] = dev_alloc(h, bytes[k], &ae);
+        if (!p[k]) {
+            cudaGetLastError();  // an optional form: out of memory is no error of the handle
+            for (int m = 0; m < k; m++) dev_free(h, p[m]);
+            return SGTV_OK;
+        }
+    }
+    h->sp_blocks.assign(p, p + 3);
+    int *const flag = d.flag + 1;  // flag itself keeps what iterations have found
+    int hflag = 0;
+    CK(h, cudaMemcpyAsync(p[0], srp.data(), bytes[0], cudaMemcpyHostToDevice, st));
+    CK(h, cudaMemsetAsync(p[1], 0xFF, bytes[1], st));  // an unwritten slot fails the check
+    CK(h, cudaMemsetAsync(p[2], 0, bytes[2], st));
+    d.sp.rp = static_cast<int64_t *>(p[0]);
+    d.sp.lidx = static_cast<uint16_t *>(p[1]);
+    d.sp.val = p[2];
+    CK(h, cudaMemsetAsync(flag, 0, sizeof(int), st));
+    CK(h, sp_build(I, d.rowptr, d.tr.lidx, d.rval, int(V), d.sp.rp, d.tr.wlen, d.tr.uoff, d.sp.lidx, d.sp.val, flag,
+                   d.sm_count, st));
+    CK(h, cudaMemcpyAsync(&hflag, flag, sizeof(int), cudaMemcpyDeviceToHost, st));
+    CK(h, cudaStreamSynchronize(st));
+    if (hflag & 32) return fail(h, SGTV_ERR_CUDA, "the single-pass row stream failed its set-up check");
+    d.sp.built = 1;
+    return SGTV_OK;
+}
+
 // Build the stacked row form (sgtv_stack.cu) where it applies: FP32 vectors,
 // tiles of at most 32 * kStkMaxWords columns, a schedule that fits the ring,
 // and a size no larger than the tiled form's by more than a quarter (thin
@@ -659,11 +715,10 @@ int build_stack(sgtv_t h, bool parts)
     int hflag = 0;
     e = cudaMemcpyAsync(m.lvl, lvl.data(), sizeof(int64_t) * (m.ntiles + 1), cudaMemcpyHostToDevice, st);
     if (e == cudaSuccess) e = cudaMemsetAsync(m.val, 0, size_t(lvl[m.ntiles]) * 32 * vb + 16, st);
-    if (e == cudaSuccess) e = cudaMemsetAsync(d.flag, 0, sizeof(int), st);
-    if (e == cudaSuccess)
-        e = stk_fill(I, J, m, d.rowptr, d.col, d.rval, vb, lanes, rank, start, d.flag, d.sm_count, st);
-    if (e == cudaSuccess) e = cudaMemcpyAsync(&hflag, d.flag, sizeof(int), cudaMemcpyDeviceToHost, st);
-    if (e == cudaSuccess) e = cudaMemsetAsync(d.flag, 0, sizeof(int), st);
+    int *const flag = d.flag + 1;  // flag itself keeps what iterations have found
+    if (e == cudaSuccess) e = cudaMemsetAsync(flag, 0, sizeof(int), st);
+    if (e == cudaSuccess) e = stk_fill(I, J, m, d.rowptr, d.col, d.rval, vb, lanes, rank, start, flag, d.sm_count, st);
+    if (e == cudaSuccess) e = cudaMemcpyAsync(&hflag, flag, sizeof(int), cudaMemcpyDeviceToHost, st);
     if (e == cudaSuccess) e = cudaStreamSynchronize(st);
     if (e != cudaSuccess) return broken(e);
     if (hflag) {
@@ -708,8 +763,42 @@ int build_stack(sgtv_t h, bool parts)
         h->u_buf = u;
     }
     drop(tmp);
+    h->st_blocks = mine;
     m.built = 1;
     return SGTV_OK;
+}
+
+// The forms of A that a variant's need (KernelSet::scatter_sp, fwd_need) names,
+// built if they are not there; which of them could be built, scatter_fits and
+// variant_ok then say.
+int need_forms(sgtv_t h, bool sp, bool stack)
+{
+    int rc = SGTV_OK;
+    if (h->d.nnz == 0 || h->persistent) return rc;
+    if (sp && h->single_pass && !h->d.sp.built) rc = build_sp(h);
+    if (rc == SGTV_OK && stack && !h->d.st.built) rc = build_stack(h, !h->single_pass);
+    return rc;
+}
+
+// Give back the forms that the chosen variants do not read (nothing that reads
+// them is in flight: the autotuner has waited for the stream).
+void drop_forms(sgtv_t h)
+{
+    auto give = [&](std::vector<void *> &list) {
+        for (void *p : list) dev_free(h, p);
+        list.clear();
+    };
+    const int sp = h->single_pass ? h->ks->scatter_sp[h->v_scatter] : 0;
+    const bool stack = h->single_pass ? sp == 2 : h->ks->back_need[h->v_back] == 2;
+    if (sp != 1) {
+        give(h->sp_blocks);
+        h->d.sp = SpStream{};
+    }
+    if (!stack) {
+        give(h->st_blocks);
+        h->d.st = StackMat{};
+        h->u_buf = nullptr;
+    }
 }
 
 // Two-pass handles: the stacked pair reads u = d - c, which the shrink writes
@@ -1077,38 +1166,6 @@ static int setup_impl(sgtv_t *out, int32_t nscans, const sgtv_scan *sc, const sg
     } else if (h->precision == SGTV_PREC_FP64) {
         convert_values_f64(fr, p_rval, nnz_pad, st);
         convert_values_f64(fc, p_cval, nnz_pad, st);
-    }
-    if (h->single_pass && nnz > 0) {
-        // the bank-dealt row stream of the single-pass scatter (sgtv_sp.cu)
-        std::vector<int64_t> srp(I + 1);
-        srp[0] = 0;
-        for (int64_t i = 0; i < I; i++) srp[i + 1] = srp[i] + ((hrp[i + 1] - hrp[i] + 3) & ~int64_t(3));
-        for (int64_t i0 = 0; i0 < I; i0 += kTliTile / 8) {
-            const int64_t span = srp[i0 + kTliTile / 8 < I ? i0 + kTliTile / 8 : I] - srp[i0];
-            if (span > h->max_sp_span) h->max_sp_span = span;
-        }
-        const int64_t nsp = srp[I] + 16;
-        void *p_srp, *p_sli, *p_sval;
-        ALLOC(p_srp, sizeof(int64_t) * (I + 1));
-        ALLOC(p_sli, sizeof(uint16_t) * nsp);
-        ALLOC(p_sval, V * nsp);
-        SK(cudaMemcpyAsync(p_srp, srp.data(), sizeof(int64_t) * (I + 1), cudaMemcpyHostToDevice, st));
-        SK(cudaMemsetAsync(p_sli, 0xFF, sizeof(uint16_t) * nsp, st));  // an unwritten slot fails the check
-        SK(cudaMemsetAsync(p_sval, 0, V * nsp, st));
-        d.sp.rp = static_cast<int64_t *>(p_srp);
-        d.sp.lidx = static_cast<uint16_t *>(p_sli);
-        d.sp.val = p_sval;
-        SK(cudaMemsetAsync(d.flag, 0, sizeof(int), st));
-        SK(sp_build(I, d.rowptr, d.tr.lidx, d.rval, int(V), d.sp.rp, d.tr.wlen, d.tr.uoff, d.sp.lidx, d.sp.val,
-                    d.flag, sms, st));
-        SK(cudaMemcpyAsync(&hflag, d.flag, sizeof(int), cudaMemcpyDeviceToHost, st));
-        SK(cudaStreamSynchronize(st));
-        if (hflag & 32) return bail(fail(h, SGTV_ERR_CUDA, "the single-pass row stream failed its set-up check"));
-        d.sp.built = 1;
-    }
-    if (nnz > 0 && !h->persistent) {
-        const int trc = build_stack(h, !h->single_pass);
-        if (trc != SGTV_OK) return bail(trc);
     }
     // y and r (expanded to one value per measurement unless a single scalar)
     {
@@ -1553,6 +1610,11 @@ int sgtv_autotune(sgtv_t h, int32_t reps)
     // products serve it only for the KKT measure).
     // The stacked pair is one choice: timed together, against the sum of the
     // best of the others.
+    if ((rc = need_forms(h, true, true)) != SGTV_OK) {
+        cudaEventDestroy(a);
+        cudaEventDestroy(b);
+        return rc;
+    }
     float best = 3.4e38f, other = 0.f;
     int best_v = 0, stk_f = -1, stk_b = -1;
     for (int v = 0; v < h->ks->n_fwd; v++)
@@ -1643,6 +1705,7 @@ int sgtv_autotune(sgtv_t h, int32_t reps)
     cudaEventDestroy(a);
     cudaEventDestroy(b);
     CK(h, follow_variants(h));
+    drop_forms(h);
     int fl = 0;
     CK(h, cudaMemcpy(&fl, h->d.flag, sizeof(int), cudaMemcpyDeviceToHost));
     if (fl & 2) return fail(h, SGTV_ERR_TIMEOUT, "a bounded device-side wait gave up");
@@ -1663,6 +1726,8 @@ int sgtv_set_variants(sgtv_t h, int32_t fwd, int32_t back)
     if (rc) return rc;
     if (fwd < 0 || fwd >= h->ks->n_fwd || back < 0 || back >= h->ks->n_back)
         return SGTV_ERR_ARG;  // not sticky: the handle keeps its variants
+    if (h->ks->fwd_need[fwd] == 2 && h->ks->back_need[back] == 2 && (rc = need_forms(h, false, true)) != SGTV_OK)
+        return rc;
     if (!variant_ok(h->d, h->d.tr, h->ks->fwd_need[fwd]) || !variant_ok(h->d, h->d.tc, h->ks->back_need[back]))
         return SGTV_ERR_ARG;  // that tiled form was not built for this matrix
     if ((h->ks->fwd_need[fwd] == 2) != (h->ks->back_need[back] == 2))
@@ -1729,7 +1794,9 @@ int sgtv_set_variant(sgtv_t h, int32_t kernel, int32_t v)
         return fwd ? sgtv_set_variants(h, v, other) : sgtv_set_variants(h, other, v);
     }
     if (kernel != SGTV_K_SCATTER || v < 0 || v >= h->ks->n_scatter) return SGTV_ERR_ARG;
-    if (!h->single_pass || !scatter_fits(h, v)) return SGTV_ERR_ARG;
+    if (!h->single_pass) return SGTV_ERR_ARG;
+    if ((rc = need_forms(h, h->ks->scatter_sp[v] == 1, h->ks->scatter_sp[v] == 2)) != SGTV_OK) return rc;
+    if (!scatter_fits(h, v)) return SGTV_ERR_ARG;
     h->v_scatter = v;
     drop_graphs(h);
     return SGTV_OK;
