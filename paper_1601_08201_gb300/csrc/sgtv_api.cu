@@ -556,17 +556,15 @@ int build_sp(sgtv_t h)
     }
     const int64_t nsp = srp[I] + 16;
     const size_t bytes[3] = {sizeof(int64_t) * (I + 1), sizeof(uint16_t) * nsp, V * nsp};
-    void *p[3];
-    for (int k = 0; k < 3; k++) {
-        cudaError_t ae;
-        p[k] = dev_alloc(h, bytes[k], &ae);
-        if (!p[k]) {
-            cudaGetLastError();  // an optional form: out of memory is no error of the handle
-            for (int m = 0; m < k; m++) dev_free(h, p[m]);
-            return SGTV_OK;
-        }
+    auto r256 = [](size_t v) { return (v + 255) & ~size_t(255); };
+    cudaError_t ae;
+    char *const all = static_cast<char *>(dev_alloc(h, r256(bytes[0]) + r256(bytes[1]) + bytes[2], &ae));
+    if (!all) {
+        cudaGetLastError();  // an optional form: out of memory is no error of the handle
+        return SGTV_OK;
     }
-    h->sp_blocks.assign(p, p + 3);
+    h->sp_blocks.assign(1, all);
+    void *const p[3] = {all, all + r256(bytes[0]), all + r256(bytes[0]) + r256(bytes[1])};
     int *const flag = d.flag + 1;  // flag itself keeps what iterations have found
     int hflag = 0;
     CK(h, cudaMemcpyAsync(p[0], srp.data(), bytes[0], cudaMemcpyHostToDevice, st));
@@ -676,8 +674,10 @@ int build_stack(sgtv_t h, bool parts)
     auto r256 = [](int64_t v) { return (v + 255) & ~int64_t(255); };
     const int64_t nd = h->g.n_dirs;
     const int64_t keep[] = {r256(4 * places), r256(rec_bytes), r256(4 * pairs), r256(8 * (m.ntiles + 1)),
-                            parts ? r256(4 * (J + 1)) : 0, parts ? r256(4 * places) : 0, parts ? r256(4 * J * nd) : 0};
-    const int64_t work[] = {r256(places), r256(2 * nnz), r256(64 * pairs), r256(4 * m.ntiles), parts ? r256(4 * J) : 0};
+                            parts ? r256(4 * (J + 1)) : 0, parts ? r256(4 * places) : 0, parts ? r256(4 * J * nd) : 0,
+                            parts ? r256(4 * places) : 0};
+    const int64_t work[] = {r256(places), r256(2 * nnz), r256(64 * pairs), r256(4 * m.ntiles), parts ? r256(4 * J) : 0,
+                            parts ? r256(4 * places) : 0};
     int64_t n_keep = 0, n_work = 0;
     for (int64_t v : keep) n_keep += v;
     for (int64_t v : work) n_work += v;
@@ -748,9 +748,8 @@ int build_stack(sgtv_t h, bool parts)
         }
         // a column in very many tiles would make its one thread sort and add for long
         if (widest > 1024) return without();
-        int32_t *ent = static_cast<int32_t *>(get(sizeof(int32_t) * off[J], tmp));
-        m.part = get(sizeof(float) * off[J], mine);
-        if (!ent || !m.part) return without();
+        m.part = next(pk, keep[7]);  // off[J] <= places
+        int32_t *ent = static_cast<int32_t *>(next(pw, work[5]));
         e = cudaMemcpyAsync(m.poff, off.data(), sizeof(int32_t) * (J + 1), cudaMemcpyHostToDevice, st);
         if (e == cudaSuccess) e = cudaMemsetAsync(m.ppos, 0xFF, sizeof(int32_t) * places, st);
         if (e == cudaSuccess) e = cudaMemsetAsync(m.part, 0, sizeof(float) * off[J], st);

@@ -386,20 +386,20 @@ k_stk_check(int64_t I, int64_t J, int tr, int words_per_tile, int ring, int64_t 
                 x += (unsigned long long)idx[p] * (unsigned long long)val[p];
             }
             const uint32_t m = (r & 1) ? Rec<M>::second(v) : Rec<M>::first(v);
-            for (int w = 0; w < words_per_tile; w++)
-                if ((m >> w) & 1u) {
-                    const int32_t col = uidx[(t * words_per_tile + w) * 32 + lane];
-                    if (level < 0 || level >= top || col < 0 || col >= J) {
-                        bad = true;
-                        break;
-                    }
-                    const unsigned long long y = (unsigned long long)sval[(lvl[t] + level) * 32 + stack];
-                    n -= 1;
-                    c -= (unsigned long long)col;
-                    b -= y;
-                    x -= (unsigned long long)col * y;
-                    level++;
-                }
+#pragma unroll 4
+            for (int w = 0; w < words_per_tile; w++) {  // several words' loads in flight
+                const int at = level + __popc(m & ((1u << w) - 1u));
+                const bool in = ((m >> w) & 1u) && at >= 0 && at < top && at < h;
+                const int32_t col = uidx[(t * words_per_tile + w) * 32 + lane];
+                const unsigned long long y = in ? (unsigned long long)sval[(lvl[t] + at) * 32 + stack] : 0ull;
+                if (!((m >> w) & 1u)) continue;
+                bad |= !in || col < 0 || col >= J;
+                n -= 1;
+                c -= (unsigned long long)col;
+                b -= y;
+                x -= (unsigned long long)col * y;
+            }
+            level += __popc(m);
             bad |= (m >> words_per_tile) != 0u;
             __syncwarp();
 #pragma unroll
