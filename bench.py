@@ -325,14 +325,18 @@ def algorithmic_bytes(P, precision, variants=None, tli=None, n_dirs=4, survey_ba
     window copies are L2 re-reads of f / ratio and are not counted. The
     single-pass row-stream variants ("sp_") stream the same 2-byte indices and
     values with each row padded to a multiple of 4 elements, plus their own
-    row pointers. The stacked forms ("stack") stream the values and one record
-    per lane and pair of rows. Survey basis (survey_basis=True): every SpMV streams a plain
+    row pointers. The stacked forms ("stack") stream what tli["stack"] (the
+    handle's stack_info) says: the levels of the stacks, a record per lane and
+    pair of rows, the copies' control words, the tiles' columns and, in two
+    passes, the places of the partial sums; without it the values and 32-bit
+    records alone, a lower bound. Survey basis (survey_basis=True): every SpMV streams a plain
     int32 index and a value per nonzero (4 + V bytes), the accounting of the
     planning survey's roofline table."""
     T = 8 if precision == "fp64" else 4
     V = {"fp32": 4, "bf16": 2, "fp64": 8}[precision]
     nnz, I, J = P.nnz, P.I, P.J
     variants = variants or {}
+    stack = (tli or {}).get("stack")
     out = {}
 
     def stream(kernel, side, nseg):
@@ -347,31 +351,47 @@ def algorithmic_bytes(P, precision, variants=None, tli=None, n_dirs=4, survey_ba
             rl = np.diff(P.csr_rowptr)
             nsp = int(((rl + 3) // 4 * 4).sum())
             return nsp * (2 + V) + meta + 8 * (I + 1)
-        if name.startswith("stack"):  # values, and at least a 32-bit record per lane and pair of rows
-            return nnz * V + 64 * I
+        if name.startswith("stack"):
+            return stacked_bytes(nnz, I, V, stack)
         return nnz * (4 + V)
 
+    def pointers(kernel):  # the stacked forms read none
+        return 0 if variants.get(kernel, "").startswith("stack") and tli and not survey_basis else (I + 1) * 8
+
     # A by rows, row pointers, f gathered once, y, r, ratio written
-    out["k_forward"] = stream("k_forward", "csr", I) + (I + 1) * 8 + J * T + I * T + I * T + P.b.size * T
+    out["k_forward"] = stream("k_forward", "csr", I) + pointers("k_forward") + J * T + I * T + I * T + P.b.size * T
     # A by columns, column pointers, ratio gathered once, f (read), s, f_new (write), d and c
     out["k_back_update"] = (stream("k_back_update", "csc", J) + (J + 1) * 8 + I * T + 3 * J * T
                             + 2 * n_dirs * J * T)
-    if variants.get("k_back_update", "").startswith("stack") and not survey_basis:
-        # the stacked pair reads A in its forward pass: at least one partial sum per hyper-voxel and its
-        # place, s, f (read), f_new (write), u = d - c
-        out["k_back_update"] = J * T + (J + 1) * 4 + 3 * J * T + n_dirs * J * T
-    single = "k_scatter" in variants
-    # f_new, c read; d, c written (and, in the single-pass form, u = d - c
+    pair = variants.get("k_back_update", "").startswith("stack")
+    if pair and not survey_basis:
+        # the stacked pair reads A in its forward pass and leaves partial sums (at least one per hyper-voxel):
+        # these and the columns' first ones, s, f (read), f_new (write), u = d - c
+        parts = stack["partials"] if stack else J
+        if stack:
+            out["k_forward"] += parts * T + 128 * stack["tiles"] * stack["words"]  # their places
+        out["k_back_update"] = parts * T + (J + 1) * 4 + 3 * J * T + n_dirs * J * T
+    writes_u = "k_scatter" in variants or pair
+    # f_new, c read; d, c written (and, in the single-pass and stacked forms, u = d - c
     # for the f-update)
-    out["k_shrink"] = J * T + (4 if single else 3) * n_dirs * J * T
+    out["k_shrink"] = J * T + (4 if writes_u else 3) * n_dirs * J * T
     # single-pass form: the CSR stream once, f gathered once, y, r, e written
     # once (its atomic adds stay in L2); the f-update reads e, s, f, u and
     # writes f_new and the cleared e
-    out["k_scatter"] = stream("k_scatter", "csr", I) + (I + 1) * 8 + J * T + I * T + P.b.size * T + J * T
+    out["k_scatter"] = stream("k_scatter", "csr", I) + pointers("k_scatter") + J * T + I * T + P.b.size * T + J * T
     out["k_fupdate"] = J * T * (5 + n_dirs)
     # the persistent one-launch iteration moves what the three kernels move
     out["k_iteration"] = out["k_forward"] + out["k_back_update"] + out["k_shrink"]
     return out
+
+
+def stacked_bytes(nnz, I, V, stack):
+    """What a pass streams of A in the stacked row form."""
+    if not stack:  # a lower bound: the values and a 32-bit record per lane and pair of rows
+        return nnz * V + 64 * I
+    pairs, rec = (I + 1) // 2, 4 if stack["words"] <= 10 else 8
+    return (32 * V * stack["levels"] + pairs * (32 * rec + 4) + 8 * (stack["tiles"] + 1)
+            + 128 * stack["tiles"] * stack["words"])
 
 
 def measured_peaks():
@@ -436,6 +456,7 @@ def batch_bytes(scans, precision, form, tli, tuning=None):
 def batch_bytes_by_kernel(scans, precision, form, tli, tuning=None):
     """batch_bytes split by kernel; `tuning`: the chosen variants by kernel (the stacked forms stream other bytes)."""
     stacked = any(v.startswith("stack") for v in (tuning or {}).values())
+    stack = tli.get("stack")
     T = 8 if precision == "fp64" else 4
     V = {"fp32": 4, "bf16": 2, "fp64": 8}[precision]
     I = sum(P.I for P in scans)
@@ -447,12 +468,14 @@ def batch_bytes_by_kernel(scans, precision, form, tli, tuning=None):
     if form == "single_pass":
         nsp = sum(int(((np.diff(P.csr_rowptr) + 3) // 4 * 4).sum()) for P in scans)
         # f-update: e, s, f, u (4 directions), f_new, e cleared; shrink: f, c read, d, c, u written
-        rows = nnz * V + 64 * I if stacked else nsp * (2 + V) + meta_r + 16 * (I + 1)
+        rows = stacked_bytes(nnz, I, V, stack) if stacked else nsp * (2 + V) + meta_r + 16 * (I + 1)
         return {"k_scatter": rows + T * (J + 2 * I + J),
                 "k_fupdate": T * J * 9, "k_shrink": T * J * 17}
     if stacked:
-        return {"k_forward": nnz * V + 64 * I + T * (J + 3 * I), "k_back_update": 4 * (J + 1) + 8 * T * J,
-                "k_shrink": 17 * T * J}
+        parts = stack["partials"] if stack else J
+        places = 128 * stack["tiles"] * stack["words"] + T * parts if stack else 0
+        return {"k_forward": stacked_bytes(nnz, I, V, stack) + places + T * (J + 3 * I),
+                "k_back_update": T * parts + 4 * (J + 1) + 7 * T * J, "k_shrink": 17 * T * J}
     return {"k_forward": nnz * (2 + V) + meta_r + 8 * (I + 1) + T * (J + 3 * I),
             "k_back_update": nnz * (2 + V) + meta_c + 8 * (J + 1) + T * I + 3 * T * J + 8 * T * J,
             "k_shrink": 13 * T * J}
@@ -479,7 +502,7 @@ def batched_form(sgtv, synth, args, stream, torch, form, K, W, sample_clocks=Fal
             prof = {k: v for k, v in h.profile_read().items() if v[1] > 0}
             h.profile(False)
             h.sync()
-            tli = h.tli_info()
+            tli = {**h.tli_info(), "stack": h.stack_info()}
             names = h.variant_names()
             tuning = ({"k_scatter": names["k_scatter"][h.get_variant(sgtv.K_SCATTER)]} if form == "single_pass" else
                       {"k_forward": names["k_forward"][h.get_variants()[0]]})
@@ -496,7 +519,7 @@ def batched_form(sgtv, synth, args, stream, torch, form, K, W, sample_clocks=Fal
         torch.cuda.synchronize()
         out = dict(ms=e0.elapsed_time(e1) / K, clocks=sampler.stop() if sampler else None)
         if isinstance(problem, list):
-            out.update(f=h.get_state_f64()[0], info=h.batch_info(), tli=h.tli_info())
+            out.update(f=h.get_state_f64()[0], info=h.batch_info(), tli={**h.tli_info(), "stack": h.stack_info()})
             names = h.variant_names()
             out["tuning"] = ({"k_scatter": names["k_scatter"][h.get_variant(sgtv.K_SCATTER)]}
                              if form == "single_pass" else
@@ -631,7 +654,7 @@ def time_form(sgtv, P, args, form, stream, torch, barrier, ws, sample_clocks=Fal
     h.sync()
     h.set_serial(False)
     ms_serial = a0.elapsed_time(a1)
-    tli = h.tli_info()
+    tli = {**h.tli_info(), "stack": h.stack_info()}
     h.close()
     ab = algorithmic_bytes(P, args.precision, tuning, tli)
     peak, peak_kind = measured_peaks()
@@ -695,8 +718,8 @@ def main():
     it_survey = sum(sb[k] * v[1] for k, v in prof.items()) / args.steps
     roofline = {"bound": "hbm", "kernel": dom, "achieved": achieved, "peak": peak, "unit": "GB/s",
                 "frac": achieved / peak, "peak_source": peak_kind,
-                "bytes_basis": "the kernel's stored format (stack: values, bit records, tiles' columns; others: 16-bit local "
-                               "indices, padded rows)",
+                "bytes_basis": "the kernel's stored format (stack: levels of values, bit records, control words, tiles' "
+                               "columns; others: 16-bit local indices, padded rows)",
                 "survey_basis": {"kernel_bytes": sb[dom], "achieved": sb[dom] / (dom_ms / 1e3) / 1e9,
                                  "frac": sb[dom] / (dom_ms / 1e3) / 1e9 / peak,
                                  "iteration_bytes": it_survey,

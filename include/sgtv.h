@@ -275,6 +275,14 @@ const char *sgtv_variant_name(sgtv_t h, int32_t kernel, int32_t v);
 int sgtv_tli_info(sgtv_t h, int32_t *fmt, int64_t *list_entries, int64_t *window_elems,
                   int64_t *max_stage);
 
+/* The stacked row form where it is held (zeros elsewhere): words = columns per
+ * lane, tile_rows = rows per tile, tiles, levels = 32-value levels of its stacks,
+ * partials = partial sums of e (two-pass handles). Per pass it streams levels * 32
+ * values, a record per lane and pair of rows (4 bytes up to 10 words, else 8), 4
+ * bytes per pair of rows and tiles * words * 32 column indices. Each non-NULL
+ * pointer receives one value. */
+int sgtv_stack_info(sgtv_t h, int32_t *words, int32_t *tile_rows, int64_t *tiles, int64_t *levels, int64_t *partials);
+
 /* Replace the counts y [I], the background b [b_len] (b_len as at set-up) and
  * the regularisation weight lambda of a one-scan handle, keeping A, and
  * re-initialise the state by the set-up rule (host pointers, copied). Many

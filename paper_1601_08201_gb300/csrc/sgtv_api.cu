@@ -69,6 +69,7 @@ struct sgtv_ctx {
     bool use_graph = false;     // iterations replayed from captured CUDA graphs
     bool single_pass = false;   // A streamed once per surrogate step (scatter + f-update)
     void *e_acc = nullptr;      // its accumulator of e (all zero between iterations)
+    int64_t stk_levels = 0, stk_partials = 0;  // of the stacked form: levels of its stacks, partial sums
     void *u_buf = nullptr;      // u = d - c of a two-pass handle's stacked form (in Dev::u while that form is chosen)
     int v_scatter = 0;          // its scatter variant (KernelSet::scatter)
     int64_t max_warp_span = 0;  // most nonzeros in kTliTile / 8 consecutive rows
@@ -710,6 +711,8 @@ int build_stack(sgtv_t h, bool parts)
     std::vector<int64_t> lvl(m.ntiles + 1, 0);
     for (int64_t t = 0; t < m.ntiles; t++) lvl[t + 1] = lvl[t] + hh[t];
     if (m.ring > kStkMaxRing || lvl[m.ntiles] * 32 * vb + rec_bytes + places * 4 > most_bytes) return without();
+    h->stk_levels = lvl[m.ntiles];
+    h->stk_partials = 0;
     m.val = get(size_t(lvl[m.ntiles]) * 32 * vb + 16, mine);
     if (!m.val) return without();
     int hflag = 0;
@@ -746,6 +749,7 @@ int build_stack(sgtv_t h, bool parts)
             off[j + 1] = off[j] + hc[j];
             if (hc[j] > widest) widest = hc[j];
         }
+        h->stk_partials = off[J];
         // a column in very many tiles would make its one thread sort and add for long
         if (widest > 1024) return without();
         m.part = next(pk, keep[7]);  // off[J] <= places
@@ -1818,6 +1822,18 @@ int sgtv_tli_info(sgtv_t h, int32_t *fmt, int64_t *list_entries, int64_t *window
         if (list_entries) list_entries[k] = nl;
         if (window_elems) window_elems[k] = nw;
     }
+    return SGTV_OK;
+}
+
+int sgtv_stack_info(sgtv_t h, int32_t *words, int32_t *tile_rows, int64_t *tiles, int64_t *levels, int64_t *partials)
+{
+    if (!h) return SGTV_ERR_ARG;
+    const StackMat &m = h->d.st;
+    if (words) *words = m.built ? m.words : 0;
+    if (tile_rows) *tile_rows = m.built ? m.tr : 0;
+    if (tiles) *tiles = m.built ? m.ntiles : 0;
+    if (levels) *levels = m.built ? h->stk_levels : 0;
+    if (partials) *partials = m.built ? h->stk_partials : 0;
     return SGTV_OK;
 }
 

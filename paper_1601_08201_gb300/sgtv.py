@@ -110,6 +110,7 @@ def load():
             "sgtv_variant_count": (ctypes.c_int, [_P, _I32]),
             "sgtv_variant_name": (ctypes.c_char_p, [_P, _I32, _I32]),
             "sgtv_tli_info": (ctypes.c_int, [_P, _P, _P, _P, _P]),
+            "sgtv_stack_info": (ctypes.c_int, [_P, _P, _P, _P, _P, _P]),
             "sgtv_kkt_residual_noalloc": (ctypes.c_int, [_I64, _I64, _P, _P, _P, _P, _P, _P, _I32, _I32, _I32,
                                                          _I32, _P, _P, _P, _I64, _P, _P, _P, _D, _P, _P]),
             "sgtv_noalloc_last_error": (ctypes.c_char_p, []),
@@ -134,7 +135,7 @@ def exported_symbols():
             "sgtv_kkt_residual_noalloc", "sgtv_noalloc_last_error", "sgtv_setup_batch", "sgtv_batch_info",
             "sgtv_objective_scan", "sgtv_set_data", "sgtv_normalized_backprojection", "sgtv_warm_start",
             "sgtv_get_variant", "sgtv_set_variant", "sgtv_warm_start_dual", "sgtv_set_wait_limit",
-            "sgtv_set_serial"]
+            "sgtv_set_serial", "sgtv_stack_info"]
 
 
 def _ptr(a):
@@ -392,6 +393,14 @@ def tli_info(h):
             for k, name in enumerate(("csr", "csc"))}
 
 
+def stack_info(h):
+    w, r = _I32(), _I32()
+    t, lv, pa = _I64(), _I64(), _I64()
+    _check(load().sgtv_stack_info(h, ctypes.byref(w), ctypes.byref(r), ctypes.byref(t), ctypes.byref(lv),
+                                  ctypes.byref(pa)), h)
+    return dict(words=w.value, tile_rows=r.value, tiles=t.value, levels=lv.value, partials=pa.value)
+
+
 def kkt_residual_noalloc(I, J, csr_rowptr, csr_col, csr_val, csc_colptr, csc_row, csc_val, Nx, Nz, Nq,
                          n_dirs, w, y, b, s, f, c, rho, out, stream=0):
     """sgtv_kkt_residual_noalloc: array arguments are device addresses (ints,
@@ -512,6 +521,9 @@ class Handle:
 
     def tli_info(self):
         return tli_info(self.h)
+
+    def stack_info(self):
+        return stack_info(self.h)
 
     def set_wait_limit(self, ns):
         set_wait_limit(self.h, ns)
