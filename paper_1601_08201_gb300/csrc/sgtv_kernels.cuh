@@ -373,76 +373,35 @@ __device__ __forceinline__ int64_t step_of(const Geom &g, const Loc &L, int p)
     return (int64_t(g.dx[p]) * L.Nz + g.dz[p]) * L.Nq;
 }
 
-// PRE = false: each direction's neighbour loads sit behind its inside test
-// (inside the fused backprojection this is the faster form); PRE = true: every
-// load first, a neighbour outside the scan reading the voxel itself (unused),
-// so a stand-alone elementwise pass has them all in flight together. Both
-// forms do the same arithmetic in the same order.
-template <typename T, bool PRE = false>
+// Each direction's neighbour loads sit behind its inside test (inside the fused
+// backprojection faster than all loads first).
+template <typename T>
 __device__ __forceinline__ T voxel_update_at(const Geom &g, const Loc &L, int64_t j, T e, const T *__restrict__ s,
                                              const T *__restrict__ f, const T *__restrict__ d,
                                              const T *__restrict__ c)
 {
     const T fj = f[j];
     T alpha = T(0), gamma = T(0);
-    if (!PRE) {
 #pragma unroll
-        for (int p = 0; p < 4; p++) {
-            if (p >= g.n_dirs) break;
-            const int dx = g.dx[p], dz = g.dz[p];
-            const T w = wgt<T>(g, p);
-            const T w2 = w * w;
-            const int64_t step = step_of(g, L, p);
-            const int64_t pj = int64_t(p) * g.J + j;
-            const T u_jp = d[pj] - c[pj];
-            if (inside(L, L.x + dx, L.z + dz)) {
-                alpha += w2;
-                gamma += w * (w * (fj + f[j + step]) + u_jp);
-            } else {
-                alpha += T(0.5) * w2;
-                gamma += w * u_jp;
-            }
-            if (inside(L, L.x - dx, L.z - dz)) {
-                const T u_ap = d[pj - step] - c[pj - step];
-                alpha += w2;
-                gamma += w * (w * (f[j - step] + fj) - u_ap);
-            }
+    for (int p = 0; p < 4; p++) {
+        if (p >= g.n_dirs) break;
+        const int dx = g.dx[p], dz = g.dz[p];
+        const T w = wgt<T>(g, p);
+        const T w2 = w * w;
+        const int64_t step = step_of(g, L, p);
+        const int64_t pj = int64_t(p) * g.J + j;
+        const T u_jp = d[pj] - c[pj];
+        if (inside(L, L.x + dx, L.z + dz)) {
+            alpha += w2;
+            gamma += w * (w * (fj + f[j + step]) + u_jp);
+        } else {
+            alpha += T(0.5) * w2;
+            gamma += w * u_jp;
         }
-    } else {
-        T fF[4], fB[4], uF[4], uB[4];
-        bool inF[4], inB[4];
-#pragma unroll
-        for (int p = 0; p < 4; p++) {
-            fF[p] = fB[p] = uF[p] = uB[p] = T(0);
-            inF[p] = inB[p] = false;
-            if (p < g.n_dirs) {
-                const int64_t step = step_of(g, L, p);
-                const int64_t pj = int64_t(p) * g.J + j;
-                inF[p] = inside(L, L.x + g.dx[p], L.z + g.dz[p]);
-                inB[p] = inside(L, L.x - g.dx[p], L.z - g.dz[p]);
-                const int64_t sf = inF[p] ? step : 0, sb = inB[p] ? step : 0;
-                fF[p] = f[j + sf];
-                fB[p] = f[j - sb];
-                uF[p] = d[pj] - c[pj];
-                uB[p] = d[pj - sb] - c[pj - sb];
-            }
-        }
-#pragma unroll
-        for (int p = 0; p < 4; p++) {
-            if (p >= g.n_dirs) break;
-            const T w = wgt<T>(g, p);
-            const T w2 = w * w;
-            if (inF[p]) {
-                alpha += w2;
-                gamma += w * (w * (fj + fF[p]) + uF[p]);
-            } else {
-                alpha += T(0.5) * w2;
-                gamma += w * uF[p];
-            }
-            if (inB[p]) {
-                alpha += w2;
-                gamma += w * (w * (fB[p] + fj) - uB[p]);
-            }
+        if (inside(L, L.x - dx, L.z - dz)) {
+            const T u_ap = d[pj - step] - c[pj - step];
+            alpha += w2;
+            gamma += w * (w * (f[j - step] + fj) - u_ap);
         }
     }
     const T rho = lrho<T>(L);
@@ -452,12 +411,12 @@ __device__ __forceinline__ T voxel_update_at(const Geom &g, const Loc &L, int64_
     return sgtv_root<T>(alpha, sj - gamma, fj * e, sj);
 }
 
-template <typename T, bool PRE = false>
+template <typename T>
 __device__ __forceinline__ T voxel_update(const Geom &g, int64_t j, T e, const T *__restrict__ s,
                                           const T *__restrict__ f, const T *__restrict__ d,
                                           const T *__restrict__ c)
 {
-    return voxel_update_at<T, PRE>(g, locate_voxel(g, j), j, e, s, f, d, c);
+    return voxel_update_at<T>(g, locate_voxel(g, j), j, e, s, f, d, c);
 }
 
 // a2 + a4: backprojection fused with the f-update. One warp owns CPW
@@ -621,14 +580,6 @@ k_colsum(int64_t J, const int64_t *__restrict__ colptr, const V *__restrict__ va
 
 // ---------------------------------------------------------------------------------------
 // a5 + a6: group shrink (Eq. 6) and dual update (Eq. 7), one warp per spatial bin.
-
-template <typename T>
-__device__ __forceinline__ double wgrad_at_f64(const Geom &g, const Loc &L, const T *__restrict__ f, int64_t j,
-                                               int p)
-{
-    const bool in = inside(L, L.x + g.dx[p], L.z + g.dz[p]);
-    return g.w[p] * (double(f[j]) - (in ? double(f[j + step_of(g, L, p)]) : 0.0));
-}
 
 template <typename T>
 __device__ __forceinline__ T wgrad_at(const Geom &g, const Loc &L, const T *__restrict__ f, int64_t j, int p)
