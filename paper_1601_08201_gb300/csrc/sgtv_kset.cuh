@@ -74,12 +74,13 @@ struct Group8 {
     }
 };
 
-// Launch a TLI kernel with `smem` bytes of dynamic shared memory, raising the
-// kernel's opt-in limit the first time a launch needs more than 48 KB.
+// Raise a kernel's opt-in limit where a launch needs it: the 48 KB that a block has
+// without asking hold its static shared memory too (barriers and tile descriptors,
+// below 1 KB in all of these kernels).
 template <typename K>
 inline void ensure_smem(K kernel, int smem, int &granted)
 {
-    if (smem > 48 * 1024 && smem > granted) {
+    if (smem > 47 * 1024 && smem > granted) {
         if (cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, smem) == cudaSuccess)
             granted = smem;
     }
@@ -96,7 +97,7 @@ struct FwdTli {
     static_assert(8 * SPW == kTliTile, "tile = 8 warps x SPW rows");
     static void launch(const Dev &d, const void *f, void *ratio, cudaStream_t st)
     {
-        static int granted = 48 * 1024;
+        static int granted = 0;
         auto kern = k_forward_tli<T, V, SPW, U, PIPE, UV, MINB, L2PF>;
         const int smem = d.tr.max_stage * int(sizeof(T));
         ensure_smem(kern, smem, granted);
@@ -112,7 +113,7 @@ struct BackTli {
     static_assert(8 * SPW == kTliTile, "tile = 8 warps x SPW columns");
     static void launch(const Dev &d, const Geom &g, const void *f, void *f_new, cudaStream_t st)
     {
-        static int granted = 48 * 1024;
+        static int granted = 0;
         auto kern = k_back_update_tli<T, V, SPW, U, PIPE, UV, MINB, L2PF>;
         if (MINB > 1) {  // several large staged windows per SM: all on-chip memory as shared memory
             static const bool carved =
@@ -136,7 +137,7 @@ struct Scatter {
     static constexpr int kBufs = PRIV ? 9 : 2;
     static void launch(const Dev &d, const void *f, void *e, cudaStream_t st)
     {
-        static int granted = 48 * 1024;
+        static int granted = 0;
         auto kern = k_project_scatter_tli<T, V, SPW, U, PRIV, KEEP, MINB>;
         // all of the SM's on-chip memory as shared memory: the gathers and the
         // scatter hit shared memory and the stream bypasses L1, so the
@@ -160,7 +161,7 @@ struct ScatterV4 {
     static_assert(8 * SPW == kTliTile, "tile = 8 warps x SPW rows");
     static void launch(const Dev &d, const void *f, void *e, cudaStream_t st)
     {
-        static int granted = 48 * 1024;
+        static int granted = 0;
         auto kern = k_project_scatter_tli_v4<T, V, SPW, UV, PRIV, MINB, L2PF>;
         static const bool carved =
             cudaFuncSetAttribute(kern, cudaFuncAttributePreferredSharedMemoryCarveout, 100) == cudaSuccess;
@@ -183,7 +184,7 @@ struct ScatterSp {
     static constexpr int kBufs = PRIV ? 9 : 2;
     static void launch(const Dev &d, const void *f, void *e, cudaStream_t st)
     {
-        static int granted = 48 * 1024;
+        static int granted = 0;
         auto kern = k_scatter_sp<T, V, UV, MINB, L2PF, PRIV, PF, OPT>;
         static const bool carved =
             cudaFuncSetAttribute(kern, cudaFuncAttributePreferredSharedMemoryCarveout, 100) == cudaSuccess;
@@ -208,7 +209,7 @@ struct ScatterSp {
 template <typename V, bool PART, int W>
 inline void rows_stack_w(const Dev &d, const void *f, void *out, void *ratio, cudaStream_t st)
 {
-    static int granted = 48 * 1024;
+    static int granted = 0;
     auto kern = k_rows_stack<V, W, PART>;
     static const bool carved =
         cudaFuncSetAttribute(kern, cudaFuncAttributePreferredSharedMemoryCarveout, 100) == cudaSuccess;
@@ -277,7 +278,7 @@ template <typename T, typename V, int NS, int NW>
 struct FwdTma {
     static void launch(const Dev &d, const void *f, void *ratio, cudaStream_t st)
     {
-        static int granted = 48 * 1024, cs = -1, nb = 1;
+        static int granted = 0, cs = -1, nb = 1;
         auto kern = k_forward_tma<T, V, NS, NW>;
         const int smem = NS * d.tr.tma_stage_bytes;
         const int grid = tma_grid(kern, 32 * (NW + 1), smem, d.sm_count, d.tr.ntiles, granted, cs, nb);
@@ -292,7 +293,7 @@ template <typename T, typename V, int NS, int NW>
 struct BackTma {
     static void launch(const Dev &d, const Geom &g, const void *f, void *f_new, cudaStream_t st)
     {
-        static int granted = 48 * 1024, cs = -1, nb = 1;
+        static int granted = 0, cs = -1, nb = 1;
         auto kern = k_back_update_tma<T, V, NS, NW>;
         const int smem = NS * d.tc.tma_stage_bytes;
         const int grid = tma_grid(kern, 32 * (NW + 1), smem, d.sm_count, d.tc.ntiles, granted, cs, nb);
@@ -311,7 +312,7 @@ struct Pers {
     static cudaError_t launch(const Dev &d, const Geom &g, const void *f, void *f_new, int do_shrink, GridBar *bar,
                               cudaStream_t st)
     {
-        static int granted = 48 * 1024, cached_smem = -1, nb = 1;
+        static int granted = 0, cached_smem = -1, nb = 1;
         auto kern = k_iteration<T, V, UVF, UVB, MINB>;
         const int smem = int(sizeof(T)) * (d.tr.max_stage > d.tc.max_stage ? d.tr.max_stage : d.tc.max_stage);
         ensure_smem(kern, smem, granted);
