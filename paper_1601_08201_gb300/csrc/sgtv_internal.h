@@ -168,8 +168,11 @@ struct KernelSet {
     int n_fwd;
     ForwardFn fwd[kMaxVariants];
     const char *fwd_name[kMaxVariants];
-    // *_untimed = 1: kept for callers that pin it, but not a candidate of the autotuner (another form of
-    // the list was faster on every problem measured)
+    // *_untimed = 1: kept for callers that pin it, but not a candidate of the autotuner: on none of 31 problems (8 to
+    // 262,144 rows of 2 to 10,000 nonzeros, list and window tiles; 87 forward, 93 backprojection and 49 scatter
+    // timings over the three precisions) more than 1 % faster than the best of the others. Timed where they were: the
+    // forward "tli_v4x2_min8" in FP32 and BF16 (up to 10 %, 64^3 with 128 a row), the scatters "tli_u8_private_keep" and
+    // "tli_v4x3_private_min4" in FP64 (up to 4 %, 2^26 nonzeros).
     int fwd_untimed[kMaxVariants], back_untimed[kMaxVariants], scatter_untimed[kMaxVariants];
     int fwd_need[kMaxVariants];     // 0 plain; 1 tiled (Dev::tr); 2 stacked (Dev::st with partial sums;
                                     // both products or neither); NS >= 3: TMA pipeline of NS stages

@@ -545,7 +545,7 @@ struct Impl {
         k.fwd[n] = FwdTli<T, V, kTliTile / 8, 8, false, 2>::launch; k.fwd_name[n] = "tli_v4x2"; k.fwd_need[n++] = 1;
         k.fwd[n] = FwdTli<T, V, kTliTile / 8, 8, false, 3>::launch; k.fwd_name[n] = "tli_v4x3"; k.fwd_need[n++] = 1;
         k.fwd[n] = FwdTli<T, V, kTliTile / 8, 8, false, 2, 8>::launch; k.fwd_name[n] = "tli_v4x2_min8";
-        k.fwd_untimed[n] = 1; k.fwd_need[n++] = 1;
+        k.fwd_untimed[n] = sizeof(T) == 8; k.fwd_need[n++] = 1;
         k.fwd[n] = FwdTli<T, V, kTliTile / 8, 8, false, 3, 6>::launch; k.fwd_name[n] = "tli_v4x3_min6";
         k.fwd_untimed[n] = 1; k.fwd_need[n++] = 1;
         // the same forms with the block's tile stream bulk-prefetched into L2 at its start
@@ -603,9 +603,9 @@ struct Impl {
         k.scatter[n] = Scatter<T, V, kTliTile / 8, 8, false, true, 4>::launch;
         k.scatter_name[n] = "tli_u8_atomic_keep"; k.scatter_bufs[n++] = 2;
         k.scatter[n] = Scatter<T, V, kTliTile / 8, 8, true, true, 4>::launch;
-        k.scatter_name[n] = "tli_u8_private_keep"; k.scatter_untimed[n] = 1; k.scatter_bufs[n++] = 9;
+        k.scatter_name[n] = "tli_u8_private_keep"; k.scatter_untimed[n] = sizeof(T) == 4; k.scatter_bufs[n++] = 9;
         k.scatter[n] = ScatterV4<T, V, kTliTile / 8, 3, true, 4>::launch;
-        k.scatter_name[n] = "tli_v4x3_private_min4"; k.scatter_untimed[n] = 1; k.scatter_bufs[n++] = 9;
+        k.scatter_name[n] = "tli_v4x3_private_min4"; k.scatter_untimed[n] = sizeof(T) == 4; k.scatter_bufs[n++] = 9;
         k.scatter[n] = ScatterV4<T, V, kTliTile / 8, 2, true, 5>::launch;
         k.scatter_name[n] = "tli_v4x2_private_min5"; k.scatter_untimed[n] = 1; k.scatter_bufs[n++] = 9;
         k.scatter[n] = ScatterV4<T, V, kTliTile / 8, 2, true, 5, true>::launch;
