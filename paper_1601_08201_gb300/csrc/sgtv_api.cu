@@ -586,11 +586,16 @@ int build_sp(sgtv_t h)
 
 // Build the stacked row form (sgtv_stack.cu) where it applies: FP32 vectors,
 // tiles of at most 32 * kStkMaxWords columns, a schedule that fits the ring,
-// and a size no larger than the tiled form's by more than a quarter (thin
-// tiles, whose columns most rows miss, pay a bit per column and row) unless it
-// stays in the L2 cache anyway (64 MB). Where
-// it does not apply, or its memory is refused, the handle runs without it:
-// d.st.built stays 0. `parts`: with the two-pass form's partial sums.
+// and a size no larger than the tiled form's by more than a quarter, unless it
+// stays in the L2 cache anyway (64 MB): thin tiles, whose columns most rows miss,
+// pay a bit per column and row. That bounds memory and set-up; which form is
+// faster the timing says, and the ratio of the sizes does not (an iteration in one
+// pass, microseconds, the stacked form against the best of the others; 2^20 rows of
+// 8 nonzeros in windows of 128 columns, 2.3 times the size: 132 and 230, of 32 in
+// 512, 1.5 times: 227 and 247, of 64 in 2048, 1.75 times: 395 and 329; 65,536 rows of 8
+// in 512, 2.9 times but 9 MB: 15.6 and 21.0). Where it does not apply, or its memory
+// is refused, the handle runs without it: d.st.built stays 0. `parts`: with the
+// two-pass form's partial sums.
 int build_stack(sgtv_t h, bool parts)
 {
     Dev &d = h->d;
@@ -750,7 +755,9 @@ int build_stack(sgtv_t h, bool parts)
             if (hc[j] > widest) widest = hc[j];
         }
         h->stk_partials = off[J];
-        // a column in very many tiles would make its one thread sort and add for long
+        // One thread sorts a column's places by insertion (k_stk_order) and one adds its sums up: a column in very
+        // many tiles would keep set-up waiting. Not a line of speed either: 500 columns in windows that are the
+        // image, 1911 tiles a column, two passes 128 us against 363, but 967 tiles 62 against 45.
         if (widest > 1024) return without();
         m.part = next(pk, keep[7]);  // off[J] <= places
         int32_t *ent = static_cast<int32_t *>(next(pw, work[5]));
