@@ -411,7 +411,7 @@ def kernel_source_hash():
     import re
     h = hashlib.sha256()
     csrc = os.path.join(ROOT, "paper_1601_08201_gb300", "csrc")
-    files = ["sgtv_kernels.cuh", "sgtv_kset.cuh", "sgtv_internal.h", "kset_f32.cu", "kset_bf16.cu", "kset_f64.cu"]
+    files = ["sgtv_kernels.cuh", "sgtv_kset.cuh", "sgtv_internal.h", "sgtv_rules.h", "kset_f32.cu", "kset_bf16.cu", "kset_f64.cu"]
     for f in files:
         text = open(os.path.join(csrc, f), encoding="utf-8").read()
         text = re.sub(r"/\*.*?\*/", "", text, flags=re.S)
