@@ -428,7 +428,8 @@ def recorded_traffic(kernel, workload, precision, variant=None):
         rec = json.load(open(path))
     except Exception:
         return None
-    ent = rec.get(f"{kernel}|{workload}|{precision}")
+    key = f"{kernel}|{workload}|{precision}"
+    ent = rec.get(f"{key}|{variant}") or rec.get(key)
     if not ent or ent.get("source_sha") != kernel_source_hash():
         return None
     if variant is not None and ent.get("variant") not in (None, variant):
