@@ -183,9 +183,11 @@ int sgtv_objective_scan(sgtv_t h, int32_t k, double *phi, double *dev, double *t
 /* Enqueue n >= 0 ADMM iterations (Eqs. 5-7) on the handle's stream. Each
  * iteration launches three kernels: forward projection with the ratio y/ybar,
  * backprojection fused with the closed-form f-update, and the group shrink
- * fused with the dual update -- with SGTV_FLAG_SINGLE_PASS the first two are
- * one pass over the rows that scatters into e, then the f-update -- or, with
- * SGTV_FLAG_PERSISTENT, one cooperative
+ * fused with the dual update. With the stacked pair of variants (see
+ * sgtv_autotune) the first two are one pass over the rows, which forms both
+ * products, and the f-update, which adds up the pass's partial sums of e; with
+ * SGTV_FLAG_SINGLE_PASS one pass over the rows that adds into e, then the
+ * f-update; with SGTV_FLAG_PERSISTENT all three are one cooperative
  * kernel doing the three phases between grid-wide barriers (each wait is
  * bounded: a barrier that does not complete within about 1 s records
  * SGTV_ERR_TIMEOUT, reported by the next sgtv_sync). With SGTV_FLAG_GRAPH,
@@ -234,8 +236,8 @@ int sgtv_set_state_f64(sgtv_t h, const double *f, const double *d, const double 
 /* SpMV autotuner. The forward projection and the fused backprojection come
  * in several tilings (segments per warp, prefetch depth, pipelining, register
  * cap). Variants of one element order give bit-identical results; the
- * 4-wide forms ("v4" in the name) split a segment among lanes differently and
- * round differently (equally deterministic), so with the autotuner on, the
+ * 4-wide forms ("v4" in the name) and FP64's "lanes8" split a segment among
+ * lanes differently and round differently (equally deterministic), so with the autotuner on, the
  * chosen pair decides the last bits; pin the variants (SGTV_FLAG_NO_AUTOTUNE +
  * sgtv_set_variants) for bit-reproducible runs. The stacked pair ("stack_v4"
  * in both products: A read once, by rows, e from partial sums added in a fixed
@@ -249,12 +251,15 @@ int sgtv_set_state_f64(sgtv_t h, const double *f, const double *d, const double 
  * With SGTV_FLAG_SINGLE_PASS it also times the single-pass scatter's forms
  * (one accumulator per block with shared-memory atomic adds, or one per warp
  * summed in a fixed order; prefetch depth; register cap; "stack": sums in
- * registers) that fit in shared memory. kernel is SGTV_K_FORWARD, SGTV_K_BACK_UPDATE or SGTV_K_SCATTER (the
+ * registers) that fit in shared memory. A form of A that only some variants read
+ * (the row stream of the "sp_" scatters, the stacked form) is built for the
+ * timing, or when such a variant is set, and given back where the timing chose
+ * another. kernel is SGTV_K_FORWARD, SGTV_K_BACK_UPDATE or SGTV_K_SCATTER (the
  * latter in sgtv_variant_count / _name and sgtv_get_variant / sgtv_set_variant
  * only). Where sgtv_set_variant takes one product into or out of the stacked
  * pair, the other goes with it: into the pair, or back to the form it was last
  * set to or timed best in. The set functions return SGTV_ERR_ARG (not sticky) for an index out
- * of range or a form that does not fit; sgtv_variant_name returns "" for one. */
+ * of range or a form that does not fit (or has no memory); sgtv_variant_name returns "" for one. */
 int sgtv_autotune(sgtv_t h, int32_t reps);
 int sgtv_get_variants(sgtv_t h, int32_t *fwd, int32_t *back);
 int sgtv_set_variants(sgtv_t h, int32_t fwd, int32_t back);

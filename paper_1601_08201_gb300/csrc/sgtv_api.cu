@@ -646,7 +646,7 @@ int build_stack(sgtv_t h, bool parts)
     };
     // Rows per tile. A tile costs its rows and about 9 rows' worth of reading
     // its columns' f and adding its sums; the last wave of warps is half
-    // empty. Measured, microseconds for 64 / 32 / 16 rows: 2^28 nonzeros 252 /
+    // empty. Measured in one pass, microseconds for 64 / 32 / 16 rows: 2^28 nonzeros 252 /
     // 273 / 369, 2^26 84 / 79 / 105, 2^25 47 / 49 / 57; a 41 x 9 x 54 scan,
     // whose tiles fill no wave, takes 8 (whole iterations: 16.4 for 32, 12.0
     // for 16, 10.4 for 8, 10.8 for 4).

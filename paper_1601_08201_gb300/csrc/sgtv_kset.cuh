@@ -201,9 +201,9 @@ struct ScatterSp {
 
 // Row pass over the stacked form, by the number of words. One warp per tile,
 // with the ring's levels in shared memory. Measured against the forms it was
-// chosen over (microseconds): 2^28 nonzeros, 256 a row, FP32 / BF16 values 249 /
-// 252 against 391 / 366 for the row-stream scatter; both products of a two-pass
-// iteration 278 and 26 for the f-update, against 607; 41 x 9 x 54 scan, whose
+// chosen over (microseconds): 2^28 nonzeros, 256 a row, FP32 / BF16 values 254 /
+// 251 against 391 / 366 for the row-stream scatter; both products of a two-pass
+// iteration 263 and 25 for the f-update, against 607; 41 x 9 x 54 scan, whose
 // row-stream tiles stage 80 KB windows, 6.1 against 19.0.
 
 template <typename V, bool PART, int W>
