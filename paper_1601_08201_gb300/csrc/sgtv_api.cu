@@ -1736,7 +1736,8 @@ int sgtv_set_variants(sgtv_t h, int32_t fwd, int32_t back)
     if (rc) return rc;
     if (fwd < 0 || fwd >= h->ks->n_fwd || back < 0 || back >= h->ks->n_back)
         return SGTV_ERR_ARG;  // not sticky: the handle keeps its variants
-    if (h->ks->fwd_need[fwd] == 2 && h->ks->back_need[back] == 2 && (rc = need_forms(h, false, true)) != SGTV_OK)
+    if (h->ks->fwd_need[fwd] == 2 && h->ks->back_need[back] == 2 && !h->single_pass &&
+        (rc = need_forms(h, false, true)) != SGTV_OK)
         return rc;
     if (!variant_ok(h->d, h->d.tr, h->ks->fwd_need[fwd]) || !variant_ok(h->d, h->d.tc, h->ks->back_need[back]))
         return SGTV_ERR_ARG;  // that tiled form was not built for this matrix

@@ -73,6 +73,22 @@ def test_two_passes_hold_the_form_in_use():
         assert np.linalg.norm(h.get_state_f64()[0] - ref[0]) <= 1e-5 * np.linalg.norm(ref[0])
 
 
+def test_a_refused_pin_builds_nothing():
+    P = synth.preset("wide_64x16x32")
+    with sgtv.Handle(P, flags=SP | TUNE) as h:  # its products serve the KKT measure only
+        bare = held(h)
+        with pytest.raises(sgtv.SgtvError):
+            pair(h)
+        assert held(h) == bare
+    with sgtv.Handle(P, flags=TUNE) as h:
+        bare = held(h)
+        with pytest.raises(sgtv.SgtvError):
+            scatter(h, "stack")
+        with pytest.raises(sgtv.SgtvError):
+            h.set_variants(h.variant_names()["k_forward"].index("stack_v4"), 0)
+        assert held(h) == bare
+
+
 @pytest.mark.parametrize("flags", [0, sgtv.FLAG_GRAPH])
 def test_a_form_given_back_and_pinned_again_gives_the_same(flags):
     P = synth.preset("ragged_13x7x37")
