@@ -629,7 +629,7 @@ int build_stack(sgtv_t h, bool parts)
         m = StackMat{};
         return cuda_fail(h, e, "stacked row form");
     };
-    int *cnt = reinterpret_cast<int *>(d.red);  // scratch until the first reduction
+    int *cnt = reinterpret_cast<int *>(d.red);  // scratch: every reduction writes it before it is read
     int most = 0;
     auto count = [&](int rows) {
         cudaError_t e = cudaMemsetAsync(cnt, 0, sizeof(int) * 4, st);
